@@ -22,6 +22,7 @@ __global__ void chi_table_kernel(int, int, const double*, const double*, Lattice
                                  float*, double*, float*);
 __global__ void dof_consts_kernel(Dims, Layout, const double*, int, double*, double*, float*);
 __global__ void t1_table_kernel(int, const double*, const double*, float2*, int);
+__global__ void h1_table_kernel(const double*, double*, int);
 __global__ void widen_kernel(const float*, long long, Dims, double*);
 __global__ void widen_pairs_kernel(const float*, long long, int, double*, double*, double*, double*);
 __global__ void narrow_kernel(const double*, Dims, float*);
@@ -77,6 +78,7 @@ struct cfust_ctx {
     int *flags = nullptr, *comp_status = nullptr;
     float* stage32 = nullptr;
     float2* t1tab = nullptr;  // FP32 T_2: per-dof tables of T_1 at dof + 1
+    double* h1tab = nullptr;  // FP64 T_2 (and the T_1 beside it): per-dof tables of H (H1_*)
     // mixed precision: FP32 copies of the observations and factor blocks
     bool mixed = false;
     bool tc_stats = false;  // mixed form: cross statistics on the tensor cores (reduce_tc.cu)
@@ -375,7 +377,7 @@ static void free_all(cfust_ctx* c)
                     c->logf, c->u, c->elogu, c->eu,
                     c->euu, c->se, c->tau, c->partial, c->stats, c->flags, c->comp_status,
                     c->stage32, c->pd, c->pc, c->fix_count, c->fix_list, c->y32, c->F32, c->pr32, c->pd32, c->pc32, c->res32_l0, c->t1tab,
-                    c->work_dev, c->seg, c->lchi64, c->lchi32};
+                    c->work_dev, c->seg, c->lchi64, c->lchi32, c->h1tab};
     for (void* b : bufs)
         if (b) cudaFree(b);
     for (RecSet& r : c->rec) {
@@ -542,6 +544,10 @@ extern "C" cfust_status cfust_create(cfust_ctx** out, int p, int q, int g, int64
     if (o.precision != CFUST_PREC_FP64 && (q == 2 || (!c->single_pass && (q == 3 || q == 4)))) {
         ALLOC(t1tab, (size_t)3 * g * T1TAB_N);
     }
+    if (o.precision == CFUST_PREC_FP64 && o.model == CFUST_MODEL_CFUST &&
+        (q == 2 || (!c->single_pass && (q == 3 || q == 4)))) {
+        ALLOC(h1tab, (size_t)4 * g * H1_SIZE);
+    }
     {
         const bool sp = c->single_pass;
         const int kdim[4] = {q, q - 1, q - 2, q};
@@ -648,7 +654,7 @@ extern "C" cfust_status cfust_create(cfust_ctx** out, int p, int q, int g, int64
                     delete c;
                     return fail(nullptr, CFUST_ECUDA, "cfust_create: cudaEventCreate failed");
                 }
-    if (c->t1tab && (cudaStreamCreateWithFlags(&c->st2, cudaStreamNonBlocking) != cudaSuccess ||
+    if ((c->t1tab || c->h1tab) && (cudaStreamCreateWithFlags(&c->st2, cudaStreamNonBlocking) != cudaSuccess ||
                      cudaEventCreateWithFlags(&c->ev_fork, cudaEventDisableTiming) != cudaSuccess ||
                      cudaEventCreateWithFlags(&c->ev_join, cudaEventDisableTiming) != cudaSuccess)) {
         free_all(c);
@@ -750,7 +756,7 @@ extern "C" cfust_status cfust_get_params(cfust_ctx* c, cfust_params* P)
 }
 
 // S0 + S1: per-component factors and (q >= 3) the chi tables.
-static cfust_status launch_setup(cfust_ctx* c)
+static cfust_status launch_setup(cfust_ctx* c, int density_only)
 {
     prof_begin(c, CFUST_PROF_SETUP);
     setup_components_kernel<<<c->g, 32, 0, c->st>>>(c->D, c->Ly, c->mu, c->Sigma, c->Delta, c->nu,
@@ -776,11 +782,31 @@ static cfust_status launch_setup(cfust_ctx* c)
         CU(cudaEventRecord(c->ev_join, c->st2));
         c->t1_pending = true;
     }
+    if (c->h1tab) {
+        // tables 4h + e hold H at dof nu_h + p + e: a T_2 record of index 3h + j reads e = j and
+        // j + 1, a T_1 record e = j (level 0: j = 0, and 2 unless density_only; level 1: 1; level 2: 0)
+        int emask = 0;
+        for (int l = 0; l < (density_only ? 1 : 3); ++l) {
+            const RecSet& r = c->rec[l];
+            if (r.nrec == 0) continue;
+            const int j0 = l == 1 ? 1 : 0;
+            if (r.k == 2) emask |= 3 << j0 | (l == 0 && !density_only ? 3 << 2 : 0);
+            if (r.k == 1) emask |= 1 << j0;
+        }
+        if (emask) {
+            CU(cudaEventRecord(c->ev_fork, c->st));
+            CU(cudaStreamWaitEvent(c->st2, c->ev_fork, 0));
+            h1_table_kernel<<<dim3(H1_CELLS / 16, 4 * c->g), 16 * H1_NC, 0, c->st2>>>(c->dofs, c->h1tab, emask);
+            LAUNCHED();
+            CU(cudaEventRecord(c->ev_join, c->st2));
+            c->t1_pending = true;
+        }
+    }
     if (c->mixed) {
         cudaError_t e = launch_factors_f32(c->F, c->F32, (long long)c->g * c->Ly.stride, c->st, &c->launches);
         if (e != cudaSuccess) return fail(c, CFUST_ECUDA, std::string("factor copy: ") + cudaGetErrorString(e));
     }
-    prof_end(c, CFUST_PROF_SETUP, 2 + (c->mixed ? 1 : 0) + (c->t1tab ? 1 : 0));
+    prof_end(c, CFUST_PROF_SETUP, 2 + (c->mixed ? 1 : 0) + (c->t1tab || c->h1tab ? 1 : 0));
     if (c->q >= 3) {
         prof_begin(c, CFUST_PROF_CHI);
         // the single-pass E-step reads only the dof nu+p tables (index 3h)
@@ -809,6 +835,7 @@ static IntegArgs integ_args(const cfust_ctx* c)
     ia.glx32h = c->glx32h; ia.glw32h = c->glw32h;
     ia.t2n_lo = c->t2n_lo; ia.glx32l = c->glx32l; ia.glw32l = c->glw32l;
     ia.t1tab = c->t1tab;
+    ia.h1tab = c->h1tab;
     ia.wtab = c->wtab;
     ia.nodes = nullptr;
     int t2g = 0, mp = 0;
@@ -966,7 +993,7 @@ static cfust_status enqueue_estep_segments(cfust_ctx* c, double* seg, long long 
 {
     CU(cudaMemsetAsync(c->flags, 0, sizeof(int), c->st));
     cfust_status s;
-    if ((s = launch_setup(c)) != CFUST_OK) return s;
+    if ((s = launch_setup(c, 0)) != CFUST_OK) return s;
     if ((s = launch_pairs(c, 0)) != CFUST_OK) return s;
     ReduceArgs r;
     r.D = c->D; r.y = c->y; r.pi = c->pi; r.mu = c->mu; r.logf = c->logf; r.u = c->u;
@@ -1132,7 +1159,7 @@ static cfust_status enqueue_loglik(cfust_ctx* c)
 {
     CU(cudaMemsetAsync(c->flags, 0, sizeof(int), c->st));
     cfust_status s;
-    if ((s = launch_setup(c)) != CFUST_OK) return s;
+    if ((s = launch_setup(c, 1)) != CFUST_OK) return s;
     if ((s = launch_pairs(c, 1)) != CFUST_OK) return s;
     prof_begin(c, CFUST_PROF_REDUCE);
     loglik_partial_kernel<<<c->nblocks_ll, 256, 0, c->st>>>(c->D, c->pi, c->logf, c->partial);
@@ -1956,6 +1983,7 @@ extern "C" cfust_status cfust_tk_eval(cfust_ctx* c, int k, int count, const doub
         }
         IntegArgs ia = integ_args(c);
         ia.t1tab = use_t1tab ? t1t : nullptr;
+        ia.h1tab = nullptr;  // the tables are per component, not per case
         ia.cst64 = k64;
         ia.cst32 = k32;
         ia.F = dF;

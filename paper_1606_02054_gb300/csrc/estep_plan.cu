@@ -325,7 +325,8 @@ __global__ void __launch_bounds__(128) combine_kernel(CombineArgs a)
 
 // FP32 with the T_1 tables (a.t1tab) and a record of table index 3h + 1 (dof nu + p + 1,
 // the q = 2 moments' level 1): T_1 by interpolation in the table 3h, which holds T_1 at
-// that dof (see t1cdf_table), instead of the continued fraction.
+// that dof (see t1cdf_table), instead of the continued fraction.  FP64 with the tables of H
+// (a.h1tab): T_1 at dof nu_h + p + e, table index 3h + e, from the table 4h + e.
 template <typename R>
 __global__ void __launch_bounds__(128) t1_records_kernel(RecSet r, IntegArgs a)
 {
@@ -334,9 +335,13 @@ __global__ void __launch_bounds__(128) t1_records_kernel(RecSet r, IntegArgs a)
          i += (long long)gridDim.x * blockDim.x) {
         const R dof = (R)r.dof[i];  // infinite: the normal limit, Phi
         const int tab = r.tab[i];
-        if (sizeof(R) == sizeof(float) && a.t1tab && tab % 3 == 1 && !isinf(dof))
+        if (sizeof(R) == sizeof(float) && a.t1tab && tab % 3 == 1 && !isinf(dof)) {
             r.res[i] = (double)t1cdf_table((float)r.bt[i], a.t1tab + (size_t)(tab - 1) * T1TAB_N);
-        else
+        } else if (sizeof(R) == sizeof(double) && a.h1tab && dof <= R(H1_DOF_MAX)) {
+            const double x = r.bt[i], v = r.dof[i], rr = rsqrt(v + x * x);
+            const double t = h1_tail(sqrt(v) * rr, fabs(x) * rr, v, a.h1tab + (size_t)(tab / 3 * 4 + tab % 3) * H1_SIZE);
+            r.res[i] = x > 0.0 ? 1.0 - t : t;
+        } else
             r.res[i] = isinf(dof) ? (double)m_ncdf((R)r.bt[i])
                                   : (double)t1cdf_dev<R>((R)r.bt[i], dof, cst[tab * CST_STRIDE + CST_LGB]);
         if (r.se) r.se[i] = 0.0;
@@ -413,7 +418,7 @@ cudaError_t launch_integrals(const RecSet& r, const IntegArgs& a, int fp32, int 
         const long long blocks_needed = (r.nrec + 7) / 8;
         const int cap = nsm * 16;
         const int blocks = (int)(blocks_needed < cap ? blocks_needed : cap);
-        if (r.k == 2) e = launch_t2(r, a, fp32, blocks, st);
+        if (r.k == 2) e = launch_t2(r, a, fp32, blocks, nsm, st);
         else if (fp32) e = launch_lattice32(r.k, r, a, blocks, st);
         else e = launch_lattice64(r.k, r, a, blocks, st);
     }

@@ -248,6 +248,149 @@ __global__ void __launch_bounds__(T2P_WARPS * CF_WARP, 4) t2_pieces_kernel(RecSe
     }
 }
 
+// FP64 T_2 records of a finite dof (the pieces of t2_setup, the same nodes).  With v = nu + 1
+// and c = zs^2/v, the inner T_1 of a node is, where its argument z = zs sin(phi - phi*) is
+// negative, sin^v(phi_z) H(sigma) with sin phi_z = r = 1/sqrt(1 + c sin^2(phi - phi*)) and
+// sigma = sqrt(c) |sin(phi - phi*)| r, so the node's integrand is
+//   sin^(nu-1)(phi) T_1 = (sin(phi) r)^(nu-1) r^2 H(sigma):
+// one logarithm, one exponential, one rsqrt and a table polynomial.  On a piece where z > 0
+// it is sin^(nu-1)(phi) (1 - T_1(-z)): the same integrand subtracted from the piece's part of
+// the univariate T_1(.; nu), also by H.  z changes sign at phi* only, so its sign is one per
+// piece; 1 - T_1(-z) >= 1/2 there, so the subtraction costs at most one bit.  Where the piece's
+// part is itself a difference T_1(h) - T_1(k / rho) that loses more than two bits (rho < 0, phi*
+// near phi_h), the factor 1 - T_1(-z) is formed at the nodes, a second logarithm and exponential.
+//
+// Bound by the FP64 pipe (1/64 of the FP32 rate): a node was a continued fraction with six
+// divisions an iteration, about 1460 FP64 slots, and is about 100.  A warp takes up to 32
+// records: lane l sets up record l (two arctangents, three square roots, the univariate
+// part), then the warp runs each record's nodes over its lanes.  Measured on a GB300:
+// p = 16, q = 2, g = 8, n = 20,000 (3.2e5 records of 97 nodes): 72.1 -> 7.6 ms;
+// p = q = g = 2, n = 1000 (4000 records): 1.48 -> 0.22 ms.
+constexpr int T2D_WARPS = 8;
+enum { T2D_ANC0, T2D_PHIS, T2D_L0, T2D_L1, T2D_D0, T2D_SC, T2D_NU, T2D_N };
+
+// records outside the tables (|rho| = 1, dof above H1_DOF_MAX): the general routine
+static __device__ __noinline__ double t2_general_f64(const RecSet& r, const IntegArgs& a, long long i, int lane, int* nn)
+{
+    const double* c = a.cst64 + r.tab[i] * CST_STRIDE;
+    const double h = r.bt[2 * i], k = r.bt[2 * i + 1], rho = a.F[r.fac[i] + 2];
+    return t2cdf_warp<double>(h, k, rho, r.dof[i], (1.0 - rho) * (1.0 + rho),
+                              h * (rho > 0.0 ? rho : -rho) - (rho > 0.0 ? k : -k), c[CST_LGB], c[CST_LGB1], c[CST_C2],
+                              a.t2n, a.glx64, a.glw64, a.t2n, a.glx64, a.glw64, lane, nullptr, nn);
+}
+
+// chunk: records per warp, 1..32
+__global__ void __launch_bounds__(T2D_WARPS * CF_WARP, 2) t2_records_h1_kernel(RecSet r, IntegArgs a, int chunk)
+{
+    __shared__ double sf[T2D_WARPS][T2D_N][CF_WARP];
+    const int lane = threadIdx.x & (CF_WARP - 1), wib = threadIdx.x >> 5;
+    const long long warp = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const long long nwarps = ((long long)gridDim.x * blockDim.x) >> 5;
+    double (*R)[CF_WARP] = sf[wib];
+    const int n = a.t2n;
+    unsigned long long nodes = 0;  // this warp's quadrature nodes (profiler count)
+    for (long long base = warp * chunk; base < r.nrec; base += nwarps * chunk) {
+        const int cnt = r.nrec - base < chunk ? (int)(r.nrec - base) : chunk;
+        // bits: 0 split, 1 the first piece's z > 0 (the second one's is the opposite), 2 graded,
+        // 3 general routine, 4 the second piece's factor 1 - T_1(-z) at the nodes
+        int kind = 0, tab = 0;
+        double C2 = 0.0, part = 0.0;
+        if (lane < cnt) {
+            const long long i = base + lane;
+            const double h = r.bt[2 * i], k = r.bt[2 * i + 1], nu = r.dof[i];
+            const double rho = a.F[r.fac[i] + 2];  // L[1][0] of the 2 x 2 correlation factor
+            tab = r.tab[i];
+            C2 = a.cst64[tab * CST_STRIDE + CST_C2];
+            tab = tab / 3 * 4 + tab % 3;  // the table at this dof; the next one at dof + 1
+            if (!(fabs(rho) < 1.0) || !(nu <= H1_DOF_MAX)) {
+                kind = 8;
+            } else {
+                const double omr2 = (1.0 - rho) * (1.0 + rho), ar = fabs(rho), sg = rho > 0.0 ? 1.0 : -1.0;
+                const double cr = h * ar - sg * k, sn = sqrt(nu);
+                // D = phi_h - phi*, as in t2_setup; then the one angle that the pieces need
+                const double D = atan2(sn * cr, sg * h * k + ar * nu);
+                const bool split = rho != 0.0 && D > 0.0;
+                const double anc = split ? atan2(ar * sn, -sg * k) : atan2(sn, -h);
+                const double R2 = rho * rho * nu + k * k;
+                const bool pos0 = rho == 0.0 ? k > 0.0 : sg > 0.0;
+                kind = (split ? 1 : 0) | (pos0 ? 2 : 0) | (ar > 0.99 ? 4 : 0);
+                R[T2D_ANC0][lane] = anc;
+                R[T2D_PHIS][lane] = anc;
+                R[T2D_L0][lane] = -anc;
+                R[T2D_L1][lane] = D;
+                R[T2D_D0][lane] = split ? 0.0 : D;
+                R[T2D_SC][lane] = sqrt(R2 / (omr2 * nu));  // |zs| / sqrt(nu + 1)
+                R[T2D_NU][lane] = nu;
+                if (pos0 || split) {  // a piece with z > 0: its part of T_1(.; nu)
+                    const double* t1 = a.h1tab + (size_t)tab * H1_SIZE;
+                    double th = 0.0, ts = 0.0;
+                    const double rh = rsqrt(nu + h * h), rs = rsqrt(R2);
+                    if (!split || !pos0) th = h1_tail(sn * rh, fabs(h) * rh, nu, t1);
+                    if (split) ts = h1_tail(ar * sn * rs, fabs(k) * rs, nu, t1);
+                    const bool xneg = -sg * k > 0.0;  // cos phi* > 0: x* = k / rho < 0
+                    if (!split) part = h > 0.0 ? 1.0 - th : th;
+                    else if (pos0) part = xneg ? ts : 1.0 - ts;
+                    else {
+                        part = h <= 0.0 ? th - ts : xneg ? (1.0 - th) - ts : ts - th;
+                        if (part < 0.25 * (h <= 0.0 ? th : 1.0 - th)) {
+                            part = 0.0;
+                            kind |= 16;
+                        }
+                    }
+                }
+            }
+        }
+        __syncwarp();
+        double mine = 0.0;  // lane l: the quadrature sum of record l
+        for (int l = 0; l < cnt; ++l) {
+            const int kd = __shfl_sync(CF_FULL, kind, l), tb = __shfl_sync(CF_FULL, tab, l);
+            if (kd & 8) {
+                int nn = 0;
+                const double v = t2_general_f64(r, a, base + l, lane, &nn);
+                nodes += (unsigned long long)nn;
+                if (lane == l) mine = v;
+                continue;
+            }
+            const double sc = R[T2D_SC][l], num1 = R[T2D_NU][l] - 1.0;
+            const double* __restrict__ t2 = a.h1tab + (size_t)(tb + 1) * H1_SIZE;
+            double acc = 0.0;
+            for (int pc = 0; pc <= (kd & 1); ++pc) {
+                const double anc = pc ? R[T2D_PHIS][l] : R[T2D_ANC0][l], d0 = pc ? 0.0 : R[T2D_D0][l];
+                const double L = pc ? R[T2D_L1][l] : R[T2D_L0][l];
+                double s = 0.0;
+                for (int t = lane; t < n; t += CF_WARP) {
+                    const double u = a.glx64[t];
+                    double w = a.glw64[t], um = u;
+                    if (kd & 4) {  // nodes anchor + L u^3, weights 3 u^2
+                        um = u * u * u;
+                        w *= 3.0 * u * u;
+                    }
+                    const double off = L * um;
+                    const double sp = cf_sin_pi(anc + off);  // both arguments lie in [-pi, pi]
+                    const double q = sc * cf_sin_pi(d0 + off);
+                    const double rr = rsqrt(fma(q, q, 1.0));
+                    const double H = h1_eval(fabs(q) * rr, t2);
+                    if (kd & pc << 4)
+                        s = fma(w * exp(num1 * log(fabs(sp))), 1.0 - exp(num1 * log(rr)) * (rr * rr) * H, s);
+                    else
+                        s = fma(w * (rr * rr), exp(num1 * log(fabs(sp) * rr)) * H, s);
+                }
+                acc = fma(((kd >> 1) ^ pc) & !(kd & pc << 4) ? -fabs(L) : fabs(L), s, acc);
+            }
+            nodes += (unsigned long long)(n << (kd & 1));
+            acc = warp_sum(acc);
+            if (lane == l) mine = acc;
+        }
+        if (lane < cnt) {
+            const long long i = base + lane;
+            r.res[i] = kind & 8 ? mine : fma(C2, mine, part);
+            if (r.se) r.se[i] = 0.0;
+        }
+        __syncwarp();
+    }
+    if (a.nodes && lane == 0 && nodes) atomicAdd(a.nodes, nodes);
+}
+
 // Lanes per FP32 T_2 piece (finite dof), a.t2_group in {2, 4, 8, 16}; 32 (or 0: the CFUSN
 // model's records) = the warp-per-record kernel.
 template <int L>
@@ -260,8 +403,19 @@ static void go_group(const RecSet& r, const IntegArgs& a, int blocks, cudaStream
     else t2_pieces_kernel<L, false><<<gb > 0 ? gb : 1, T2P_WARPS * CF_WARP, 0, st>>>(r, a);
 }
 
-cudaError_t launch_t2(const RecSet& r, const IntegArgs& a, int fp32, int blocks, cudaStream_t st)
+cudaError_t launch_t2(const RecSet& r, const IntegArgs& a, int fp32, int blocks, int nsm, cudaStream_t st)
 {
+    if (!fp32 && a.h1tab) {
+        // records per warp: a record's set-up takes a warp about as long as 8 records' nodes
+        // over its lanes, so up to 32 share one; fewer where that would leave the SMs with
+        // less than 4 warps each (one per scheduler keeps the FP64 pipes busy)
+        long long ch = r.nrec / (4LL * nsm);
+        ch = ch < 1 ? 1 : ch > CF_WARP ? CF_WARP : ch;
+        const long long need = (r.nrec + ch * T2D_WARPS - 1) / (ch * T2D_WARPS);
+        const long long cap = 8LL * nsm;
+        t2_records_h1_kernel<<<(int)(need < cap ? need : cap), T2D_WARPS * CF_WARP, 0, st>>>(r, a, (int)ch);
+        return cudaGetLastError();
+    }
     const int L = a.t2_group;
     if (fp32 && L == 2) go_group<2>(r, a, blocks, st);
     else if (fp32 && L == 4) go_group<4>(r, a, blocks, st);

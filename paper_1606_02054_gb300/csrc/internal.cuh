@@ -202,7 +202,21 @@ struct IntegArgs {
     // exact E[log W] (else null): log(s^2) at every point of the chi tables, same layout
     const double* lchi64;
     const float* lchi32;
+    // FP64 T_1 and T_2 (else null): the tables of H1_* below, index 4 h + e
+    const double* h1tab;
 };
+
+// FP64 univariate t CDFs through a table per dof.  With sin phi = sqrt(v/(v + x^2)) and
+// sigma = |cos phi| = |x| / sqrt(v + x^2),
+//   T_1(-|x|; v) = sin^v(phi) H(sigma),   H(sigma) = (1 - sigma^2)^(-v/2) C int_sigma^1 (1 - s^2)^(v/2 - 1) ds,
+// C = Gamma((v+1)/2) / (Gamma(v/2) sqrt(pi)): H is analytic on [0, 1] (a Mills ratio in the
+// angle's coordinate, 1/2 at 0 and C/v at 1), so polynomials of degree H1_D on H1_CELLS equal
+// cells give it to 2e-17 relative at v = 130, 4e-16 at v = 260 (against 40-digit values;
+// smaller below).  Tables for the dofs nu_h + p + e, e = 0..3, index 4 h + e: a T_2 at dof
+// nu + p + j reads e = j and e = j + 1.  Above H1_DOF_MAX the continued fraction is used.
+constexpr int H1_CELLS = 64, H1_D = 9, H1_NC = H1_D + 1;
+constexpr int H1_SIZE = H1_CELLS * H1_NC;  // doubles per table
+constexpr double H1_DOF_MAX = 250.0;
 
 constexpr int T1TAB_N = 2048;
 constexpr int T2_NH = 64;
@@ -347,7 +361,7 @@ cudaError_t launch_tk_eval(int k, int count, const double* b, const double* V, c
                            long long* launches);
 cudaError_t launch_lattice32(int k, const RecSet& r, const IntegArgs& a, int blocks, cudaStream_t st);
 cudaError_t launch_lattice64(int k, const RecSet& r, const IntegArgs& a, int blocks, cudaStream_t st);
-cudaError_t launch_t2(const RecSet& r, const IntegArgs& a, int fp32, int blocks, cudaStream_t st);
+cudaError_t launch_t2(const RecSet& r, const IntegArgs& a, int fp32, int blocks, int nsm, cudaStream_t st);
 cudaError_t launch_factors_f32(const double* F, float* F32, long long count, cudaStream_t st,
                                long long* launches);
 cudaError_t launch_moments(const RecSet& r, const IntegArgs& a, int fp32, int nsm, cudaStream_t st,

@@ -246,7 +246,7 @@ __global__ void dof_consts_kernel(Dims D, Layout Ly, const double* __restrict__ 
         const double lt = lgamma(0.5 * (v + 1.0)) - lgamma(0.5 * v) - 0.5 * log(v * CF_PI);
         const double ltm = lgamma(0.5 * v) - lgamma(0.5 * (v - 1.0)) - 0.5 * log((v - 1.0) * CF_PI);
         const double c[CST_STRIDE] = {t1_lgb(v), t1_lgb(v + 1.0),
-                                      exp(lgamma(0.5 * (v + 1.0)) - lgamma(0.5 * v)) / sqrt(CF_PI),
+                                      cf_t_const(v),
                                       lt, v > 1.0 ? ltm : 0.0, lgamma(0.5 * v), 0.0, 0.0};
         for (int k = 0; k < CST_STRIDE; ++k) {
             c64[t * CST_STRIDE + k] = c[k];
@@ -321,4 +321,49 @@ __global__ void t1_table_kernel(int ndof, const double* __restrict__ dofs, const
         const double d = -exp(lt - lT) * (1.0 + w);
         tab[e] = make_float2((float)(lT / CF_LN2), (float)d);
     }
+}
+
+// Tables of H for the dofs v = nu_h + p + e (internal.cuh, H1_*): per cell, H at the H1_NC
+// Chebyshev nodes (from the continued fraction: with y = 1 - sigma^2 and a = v/2,
+// H = sigma C betacf(a, 1/2, y) / v where that one converges fast, else
+// 1/2 y^-a - sigma C betacf(1/2, a, sigma^2)), their Chebyshev coefficients and those as powers
+// of t in [-1/2, 1/2].  One value of the cell is taken off first, so the sums carry its small
+// changes only.  Blocks of 16 cells (blockIdx.x) of table 4h + e (blockIdx.y); a thread per
+// node, then per coefficient.
+constexpr int H1_TC = 16;  // cells per block
+__constant__ double h1_cheb[H1_NC][H1_NC] = {  // powers of x in T_n(x)
+    {1, 0, 0, 0, 0, 0, 0, 0, 0, 0},       {0, 1, 0, 0, 0, 0, 0, 0, 0, 0},
+    {-1, 0, 2, 0, 0, 0, 0, 0, 0, 0},      {0, -3, 0, 4, 0, 0, 0, 0, 0, 0},
+    {1, 0, -8, 0, 8, 0, 0, 0, 0, 0},      {0, 5, 0, -20, 0, 16, 0, 0, 0, 0},
+    {-1, 0, 18, 0, -48, 0, 32, 0, 0, 0},  {0, -7, 0, 56, 0, -112, 0, 64, 0, 0},
+    {1, 0, -32, 0, 160, 0, -256, 0, 128, 0}, {0, 9, 0, -120, 0, 432, 0, -576, 0, 256}};
+
+__global__ void __launch_bounds__(H1_TC * H1_NC) h1_table_kernel(const double* __restrict__ dofs,
+                                                                 double* __restrict__ tab, int emask)
+{
+    __shared__ double cosv[4 * H1_NC], f[H1_TC][H1_NC], cn[H1_TC][H1_NC];
+    const int h = blockIdx.y >> 2, e = blockIdx.y & 3;
+    if (!((emask >> e) & 1)) return;
+    const double v = dofs[3 * h] + e;
+    if (!(v <= H1_DOF_MAX + 4.0)) return;  // read by no record; also the normal limit
+    const int lc = threadIdx.x / H1_NC, j = threadIdx.x % H1_NC;
+    const int cell = blockIdx.x * H1_TC + lc;
+    if (threadIdx.x < 4 * H1_NC) cosv[threadIdx.x] = cospi(threadIdx.x / (2.0 * H1_NC));
+    __syncthreads();
+    const double C = cf_t_const(v), a = 0.5 * v;
+    const double sg = (cell + 0.5 + 0.5 * cosv[2 * j + 1]) * (1.0 / H1_CELLS);
+    const double y = (1.0 - sg) * (1.0 + sg);
+    const bool direct = y < (a + 1.0) / (a + 2.5);
+    const double cf = betacf_dev<double>(direct ? a : 0.5, direct ? 0.5 : a, direct ? y : sg * sg);
+    f[lc][j] = direct ? sg * C * cf / v : 0.5 * exp(-a * log1p(-sg * sg)) - sg * C * cf;
+    __syncthreads();
+    const double f0 = f[lc][H1_NC / 2];
+    double s = 0.0;
+    for (int i = 0; i < H1_NC; ++i) s += (f[lc][i] - f0) * cosv[(j * (2 * i + 1)) % (4 * H1_NC)];
+    cn[lc][j] = s * (j ? 2.0 / H1_NC : 1.0 / H1_NC);
+    __syncthreads();
+    s = 0.0;
+    for (int n = H1_NC - 1; n >= j; --n) s += cn[lc][n] * h1_cheb[n][j];
+    s *= (double)(1 << j);  // x = 2 t
+    tab[(size_t)blockIdx.y * H1_SIZE + cell * H1_NC + j] = j ? s : s + f0;
 }
