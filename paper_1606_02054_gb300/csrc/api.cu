@@ -93,6 +93,9 @@ struct cfust_ctx {
     Surrogate sur;    // learned surrogate of the level-0 and moment records
     bool single_pass = false;
     int *fix_count = nullptr, *fix_list = nullptr;
+    double* fix_part = nullptr;  // the fix-up's task sums (FixArgs) and counters
+    int* fix_done = nullptr;
+    int fix_cap = 0;
     // optional per-kernel-class timing (opts.profile)
     cudaEvent_t ev[CFUST_NPROF][2]{};
     bool pending[CFUST_NPROF]{};
@@ -377,7 +380,7 @@ static void free_all(cfust_ctx* c)
                     c->logf, c->u, c->elogu, c->eu,
                     c->euu, c->se, c->tau, c->partial, c->stats, c->flags, c->comp_status,
                     c->stage32, c->pd, c->pc, c->fix_count, c->fix_list, c->y32, c->F32, c->pr32, c->pd32, c->pc32, c->res32_l0, c->t1tab,
-                    c->work_dev, c->seg, c->lchi64, c->lchi32, c->h1tab};
+                    c->work_dev, c->seg, c->lchi64, c->lchi32, c->h1tab, c->fix_part, c->fix_done};
     for (void* b : bufs)
         if (b) cudaFree(b);
     for (RecSet& r : c->rec) {
@@ -540,6 +543,17 @@ extern "C" cfust_status cfust_create(cfust_ctx** out, int p, int q, int g, int64
         if (q == 2) ALLOC(res32_l0, 2 * ng);
     }
     ALLOC(fix_count, 1); ALLOC(fix_list, ng);
+    if (o.precision != CFUST_PREC_FP64) {
+        // room for the task sums of as many pairs as pay in parts (fewer for a small problem)
+        c->fix_cap = (int)std::min<size_t>(FIX_CAP, ng);
+        size_t per = 0;
+        for (int density = 0; density < 2; ++density) {
+            const FixArgs x = fix_args(q, c->single_pass, density, c->lat);
+            per = std::max(per, (size_t)x.ntask * x.nv);
+        }
+        ALLOC(fix_part, per * c->fix_cap);
+        ALLOC(fix_done, c->fix_cap);
+    }
     // T_2 records exist at q = 2 (level 0) and, in the recursion form, at q = 3, 4 (levels 1, 2)
     if (o.precision != CFUST_PREC_FP64 && (q == 2 || (!c->single_pass && (q == 3 || q == 4)))) {
         ALLOC(t1tab, (size_t)3 * g * T1TAB_N);
@@ -604,6 +618,8 @@ extern "C" cfust_status cfust_create(cfust_ctx** out, int p, int q, int g, int64
         if (ee != cudaSuccess && s == CFUST_OK)
             s = fail(nullptr, CFUST_ECUDA, std::string("cfust_create: cudaMemcpy: ") + cudaGetErrorString(ee));
     };
+    if (c->fix_done && (e = cudaMemset(c->fix_done, 0, sizeof(int) * c->fix_cap)) != cudaSuccess)
+        s = fail(nullptr, CFUST_ECUDA, std::string("cfust_create: cudaMemset: ") + cudaGetErrorString(e));
     cp(c->shf64, s64.data(), sizeof(double) * s64.size());
     cp(c->shf32, s32.data(), sizeof(float) * s32.size());
     if (c->single_pass && o.precision != CFUST_PREC_FP64 && q <= 4) {
@@ -979,7 +995,11 @@ static cfust_status launch_pairs(cfust_ctx* c, int density_only)
         a.flags = c->flags;
         n0 = c->launches;
         prof_begin(c, CFUST_PROF_FIXUP);
-        if ((e = launch_fixup(a, c->fix_count, c->fix_list, c->nsm, c->st, &c->launches)) != cudaSuccess)
+        FixArgs fx = fix_args(c->q, sp, density_only, c->lat);
+        fx.cap = c->fix_cap;
+        fx.part = c->fix_part;
+        fx.done = c->fix_done;
+        if ((e = launch_fixup(a, fx, c->fix_count, c->fix_list, c->nsm, c->st, &c->launches)) != cudaSuccess)
             return fail(c, CFUST_ECUDA, std::string("fix-up kernel: ") + cudaGetErrorString(e));
         prof_end(c, CFUST_PROF_FIXUP, c->launches - n0);
     }

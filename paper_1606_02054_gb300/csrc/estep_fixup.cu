@@ -1,9 +1,22 @@
-// estep_fixup.cu -- FP64 re-evaluation of listed pairs, one warp per pair.
+// estep_fixup.cu -- FP64 re-evaluation of listed pairs.
 //
 // In FP32 mode the lattice products of a pair whose alpha_s (eq 4) is below
 // 1e-35 leave the FP32 range; the combine kernel lists such pairs and this
 // kernel recomputes every integral of those pairs in FP64, then the same
 // assembly as the combine kernel.
+//
+// The list is usually short (none to a few dozen pairs of 1e5), and one pair is 8 million
+// FP64 operations at q = 4 on a pipe of 2 lanes per SM and clock: a warp that did a whole
+// pair held the E-step up for 6 to 38 ms while the rest of the GPU idled.  Up to fix_cap
+// pairs are therefore cut into tasks, a warp each: an integral of dimension >= 3 into its
+// shifts and those into parts of the points, a lower one whole.  The task sums go to
+// a buffer; the warp that finishes a pair's last task adds them in their order (the
+// same bits whichever warp it is) and assembles the pair.  Longer lists fill the GPU with a
+// warp per pair (FIX_CAP = 1024 pairs are 7 warps per SM).  Fix-up of one E-step on a GB300,
+// parameters with strongly skewed components: p = q = g = 4, n = 200,000, single pass
+// 12.2 -> 4.3 ms; the same with recursion moments, n = 20,000, 26.9 -> 2.0 ms; p = q = g = 6,
+// n = 50,000, single pass 37.9 -> 18.4 ms (there the FP64 pipe is busy: the pass of alpha_s
+// no longer runs twice).
 #include "estep_common.cuh"
 
 // T_k(bt; 0, corr(Lc Lc^T), nu) in FP64, warp-cooperative; chi = table of this dof.
@@ -33,7 +46,250 @@ __device__ double tk_fp64(int k, const double* bt, const double* Lc, double nu, 
     }
 }
 
-__global__ void __launch_bounds__(128) fixup_kernel(EstepArgs a, const int* count, const int* list)
+// Sums over the points i0 <= i < i1 of shift m of the lattice pass of T_K (the points and
+// factors of tk_lattice_warp / tk_lattice_mom_warp): out[0] = sum f and, MOM, out[1] = sum f s^2,
+// out[2] = sum f log s^2 (lrow given), out[3..] = sum f s rk y_r, then sum f rk^2 y_r y_c (c <= r).
+// All lanes; lane 0 writes.
+template <int K, bool MOM>
+__device__ void lattice_part(const double* bt, const double* Lc, const EstepArgs& a, const double* crow,
+                             const double* lrow, double rk, int m, int i0, int i1, int lane, double* out)
+{
+    constexpr int K2 = K * (K + 1) / 2, NY = MOM ? K : K - 1;
+    double b[K], invd[K], Lf[K][K];
+#pragma unroll
+    for (int r = 0; r < K; ++r) {
+        b[r] = bt[r];
+        invd[r] = 1.0 / Lc[r * K + r];
+#pragma unroll
+        for (int l = 0; l < K; ++l) Lf[r][l] = l < r ? Lc[r * K + l] : 0.0;
+    }
+    const int N = a.lat.N;
+    const double invN = 1.0 / (double)N;
+    double af = 0.0, aw = 0.0, al = 0.0, a1[K], a2[K2];
+#pragma unroll
+    for (int r = 0; r < K; ++r) a1[r] = 0.0;
+#pragma unroll
+    for (int r = 0; r < K2; ++r) a2[r] = 0.0;
+    for (int i = i0 + lane; i < i1; i += CF_WARP) {
+        const double s = crow[i];
+        double y[K], f = 1.0;
+#pragma unroll
+        for (int r = 0; r < K; ++r) {
+            double t = b[r] * s;
+#pragma unroll
+            for (int l = 0; l < r; ++l) t -= Lf[r][l] * y[l];
+            const double e = normcdf(t * invd[r]);
+            f *= e;
+            if (r < NY) {
+                double x = (double)(((long long)i * a.lat.z[r + 1]) % N) * invN + a.shf64[m * CF_MAXDIM + r + 1];
+                if (x >= 1.0) x -= 1.0;
+                double v = (1.0 - fabs(2.0 * x - 1.0)) * e;
+                v = v < Lim<double>::vmin() ? Lim<double>::vmin() : v;
+                v = v > Lim<double>::one_minus_ulp() ? Lim<double>::one_minus_ulp() : v;
+                y[r] = normcdfinv(v);
+            }
+            if (e <= Lim<double>::tiny()) f = 0.0;
+        }
+        af += f;
+        if (MOM) {
+            const double fs = f * s, w1 = fs * rk, w2 = f * (rk * rk);
+            aw += fs * s;
+            if (lrow) al += f * lrow[i];
+#pragma unroll
+            for (int r = 0; r < K; ++r) {
+                a1[r] += w1 * y[r];
+                const double t = w2 * y[r];
+#pragma unroll
+                for (int c = 0; c <= r; ++c) a2[r * (r + 1) / 2 + c] += t * y[c];
+            }
+        }
+    }
+    af = warp_sum(af);
+    if (lane == 0) out[0] = af;
+    if (MOM) {
+        aw = warp_sum(aw);
+        al = warp_sum(al);
+        if (lane == 0) { out[1] = aw; out[2] = al; }
+#pragma unroll
+        for (int r = 0; r < K; ++r) {
+            const double v = warp_sum(a1[r]);
+            if (lane == 0) out[3 + r] = v;
+        }
+#pragma unroll
+        for (int r = 0; r < K2; ++r) {
+            const double v = warp_sum(a2[r]);
+            if (lane == 0) out[3 + K + r] = v;
+        }
+    }
+}
+
+template <bool MOM>
+__device__ void lattice_part_k(int k, const double* bt, const double* Lc, const EstepArgs& a, const double* crow,
+                               const double* lrow, double rk, int m, int i0, int i1, int lane, double* out)
+{
+    switch (k) {
+    case 3: lattice_part<3, MOM>(bt, Lc, a, crow, lrow, rk, m, i0, i1, lane, out); break;
+    case 4: lattice_part<4, MOM>(bt, Lc, a, crow, lrow, rk, m, i0, i1, lane, out); break;
+    case 5: lattice_part<5, MOM>(bt, Lc, a, crow, lrow, rk, m, i0, i1, lane, out); break;
+    case 6: lattice_part<6, MOM>(bt, Lc, a, crow, lrow, rk, m, i0, i1, lane, out); break;
+    case 7: lattice_part<7, MOM>(bt, Lc, a, crow, lrow, rk, m, i0, i1, lane, out); break;
+    default: lattice_part<8, MOM>(bt, Lc, a, crow, lrow, rk, m, i0, i1, lane, out); break;
+    }
+}
+
+// A pair's integral: dimension, dof, chi table (0..2 from the component's first), factor
+// offset and standardised limits.  Numbered as its tasks run: alpha_s, alpha, then level 1 (r), then
+// level 2 (r, s); density passes and the single pass have alpha_s's only.
+__device__ void fix_integral(const EstepArgs& a, const double* F, const double* c, double d, int n, int& k,
+                             double& dof, int& tab, int& fac, double* bt)
+{
+    const int p = a.D.p, q = a.D.q, q1 = q - 1;
+    const double nu1 = F[a.Ly.scal + SC_NU] + p;
+    if (n < 2) {
+        k = q; dof = nu1 + 2.0 * n; tab = 2 * n; fac = fac_l0(a.Ly);
+        limits_l0(F, a.Ly, p, q, c, d, n, bt);
+    } else if (n < 2 + q) {
+        const int r = n - 2;
+        k = q1; dof = nu1 + 1.0; tab = 1; fac = fac_l1(a.Ly, q, r);
+        limits_l1(F, a.Ly, p, q, c, d, r, bt);
+    } else {
+        const int r = (n - 2 - q) / q1, s = (n - 2 - q) % q1;
+        k = q - 2; dof = nu1; tab = 0; fac = fac_l2(a.Ly, q, r, s);
+        limits_l2(F, a.Ly, p, q, c, d, r, s, bt);
+    }
+}
+
+__device__ void fix_store(const EstepArgs& a, long long pid, const PairOut& o, double se)
+{
+    const int q = a.D.q;
+    a.logf[pid] = o.logf;
+    if (a.se) a.se[pid] = se;
+    if (!(o.logf < INFINITY)) atomicOr(a.flags, KF_NAN);  // NaN or +inf; -inf is a null pair
+    if (a.density_only) return;
+    if (a.pr32) {
+        store_pr32(a.pr32 + pid * pr32_width(q), q, o);
+        return;
+    }
+    a.u[pid] = o.u;
+    a.elogu[pid] = o.elogu;
+    for (int k = 0; k < q; ++k) a.eu[pid * q + k] = o.eu[k];
+    for (int k = 0; k < q * q; ++k) a.euu[pid * q * q + k] = o.euu[k];
+}
+
+// Task t of pair number i of the list (fix_tasks): its sums into the pair's buffer.
+__device__ void fix_task(const EstepArgs& a, const FixArgs& x, long long pid, int t, int lane, double* out)
+{
+    const int p = a.D.p, q = a.D.q, h = (int)(pid / a.D.n);
+    const long long j = pid - (long long)h * a.D.n;
+    const double* F = a.F + (size_t)h * a.Ly.stride;
+    const size_t NM = (size_t)a.lat.N * a.lat.M;
+    double c[CF_MAXQ], d, logtp, bt[CF_MAXQ], dof;
+    pair_whiten(F, a.Ly, p, q, a.y + (size_t)j * p, &d, c, &logtp);
+    // the integral's number: 2 of dimension q, q of q - 1, the rest of q - 2
+    int n = 0, k, tab, fac;
+    for (;; ++n) {
+        const int w = fix_tasks_k(n < 2 ? q : n < 2 + q ? q - 1 : q - 2, x);
+        if (t < w) break;
+        t -= w;
+    }
+    fix_integral(a, F, c, d, n, k, dof, tab, fac, bt);
+    const double* chi = a.chi64 + (size_t)(3 * h + tab) * NM;
+    if (k < 3) {
+        const double v = tk_fp64(k, bt, F + fac, dof, chi, a, lane, nullptr);
+        if (lane == 0) out[0] = v;
+        return;
+    }
+    const int m = t / x.parts, part = t % x.parts;
+    const int i0 = (int)((long long)a.lat.N * part / x.parts), i1 = (int)((long long)a.lat.N * (part + 1) / x.parts);
+    const double* crow = chi + (size_t)m * a.lat.N;
+    if (a.single_pass && !a.density_only) {
+        const double* lrow = a.lchi64 ? a.lchi64 + (size_t)(3 * h) * NM + (size_t)m * a.lat.N : nullptr;
+        const double rk = isinf(dof) ? 1.0 : sqrt((dof + 2.0) / dof);
+        lattice_part_k<true>(k, bt, F + fac, a, crow, lrow, rk, m, i0, i1, lane, out);
+    } else {
+        lattice_part_k<false>(k, bt, F + fac, a, crow, nullptr, 1.0, m, i0, i1, lane, out);
+    }
+}
+
+// T_k from its tasks' sums (nv doubles a task): the mean over the shifts and its standard error;
+// all lanes
+__device__ double fix_value(const EstepArgs& a, const FixArgs& x, int k, const double* part, double* se)
+{
+    if (se) *se = 0.0;
+    if (k == 0) return 1.0;
+    if (k < 3) return part[0];
+    double mean = 0.0, m2 = 0.0;
+    for (int m = 0; m < a.lat.M; ++m) {
+        double s = 0.0;
+        for (int u = 0; u < x.parts; ++u) s += part[(size_t)(m * x.parts + u) * x.nv];
+        const double smean = s / (double)a.lat.N, delta = smean - mean;
+        mean += delta / (double)(m + 1);
+        m2 += delta * (smean - mean);
+    }
+    if (se) *se = a.lat.M > 1 ? sqrt(m2 / (double)(a.lat.M - 1) / (double)a.lat.M) : 0.0;
+    return mean;
+}
+
+// The pair from its tasks' sums; all lanes, sm: CF_MAXQ + CF_MAXQ (CF_MAXQ + 1) / 2 + 3 doubles
+__device__ void fix_assemble(const EstepArgs& a, const FixArgs& x, long long pid, const double* part, int lane,
+                             double* sm)
+{
+    const int p = a.D.p, q = a.D.q, q1 = q - 1, h = (int)(pid / a.D.n);
+    const long long j = pid - (long long)h * a.D.n;
+    const double* F = a.F + (size_t)h * a.Ly.stride;
+    double c[CF_MAXQ], d, logtp, se = 0.0;
+    pair_whiten(F, a.Ly, p, q, a.y + (size_t)j * p, &d, c, &logtp);
+    const double alpha_s = fix_value(a, x, q, part, &se);
+    PairOut o;
+    if (a.single_pass && !a.density_only) {
+        for (int v = lane; v < x.nv; v += CF_WARP) {  // sm[v]: sum v over the tasks, in order
+            double s = 0.0;
+            for (int t = 0; t < x.ntask; ++t) s += part[(size_t)t * x.nv + v];
+            sm[v] = s;
+        }
+        __syncwarp();
+        // m1 = L E[y/s], m2 = L E[y y^T/s^2] L^T (see tk_lattice_mom_warp)
+        const double* Lc = F + fac_l0(a.Ly);
+        const double* s1 = sm + 3;
+        const double* s2 = sm + 3 + q;
+        const double inv = sm[1] > 0.0 ? 1.0 / sm[1] : 0.0;
+        double m[CF_MAXQ + CF_MAXQ * (CF_MAXQ + 1) / 2];
+        for (int r = 0; r < q; ++r) {
+            double v = 0.0;
+            for (int l = 0; l <= r; ++l) v += Lc[r * q + l] * s1[l];
+            m[r] = v * inv;
+            for (int cc = 0; cc <= r; ++cc) {
+                double w2 = 0.0;
+                for (int i = 0; i <= r; ++i) {
+                    double w = 0.0;
+                    for (int l = 0; l <= cc; ++l) w += s2[i >= l ? i * (i + 1) / 2 + l : l * (l + 1) / 2 + i] * Lc[cc * q + l];
+                    w2 += Lc[r * q + i] * w;
+                }
+                m[q + r * (r + 1) / 2 + cc] = w2 * inv;
+            }
+        }
+        const double lw = a.lchi64 ? (sm[0] > 0.0 ? sm[2] / sm[0] : NAN) : NAN;
+        pair_assemble_sp(F, a.Ly, p, q, c, d, logtp, alpha_s, sm[1] / ((double)a.lat.N * a.lat.M), m, o, lw);
+        __syncwarp();
+    } else {
+        double alpha = 0.0, tq1[CF_MAXQ], tq2[CF_MAXQ * CF_MAXQ];
+        if (!a.density_only) {
+            const size_t wq = (size_t)fix_tasks_k(q, x) * x.nv, w1 = (size_t)fix_tasks_k(q1, x) * x.nv,
+                         w2 = (size_t)fix_tasks_k(q - 2, x) * x.nv;
+            alpha = fix_value(a, x, q, part + wq, nullptr);
+            for (int r = 0; r < q && q1 > 0; ++r) {
+                tq1[r] = fix_value(a, x, q1, part + 2 * wq + r * w1, nullptr);
+                for (int s = 0; s < q1 && q > 2; ++s)
+                    tq2[r * q1 + s] = fix_value(a, x, q - 2, part + 2 * wq + q * w1 + (size_t)(r * q1 + s) * w2, nullptr);
+            }
+        }
+        pair_assemble(F, a.Ly, p, q, c, d, logtp, alpha_s, alpha, tq1, tq2, a.density_only,
+                      a.cst64 + (size_t)(3 * h) * CST_STRIDE, o);
+    }
+    if (lane == 0) fix_store(a, pid, o, se);
+}
+
+__global__ void __launch_bounds__(128) fixup_kernel(EstepArgs a, FixArgs x, const int* count, const int* list)
 {
     const int lane = threadIdx.x & (CF_WARP - 1);
     const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -43,6 +299,25 @@ __global__ void __launch_bounds__(128) fixup_kernel(EstepArgs a, const int* coun
     const size_t NM = (size_t)a.lat.N * a.lat.M;
     __shared__ double slot[4][CF_MAXQ + CF_MAXQ * (CF_MAXQ + 1) / 2 + 3 + CF_MAXSHIFT];
     double* acc = slot[threadIdx.x >> 5];
+    if (cnt <= x.cap) {
+        const long long total = (long long)cnt * x.ntask;
+        for (long long t = warp; t < total; t += nwarps) {
+            const int i = (int)(t / x.ntask), k = (int)(t % x.ntask);
+            double* part = x.part + (size_t)i * x.ntask * x.nv;
+            fix_task(a, x, list[i], k, lane, part + (size_t)k * x.nv);
+            int last = 0;
+            if (lane == 0) {
+                __threadfence();
+                last = atomicAdd(x.done + i, 1) == x.ntask - 1;
+            }
+            last = __shfl_sync(CF_FULL, last, 0);
+            if (!last) continue;
+            __threadfence();
+            fix_assemble(a, x, list[i], part, lane, acc);
+            if (lane == 0) x.done[i] = 0;  // ready for the next E-step
+        }
+        return;
+    }
     for (int i = warp; i < cnt; i += nwarps) {
         const long long pid = list[i];
         const int h = (int)(pid / a.D.n);
@@ -75,19 +350,7 @@ __global__ void __launch_bounds__(128) fixup_kernel(EstepArgs a, const int* coun
             __syncwarp();
             PairOut o;
             pair_assemble_sp(F, a.Ly, p, q, c, d, logtp, alpha_s, alpha, m, o, lw);
-            if (lane == 0) {
-                a.logf[pid] = o.logf;
-                if (a.se) a.se[pid] = se;
-                if (!(o.logf < INFINITY)) atomicOr(a.flags, KF_NAN);  // NaN or +inf; -inf is a null pair
-                if (a.pr32) {
-                    store_pr32(a.pr32 + pid * pr32_width(q), q, o);
-                } else {
-                    a.u[pid] = o.u;
-                    a.elogu[pid] = o.elogu;
-                    for (int k = 0; k < q; ++k) a.eu[pid * q + k] = o.eu[k];
-                    for (int k = 0; k < q * q; ++k) a.euu[pid * q * q + k] = o.euu[k];
-                }
-            }
+            if (lane == 0) fix_store(a, pid, o, se);
             continue;
         }
         if (!a.density_only) {
@@ -105,26 +368,28 @@ __global__ void __launch_bounds__(128) fixup_kernel(EstepArgs a, const int* coun
         PairOut o;
         pair_assemble(F, a.Ly, p, q, c, d, logtp, alpha_s, alpha, tq1, tq2, a.density_only,
                       a.cst64 + (size_t)(3 * h) * CST_STRIDE, o);
-        if (lane == 0) {
-            a.logf[pid] = o.logf;
-            if (a.se) a.se[pid] = se;
-            if (!(o.logf < INFINITY)) atomicOr(a.flags, KF_NAN);  // NaN or +inf; -inf is a null pair
-            if (!a.density_only && a.pr32) {
-                store_pr32(a.pr32 + pid * pr32_width(q), q, o);
-            } else if (!a.density_only) {
-                a.u[pid] = o.u;
-                a.elogu[pid] = o.elogu;
-                for (int k = 0; k < q; ++k) a.eu[pid * q + k] = o.eu[k];
-                for (int k = 0; k < q * q; ++k) a.euu[pid * q * q + k] = o.euu[k];
-            }
-        }
+        if (lane == 0) fix_store(a, pid, o, se);
     }
 }
 
-cudaError_t launch_fixup(const EstepArgs& a, const int* count, const int* list, int nsm,
+// density: the tasks of a density pass, else of a full E-step (single: single-pass moments)
+FixArgs fix_args(int q, int single, int density, const Lattice& lat)
+{
+    FixArgs x{};
+    x.parts = lat.M >= 64 ? 1 : 64 / lat.M;
+    if (x.parts > (lat.N + 127) / 128) x.parts = (lat.N + 127) / 128;
+    x.tasks = lat.M * x.parts;
+    const bool mom = single && !density;
+    x.nv = mom ? 3 + q + q * (q + 1) / 2 : 1;
+    x.ntask = density || mom ? fix_tasks_k(q, x)
+                             : 2 * fix_tasks_k(q, x) + q * fix_tasks_k(q - 1, x) + q * (q - 1) * fix_tasks_k(q - 2, x);
+    return x;
+}
+
+cudaError_t launch_fixup(const EstepArgs& a, const FixArgs& x, const int* count, const int* list, int nsm,
                          cudaStream_t st, long long* launches)
 {
-    fixup_kernel<<<2 * nsm, 128, 0, st>>>(a, count, list);
+    fixup_kernel<<<4 * nsm, 128, 0, st>>>(a, x, count, list);
     ++*launches;
     return cudaGetLastError();
 }

@@ -321,6 +321,18 @@ struct EstepArgs {
     int* flags;
 };
 
+// The FP64 fix-up's tasks (estep_fixup.cu): up to cap listed pairs are cut into ntask tasks
+// each, whose nv sums go to part; done counts a pair's finished tasks (0 between launches).
+struct FixArgs {
+    int cap, ntask, nv;
+    int parts;     // parts of a shift's points
+    int tasks;     // tasks of an integral of dimension >= 3 (shifts x parts)
+    double* part;  // cap x ntask x nv
+    int* done;     // cap
+};
+constexpr int FIX_CAP = 1024;
+__host__ __device__ inline int fix_tasks_k(int k, const FixArgs& x) { return k >= 3 ? x.tasks : k > 0 ? 1 : 0; }
+
 // message returned by cfust_last_error(NULL) (calls without a context)
 // Device-side state of one EM fit run as a single CUDA graph (fit_graph.cu):
 // the iteration counter and the stopping decision live on the device so the
@@ -354,7 +366,8 @@ cudaError_t launch_plan(const PlanArgs& a, cudaStream_t st, long long* launches)
 cudaError_t launch_integrals(const RecSet& r, const IntegArgs& a, int fp32, int nsm,
                              cudaStream_t st, long long* launches);
 cudaError_t launch_combine(const CombineArgs& a, cudaStream_t st, long long* launches);
-cudaError_t launch_fixup(const EstepArgs& a, const int* count, const int* list, int nsm,
+FixArgs fix_args(int q, int single, int density, const Lattice& lat);
+cudaError_t launch_fixup(const EstepArgs& a, const FixArgs& x, const int* count, const int* list, int nsm,
                          cudaStream_t st, long long* launches);
 cudaError_t launch_tk_eval(int k, int count, const double* b, const double* V, const double* nu,
                            const IntegArgs& a, int fp32, double* out, double* se, cudaStream_t st,
