@@ -417,8 +417,8 @@ typedef struct {
                              normal CDFs (the FP32 forms of the integrators), the
                              K(K-1)/2 + 3K FMAs of the chain and the 2 + K + K(K+1)/2
                              FMAs of the weighted moment sums per point, no memory
-                             traffic; the best of 1, 2 and 4 independent points per
-                             thread; [0..2] unused (0) */
+                             traffic; the better of 1 and 2 independent pairs of points
+                             per thread (packed FP32); [0..2] unused (0) */
     double t2_nodes;      /* nodes per second of the FP32 T_2 quadrature alone -- per node
                              two sines, the sin^(nu-1) weight (lg2, ex2) and the inner T_1
                              from its per-dof table -- the best of 1, 2 and 4 independent

@@ -61,6 +61,7 @@ struct cfust_ctx {
     float* lchi32 = nullptr;
     double* shf64 = nullptr;
     float* shf32 = nullptr;
+    unsigned* latu = nullptr;  // lattice coordinates as 32-bit fractions (IntegArgs::latu)
     float4* wtab = nullptr;  // FP32 single pass: lattice coordinates of every (shift, point)
     double *glx64 = nullptr, *glw64 = nullptr;
     float *glx32 = nullptr, *glw32 = nullptr;
@@ -380,7 +381,7 @@ static void free_all(cfust_ctx* c)
                     c->logf, c->u, c->elogu, c->eu,
                     c->euu, c->se, c->tau, c->partial, c->stats, c->flags, c->comp_status,
                     c->stage32, c->pd, c->pc, c->fix_count, c->fix_list, c->y32, c->F32, c->pr32, c->pd32, c->pc32, c->res32_l0, c->t1tab,
-                    c->work_dev, c->seg, c->lchi64, c->lchi32, c->h1tab, c->fix_part, c->fix_done};
+                    c->work_dev, c->seg, c->lchi64, c->lchi32, c->h1tab, c->fix_part, c->fix_done, c->latu};
     for (void* b : bufs)
         if (b) cudaFree(b);
     for (RecSet& r : c->rec) {
@@ -523,6 +524,7 @@ extern "C" cfust_status cfust_create(cfust_ctx** out, int p, int q, int g, int64
         ALLOC(lchi64, ntab * NM);
         ALLOC(lchi32, ntab * NM);
     }
+    ALLOC(latu, (size_t)CF_MAXDIM * (33 + o.qmc_shifts));
     ALLOC(shf64, (size_t)o.qmc_shifts * CF_MAXDIM);
     ALLOC(shf32, (size_t)o.qmc_shifts * CF_MAXDIM);
     ALLOC(glx64, c->t2n); ALLOC(glw64, c->t2n); ALLOC(glx32, c->t2n); ALLOC(glw32, c->t2n);
@@ -620,6 +622,15 @@ extern "C" cfust_status cfust_create(cfust_ctx** out, int p, int q, int g, int64
     };
     if (c->fix_done && (e = cudaMemset(c->fix_done, 0, sizeof(int) * c->fix_cap)) != cudaSuccess)
         s = fail(nullptr, CFUST_ECUDA, std::string("cfust_create: cudaMemset: ") + cudaGetErrorString(e));
+    {
+        std::vector<uint32_t> lu((size_t)CF_MAXDIM * (33 + o.qmc_shifts));
+        const uint64_t N = (uint64_t)o.qmc_points;
+        for (int d = 0; d < CF_MAXDIM; ++d)  // rounded to nearest: step errors stay below 2^-33
+            for (int i = 0; i <= 32; ++i)
+                lu[d * 33 + i] = (uint32_t)((((uint64_t)i * c->lat.z[d] % N << 32) + N / 2) / N);
+        for (size_t k = 0; k < s64.size(); ++k) lu[CF_MAXDIM * 33 + k] = (uint32_t)(s64[k] * 4294967296.0);
+        cp(c->latu, lu.data(), sizeof(uint32_t) * lu.size());
+    }
     cp(c->shf64, s64.data(), sizeof(double) * s64.size());
     cp(c->shf32, s32.data(), sizeof(float) * s32.size());
     if (c->single_pass && o.precision != CFUST_PREC_FP64 && q <= 4) {
@@ -632,7 +643,9 @@ extern "C" cfust_status cfust_create(cfust_ctx** out, int p, int q, int g, int64
                 for (int d = 1; d <= q; ++d) {
                     double x = (double)(((long long)i * c->lat.z[d]) % N) / (double)N + s64[m * CF_MAXDIM + d];
                     if (x >= 1.0) x -= 1.0;
-                    wt[((size_t)m * N + i) * 4 * WQ + (d - 1)] = (float)(1.0 - std::fabs(2.0 * x - 1.0));
+                    // at most 1 - 2^-24: w Phi < 1, so that Phi^-1 needs no upper clamp
+                    wt[((size_t)m * N + i) * 4 * WQ + (d - 1)] =
+                        std::min((float)(1.0 - std::fabs(2.0 * x - 1.0)), 0.99999994f);
                 }
         if (cudaMalloc((void**)&c->wtab, sizeof(float) * wt.size()) != cudaSuccess) {
             free_all(c);
@@ -853,6 +866,7 @@ static IntegArgs integ_args(const cfust_ctx* c)
     ia.t1tab = c->t1tab;
     ia.h1tab = c->h1tab;
     ia.wtab = c->wtab;
+    ia.latu = c->latu;
     ia.nodes = nullptr;
     int t2g = 0, mp = 0;
     tune_lookup(c, &t2g, &mp);

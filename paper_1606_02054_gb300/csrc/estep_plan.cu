@@ -396,8 +396,8 @@ cudaError_t launch_moments(const RecSet& r, const IntegArgs& a, int fp32, int ns
                            long long* launches)
 {
     if (r.k < 3 || r.nrec == 0) return cudaSuccess;
-    const long long blocks_needed = (r.nrec + 7) / 8;
-    const int cap = nsm * 16;
+    const long long blocks_needed = (r.nrec + 7) / 8;  // FP32: 4 warps of 2 records; FP64: 8 of 1
+    const int cap = nsm * (fp32 ? 32 : 16);
     const int blocks = (int)(blocks_needed < cap ? blocks_needed : cap);
     cudaError_t e = fp32 ? launch_mom32(r.k, r, a, blocks, st) : launch_mom64(r.k, r, a, blocks, st);
     ++*launches;
@@ -414,9 +414,10 @@ cudaError_t launch_integrals(const RecSet& r, const IntegArgs& a, int fp32, int 
         else t1_records_kernel<double><<<grid_for(r.nrec, 128, 1 << 20), 128, 0, st>>>(r, a);
         e = cudaGetLastError();
     } else {
-        // one warp per record, 8 warps per block, enough blocks to fill every SM
+        // one warp per record, 8 warps per block (FP32 lattice: two records per warp, 4 warps),
+        // enough blocks to fill every SM
         const long long blocks_needed = (r.nrec + 7) / 8;
-        const int cap = nsm * 16;
+        const int cap = nsm * (fp32 && r.k >= 3 ? 32 : 16);
         const int blocks = (int)(blocks_needed < cap ? blocks_needed : cap);
         if (r.k == 2) e = launch_t2(r, a, fp32, blocks, nsm, st);
         else if (fp32) e = launch_lattice32(r.k, r, a, blocks, st);

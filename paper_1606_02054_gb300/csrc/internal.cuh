@@ -190,6 +190,9 @@ struct IntegArgs {
     // baker-transformed coordinates w_d = 1 - |2 frac(i z_d / N + shift_md) - 1|, d = 1..q,
     // in one float4 (computed in FP64 at creation; they are the same for every record)
     const float4* wtab;
+    // FP32 lattice coordinates as fractions of 2^32 (see mom_pair_f32): CF_MAXDIM x 33 (lane's
+    // first point i = lane: i z_d / N; then the step 32 z_d / N), then M x CF_MAXDIM shifts
+    const unsigned* latu;
     // T_2 records only (may be null): quadrature nodes evaluated, added once per warp
     // (the profiler's algorithmic work count)
     unsigned long long* nodes;

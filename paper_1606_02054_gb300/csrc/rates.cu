@@ -10,12 +10,12 @@
 //   - MUFU ex2, lg2, rcp (the approximate PTX forms the FP32 integrators use):
 //     8 independent chains per thread;
 //   - the single-pass integrand mix of dimension K: per lattice point K normal
-//     CDFs, K inverse normal CDFs (this library's FP32 forms, cf_ncdf_f32 and
-//     cf_ncdfinv_f32), the K(K-1)/2 + 3K FMAs of the chain and the
-//     2 + K + K(K+1)/2 FMAs of the weighted moment sums, with 1, 2 or 4
-//     independent points in flight per thread (the best of the three) and no
-//     memory traffic: the rate an implementation of the same algorithm could
-//     reach if it did nothing else;
+//     CDFs, K inverse normal CDFs (this library's packed FP32 forms, ncdf2_signed and
+//     ncdfinv2_abs), the K(K-1)/2 + 3K FMAs of the chain and the
+//     2 + K + K(K+1)/2 FMAs of the weighted moment sums, with 1 or 2 pairs of
+//     points in flight per thread (the better one) and no memory traffic: the
+//     rate an implementation of the same algorithm could reach if it did nothing
+//     else;
 //   - one node of the FP32 T_2 quadrature (two sines, the sin^(nu-1) weight, the
 //     inner T_1 from its table), 1, 2 or 4 independent nodes per thread (the best).
 // Every kernel runs a full grid (8 blocks of 256 threads per SM) for a fixed
@@ -95,21 +95,22 @@ __global__ void __launch_bounds__(kThreads) mufu_rate_kernel(float* out, int ite
     out[(size_t)blockIdx.x * blockDim.x + threadIdx.x] = s;
 }
 
-// The single-pass integrand of dimension K for two independent points per thread.
-// Coordinates w advance by a fixed irrational-like step (one add and one select per
-// coordinate, kept in [0, 1)); the chi variate s is taken from the first coordinate.
+// The single-pass integrand of dimension K, packed as mom_pair_f32 computes it (two points in
+// the halves of each value), P pairs in flight per thread.  Coordinates w advance by a fixed
+// irrational-like step (kept in [0, 1)); the chi variate s is taken from the first coordinate.
 template <int K, int P>
 __global__ void __launch_bounds__(kThreads) mix_rate_kernel(float* out, int iters)
 {
     constexpr int K2 = K * (K + 1) / 2;
     const float t0 = threadIdx.x * (1.0f / 4096.0f);
-    float b[K], invd[K], L[K][K];
+    f32x2 b[K];
+    float nL[K][K];
 #pragma unroll
     for (int r = 0; r < K; ++r) {
-        b[r] = 0.3f + 0.1f * r + t0;
-        invd[r] = 1.0f / (1.0f + 0.05f * r);
+        const float v = NCDF_SCALE / (1.0f + 0.05f * r);
+        b[r] = pk2((0.3f + 0.1f * r + t0) * v, (0.25f + 0.1f * r + t0) * v);
 #pragma unroll
-        for (int l = 0; l < K; ++l) L[r][l] = l < r ? 0.2f / (1 + r + l) : 0.f;
+        for (int l = 0; l < K; ++l) nL[r][l] = l < r ? -0.2f / (1 + r + l) * v : 0.f;
     }
     float w[P][K + 1], dw[K + 1];
 #pragma unroll
@@ -118,39 +119,33 @@ __global__ void __launch_bounds__(kThreads) mix_rate_kernel(float* out, int iter
 #pragma unroll
         for (int p = 0; p < P; ++p) w[p][d] = 0.5f * dw[d] + 0.125f * p + t0 * 0.1f;
     }
-    float af[P], aw[P], a1[P][K], a2[P][K2];
+    f32x2 af = 0ull, aw = 0ull, a1[K], a2[K2];
 #pragma unroll
-    for (int p = 0; p < P; ++p) {
-        af[p] = aw[p] = 0.f;
+    for (int r = 0; r < K; ++r) a1[r] = 0ull;
 #pragma unroll
-        for (int r = 0; r < K; ++r) a1[p][r] = 0.f;
-#pragma unroll
-        for (int r = 0; r < K2; ++r) a2[p][r] = 0.f;
-    }
-    const float rk = 1.1f, rk2 = rk * rk;
+    for (int r = 0; r < K2; ++r) a2[r] = 0ull;
     for (int i = 0; i < iters; ++i) {
 #pragma unroll
         for (int p = 0; p < P; ++p) {
-            const float s = 0.5f + w[p][0];
-            float y[K], f = 1.f;
+            const f32x2 s = pk2(0.5f + w[p][0]);
+            f32x2 y[K], f = 0ull;
 #pragma unroll
             for (int r = 0; r < K; ++r) {
-                float a = b[r] * s;
+                f32x2 t = mul2(b[r], s);
 #pragma unroll
-                for (int l = 0; l < r; ++l) a = fmaf(-L[r][l], y[l], a);
-                const float e = cf_ncdf_f32(a * invd[r]);
-                f *= e;
-                y[r] = cf_ncdfinv_f32(w[p][r + 1] * e);
+                for (int l = 0; l < r; ++l) t = fma2(pk2(nL[r][l]), y[l], t);
+                const f32x2 e = ncdf2_signed(t);
+                f = r == 0 ? e : mul2(f, e);
+                y[r] = ncdfinv2_abs(mul2(pk2(w[p][r + 1]), e));
             }
-            const float fs = f * s, w1 = fs * rk, w2 = f * rk2;
-            af[p] += f;
-            aw[p] = fmaf(fs, s, aw[p]);
+            af = add2(af, f);
+            aw = fma2(mul2(f, s), s, aw);
 #pragma unroll
             for (int r = 0; r < K; ++r) {
-                a1[p][r] = fmaf(w1, y[r], a1[p][r]);
-                const float t = w2 * y[r];
+                const f32x2 t = mul2(f, y[r]);
+                a1[r] = fma2(t, s, a1[r]);
 #pragma unroll
-                for (int c = 0; c <= r; ++c) a2[p][r * (r + 1) / 2 + c] = fmaf(t, y[c], a2[p][r * (r + 1) / 2 + c]);
+                for (int c = 0; c <= r; ++c) a2[r * (r + 1) / 2 + c] = fma2(t, y[c], a2[r * (r + 1) / 2 + c]);
             }
 #pragma unroll
             for (int d = 0; d <= K; ++d) {
@@ -159,16 +154,14 @@ __global__ void __launch_bounds__(kThreads) mix_rate_kernel(float* out, int iter
             }
         }
     }
-    float s = 0.f;
+    f32x2 s = add2(af, aw);
 #pragma unroll
-    for (int p = 0; p < P; ++p) {
-        s += af[p] + aw[p];
+    for (int r = 0; r < K; ++r) s = add2(s, a1[r]);
 #pragma unroll
-        for (int r = 0; r < K; ++r) s += a1[p][r];
-#pragma unroll
-        for (int r = 0; r < K2; ++r) s += a2[p][r];
-    }
-    out[(size_t)blockIdx.x * blockDim.x + threadIdx.x] = s;
+    for (int r = 0; r < K2; ++r) s = add2(s, a2[r]);
+    float s0, s1;
+    up2(s, s0, s1);
+    out[(size_t)blockIdx.x * blockDim.x + threadIdx.x] = s0 + s1;
 }
 
 // One node of the FP32 T_2 quadrature, per node: the two sines of the angle
@@ -261,7 +254,7 @@ cudaError_t calibrate(Timer& t, F launch_iters, int probe, double target, int* i
     return timed(t, [&] { launch_iters(*iters); }, secs);
 }
 
-// the best of 1, 2 and 4 independent points per thread (the rate of the arithmetic alone)
+// the better of 1 and 2 independent pairs of points per thread (the rate of the arithmetic alone)
 template <int K, int P>
 cudaError_t mix_rate_p(Timer& t, float* out, int blocks, double target, double* rate)
 {
@@ -269,7 +262,7 @@ cudaError_t mix_rate_p(Timer& t, float* out, int blocks, double target, double* 
     double s = 0.0;
     cudaError_t e = calibrate(t, [&](int n) { mix_rate_kernel<K, P><<<blocks, kThreads>>>(out, n); }, 64, target, &it, &s);
     if (e == cudaSuccess) {
-        const double r = (double)P * blocks * kThreads * it / s;
+        const double r = 2.0 * P * blocks * kThreads * it / s;
         if (r > *rate) *rate = r;
     }
     return e;
@@ -278,9 +271,8 @@ cudaError_t mix_rate_p(Timer& t, float* out, int blocks, double target, double* 
 template <int K>
 cudaError_t mix_rate(Timer& t, float* out, int blocks, double target, double* rate)
 {
-    cudaError_t e = mix_rate_p<K, 1>(t, out, blocks, target / 3, rate);
-    if (e == cudaSuccess) e = mix_rate_p<K, 2>(t, out, blocks, target / 3, rate);
-    if (e == cudaSuccess) e = mix_rate_p<K, 4>(t, out, blocks, target / 3, rate);
+    cudaError_t e = mix_rate_p<K, 1>(t, out, blocks, target / 2, rate);
+    if (e == cudaSuccess) e = mix_rate_p<K, 2>(t, out, blocks, target / 2, rate);
     return e;
 }
 
