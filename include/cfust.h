@@ -421,13 +421,13 @@ typedef struct {
                              per thread (packed FP32); [0..2] unused (0) */
     double t2_nodes;      /* nodes per second of the FP32 T_2 quadrature alone -- per node
                              two sines, the sin^(nu-1) weight (lg2, ex2) and the inner T_1
-                             from its per-dof table -- the best of 1, 2 and 4 independent
-                             nodes per thread */
+                             through its per-dof table -- the better of 1 and 2 independent
+                             packed pairs of nodes per thread */
 } cfust_rates;
 
 /* Run the microbenchmarks on `device` for about `seconds` (0 < seconds <= 5) in
  * all, on the legacy default stream, and fill *out.  Allocates one scratch
- * buffer (8 x SMs x 256 doubles and a 32 KB table) for the duration of the call.  Changes no
+ * buffer (8 x SMs x 256 doubles and a 4 KB table) for the duration of the call.  Changes no
  * device setting (clocks are read, never set). */
 cfust_status cfust_measure_rates(int device, double seconds, cfust_rates* out);
 

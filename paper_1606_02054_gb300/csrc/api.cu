@@ -21,7 +21,7 @@ __global__ void setup_components_kernel(Dims, Layout, const double*, const doubl
 __global__ void chi_table_kernel(int, int, const double*, const double*, Lattice, const double*, double, double*,
                                  float*, double*, float*);
 __global__ void dof_consts_kernel(Dims, Layout, const double*, int, double*, double*, float*);
-__global__ void t1_table_kernel(int, const double*, const double*, float2*, int);
+__global__ void h32_table_kernel(const double*, float4*, float*, int);
 __global__ void h1_table_kernel(const double*, double*, int);
 __global__ void widen_kernel(const float*, long long, Dims, double*);
 __global__ void widen_pairs_kernel(const float*, long long, int, double*, double*, double*, double*);
@@ -78,7 +78,8 @@ struct cfust_ctx {
     long long n_stats = 0;  // observations behind the current statistics (all shards'), the n of eq (18)
     int *flags = nullptr, *comp_status = nullptr;
     float* stage32 = nullptr;
-    float2* t1tab = nullptr;  // FP32 T_2: per-dof tables of T_1 at dof + 1
+    float4* h32tab = nullptr;   // FP32 T_2 (and the T_1 beside it): per-dof tables of H (H32_*)
+    float* h32scale = nullptr;
     double* h1tab = nullptr;  // FP64 T_2 (and the T_1 beside it): per-dof tables of H (H1_*)
     // mixed precision: FP32 copies of the observations and factor blocks
     bool mixed = false;
@@ -380,7 +381,7 @@ static void free_all(cfust_ctx* c)
                     c->glx64, c->glw64, c->glx32, c->glw32, c->glx32h, c->glw32h, c->glx32l, c->glw32l,
                     c->logf, c->u, c->elogu, c->eu,
                     c->euu, c->se, c->tau, c->partial, c->stats, c->flags, c->comp_status,
-                    c->stage32, c->pd, c->pc, c->fix_count, c->fix_list, c->y32, c->F32, c->pr32, c->pd32, c->pc32, c->res32_l0, c->t1tab,
+                    c->stage32, c->pd, c->pc, c->fix_count, c->fix_list, c->y32, c->F32, c->pr32, c->pd32, c->pc32, c->res32_l0, c->h32tab, c->h32scale,
                     c->work_dev, c->seg, c->lchi64, c->lchi32, c->h1tab, c->fix_part, c->fix_done, c->latu};
     for (void* b : bufs)
         if (b) cudaFree(b);
@@ -558,7 +559,8 @@ extern "C" cfust_status cfust_create(cfust_ctx** out, int p, int q, int g, int64
     }
     // T_2 records exist at q = 2 (level 0) and, in the recursion form, at q = 3, 4 (levels 1, 2)
     if (o.precision != CFUST_PREC_FP64 && (q == 2 || (!c->single_pass && (q == 3 || q == 4)))) {
-        ALLOC(t1tab, (size_t)3 * g * T1TAB_N);
+        ALLOC(h32tab, (size_t)4 * g * H32_CELLS);
+        ALLOC(h32scale, 4 * g);
     }
     if (o.precision == CFUST_PREC_FP64 && o.model == CFUST_MODEL_CFUST &&
         (q == 2 || (!c->single_pass && (q == 3 || q == 4)))) {
@@ -683,7 +685,7 @@ extern "C" cfust_status cfust_create(cfust_ctx** out, int p, int q, int g, int64
                     delete c;
                     return fail(nullptr, CFUST_ECUDA, "cfust_create: cudaEventCreate failed");
                 }
-    if ((c->t1tab || c->h1tab) && (cudaStreamCreateWithFlags(&c->st2, cudaStreamNonBlocking) != cudaSuccess ||
+    if ((c->h32tab || c->h1tab) && (cudaStreamCreateWithFlags(&c->st2, cudaStreamNonBlocking) != cudaSuccess ||
                      cudaEventCreateWithFlags(&c->ev_fork, cudaEventDisableTiming) != cudaSuccess ||
                      cudaEventCreateWithFlags(&c->ev_join, cudaEventDisableTiming) != cudaSuccess)) {
         free_all(c);
@@ -793,39 +795,25 @@ static cfust_status launch_setup(cfust_ctx* c, int density_only)
     LAUNCHED();
     dof_consts_kernel<<<1, 64, 0, c->st>>>(c->D, c->Ly, c->F, 3 * c->g, c->dofs, c->cst64, c->cst32);
     LAUNCHED();
-    if (c->t1tab) {
-        // tables t = 3h + j hold T_1 at dof nu_h + p + j + 1: the FP32 T_2 records read those of
-        // their own dof, the q = 2 level-1 T_1 records (dof nu + p + 1) the j = 0 table
-        int jmask = 0;
-        for (int l = 0; l < 3; ++l) {
-            const RecSet& r = c->rec[l];
-            if (r.nrec == 0) continue;
-            if (r.k == 2) jmask |= l == 0 ? 5 : l == 1 ? 2 : 1;  // dofs nu+p (+2), nu+p+1, nu+p
-            if (r.k == 1 && l == 1) jmask |= 1;
-        }
-        const int total = 3 * c->g * T1TAB_N;
-        CU(cudaEventRecord(c->ev_fork, c->st));
-        CU(cudaStreamWaitEvent(c->st2, c->ev_fork, 0));
-        t1_table_kernel<<<(total + 255) / 256, 256, 0, c->st2>>>(3 * c->g, c->dofs, c->cst64, c->t1tab, jmask);
-        LAUNCHED();
-        CU(cudaEventRecord(c->ev_join, c->st2));
-        c->t1_pending = true;
-    }
-    if (c->h1tab) {
-        // tables 4h + e hold H at dof nu_h + p + e: a T_2 record of index 3h + j reads e = j and
-        // j + 1, a T_1 record e = j (level 0: j = 0, and 2 unless density_only; level 1: 1; level 2: 0)
+    if (c->h32tab || c->h1tab) {
+        // tables 4h + e hold H at dof nu_h + p + e: a T_2 record of index 3h + j reads e = j + 1, in FP64
+        // also e = j, a T_1 record e = j (level 0: j = 0, and 2 unless density_only; level 1: 1; level 2: 0)
         int emask = 0;
         for (int l = 0; l < (density_only ? 1 : 3); ++l) {
             const RecSet& r = c->rec[l];
             if (r.nrec == 0) continue;
             const int j0 = l == 1 ? 1 : 0;
-            if (r.k == 2) emask |= 3 << j0 | (l == 0 && !density_only ? 3 << 2 : 0);
+            const int t2 = (c->h1tab ? 3 : 2) << j0;
+            if (r.k == 2) emask |= t2 | (l == 0 && !density_only ? t2 << 2 : 0);
             if (r.k == 1) emask |= 1 << j0;
         }
-        if (emask) {
+        if (emask) {  // on the side stream, beside the plan
             CU(cudaEventRecord(c->ev_fork, c->st));
             CU(cudaStreamWaitEvent(c->st2, c->ev_fork, 0));
-            h1_table_kernel<<<dim3(H1_CELLS / 16, 4 * c->g), 16 * H1_NC, 0, c->st2>>>(c->dofs, c->h1tab, emask);
+            if (c->h1tab)
+                h1_table_kernel<<<dim3(H1_CELLS / 16, 4 * c->g), 16 * H1_NC, 0, c->st2>>>(c->dofs, c->h1tab, emask);
+            else
+                h32_table_kernel<<<dim3(H32_CELLS / 32, 4 * c->g), 128, 0, c->st2>>>(c->dofs, c->h32tab, c->h32scale, emask);
             LAUNCHED();
             CU(cudaEventRecord(c->ev_join, c->st2));
             c->t1_pending = true;
@@ -835,7 +823,7 @@ static cfust_status launch_setup(cfust_ctx* c, int density_only)
         cudaError_t e = launch_factors_f32(c->F, c->F32, (long long)c->g * c->Ly.stride, c->st, &c->launches);
         if (e != cudaSuccess) return fail(c, CFUST_ECUDA, std::string("factor copy: ") + cudaGetErrorString(e));
     }
-    prof_end(c, CFUST_PROF_SETUP, 2 + (c->mixed ? 1 : 0) + (c->t1tab || c->h1tab ? 1 : 0));
+    prof_end(c, CFUST_PROF_SETUP, 2 + (c->mixed ? 1 : 0) + (c->h32tab || c->h1tab ? 1 : 0));
     if (c->q >= 3) {
         prof_begin(c, CFUST_PROF_CHI);
         // the single-pass E-step reads only the dof nu+p tables (index 3h)
@@ -863,7 +851,9 @@ static IntegArgs integ_args(const cfust_ctx* c)
     ia.t2n = c->t2n;
     ia.glx32h = c->glx32h; ia.glw32h = c->glw32h;
     ia.t2n_lo = c->t2n_lo; ia.glx32l = c->glx32l; ia.glw32l = c->glw32l;
-    ia.t1tab = c->t1tab;
+    ia.h32tab = c->h32tab;
+    ia.h32scale = c->h32scale;
+    ia.h32_case = 0;
     ia.h1tab = c->h1tab;
     ia.wtab = c->wtab;
     ia.latu = c->latu;
@@ -890,7 +880,7 @@ static cfust_status launch_pairs(cfust_ctx* c, int density_only)
     pa.pd = c->pd; pa.pc = c->pc;
     pa.pd32 = c->mixed ? c->pd32 : nullptr; pa.pc32 = c->mixed ? c->pc32 : nullptr;
     // mixed form at q = 2: the level-1 T_1s are table lookups done by combine, not records
-    const int fuse_l1 = c->mixed && c->q == 2 && !c->single_pass && c->t1tab != nullptr;
+    const int fuse_l1 = c->mixed && c->q == 2 && !c->single_pass && c->h32tab != nullptr;
     pa.fuse_l1 = fuse_l1;
     pa.blocks = 16 * c->nsm;
     pa.L0 = c->rec[0]; pa.L1 = c->rec[1]; pa.L2 = c->rec[2]; pa.LM = c->rec[3];
@@ -980,7 +970,7 @@ static cfust_status launch_pairs(cfust_ctx* c, int density_only)
     CombineArgs ca;
     ca.D = c->D; ca.Ly = c->Ly; ca.cst64 = c->cst64; ca.cst32 = c->cst32; ca.F = c->F; ca.pd = c->pd; ca.pc = c->pc;
     ca.pd32 = c->mixed ? c->pd32 : nullptr; ca.pc32 = c->mixed ? c->pc32 : nullptr;
-    ca.t1tab = c->t1tab; ca.fuse_l1 = fuse_l1;
+    ca.h32tab = c->h32tab; ca.h32scale = c->h32scale; ca.fuse_l1 = fuse_l1;
     ca.F32 = c->mixed ? c->F32 : nullptr;
     ca.L0 = pa.L0; ca.L1 = c->rec[1]; ca.L2 = c->rec[2]; ca.LM = c->rec[3];
     ca.density_only = density_only; ca.single_pass = sp; ca.fp32 = fp32;
@@ -1962,14 +1952,15 @@ extern "C" cfust_status cfust_tk_eval(cfust_ctx* c, int k, int count, const doub
     r.nrec = count;
     double *dF = nullptr, *t64 = nullptr, *k64 = nullptr;
     float *t32 = nullptr, *k32 = nullptr;
-    float2* t1t = nullptr;
-    // FP32 T_2 reads per-case T_1 tables (32 KB each) when the cases are few
-    const bool use_t1tab = k == 2 && c->opts.precision != CFUST_PREC_FP64 && count <= 4096;
+    float4* h32 = nullptr;
+    float* h32s = nullptr;
+    // FP32 T_2 reads per-case tables of H (4 KB each) when the cases are few
+    const bool use_h32 = k == 2 && c->opts.precision != CFUST_PREC_FP64 && count <= 4096;
     cudaError_t e = cudaSuccess;
     auto cleanup = [&]() {
         cudaFree(r.bt); cudaFree(r.fac); cudaFree(r.tab); cudaFree(r.dof); cudaFree(r.res);
         cudaFree(r.se); cudaFree(dF); cudaFree(t64); cudaFree(t32); cudaFree(k64); cudaFree(k32);
-        cudaFree(t1t); cudaFree(r.t2f);
+        cudaFree(h32); cudaFree(h32s); cudaFree(r.t2f);
     };
     if ((e = dalloc(&r.bt, bt.size())) != cudaSuccess || (e = dalloc(&r.fac, count)) != cudaSuccess ||
         (e = dalloc(&r.tab, count)) != cudaSuccess || (e = dalloc(&r.dof, count)) != cudaSuccess ||
@@ -1979,7 +1970,8 @@ extern "C" cfust_status cfust_tk_eval(cfust_ctx* c, int k, int count, const doub
         (e = dalloc(&k32, (size_t)count * CST_STRIDE)) != cudaSuccess ||
         (e = dalloc(&t64, lattice ? NM * count : 1)) != cudaSuccess ||
         (e = dalloc(&t32, lattice ? NM * count : 1)) != cudaSuccess ||
-        (e = dalloc(&t1t, use_t1tab ? (size_t)count * T1TAB_N : 1)) != cudaSuccess ||
+        (e = dalloc(&h32, use_h32 ? (size_t)count * H32_CELLS : 1)) != cudaSuccess ||
+        (e = dalloc(&h32s, use_h32 ? (size_t)count : 1)) != cudaSuccess ||
         (k == 2 && c->opts.precision != CFUST_PREC_FP64 && (e = dalloc(&r.t2f, (size_t)2 * count)) != cudaSuccess)) {
         cleanup();
         return fail(c, CFUST_ENOMEM, std::string("cfust_tk_eval: ") + cudaGetErrorString(e));
@@ -2009,14 +2001,15 @@ extern "C" cfust_status cfust_tk_eval(cfust_ctx* c, int k, int count, const doub
             c->launches++;
             if ((e = cudaGetLastError())) break;
         }
-        if (use_t1tab) {
-            const int total = count * T1TAB_N;
-            t1_table_kernel<<<(total + 255) / 256, 256, 0, c->st>>>(count, r.dof, k64, t1t, 7);
+        if (use_h32) {
+            h32_table_kernel<<<dim3(H32_CELLS / 32, count), 128, 0, c->st>>>(r.dof, h32, h32s, 0);
             c->launches++;
             if ((e = cudaGetLastError())) break;
         }
         IntegArgs ia = integ_args(c);
-        ia.t1tab = use_t1tab ? t1t : nullptr;
+        ia.h32tab = use_h32 ? h32 : nullptr;
+        ia.h32scale = h32s;
+        ia.h32_case = 1;
         ia.h1tab = nullptr;  // the tables are per component, not per case
         ia.cst64 = k64;
         ia.cst32 = k32;

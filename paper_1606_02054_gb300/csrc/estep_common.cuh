@@ -333,6 +333,76 @@ __device__ inline void pair_assemble_sp(const double* F, const Layout& Ly, int p
         }
 }
 
+// q = 2: the assembly with the level-1 T_1 inside, in T = float (the mixed form) or double.
+// With w0 = c_r^2 / (nu1 S_rr) and w = the T_1's argument squared over its dof nu2 = nu1 + 1,
+// the t densities and that T_1 are powers of 1 + w0 and 1 + w,
+//   t_1(c_r; S_rr, nu1)              = K (S_rr)^(-1/2) (1 + w0)^(-(nu1+1)/2)
+//   t_1(c'; V, nu2 - 2)              = K' V^(-1/2) E,   E = (1 + w)^(-(nu2-1)/2)
+//   T_1(-|b|; nu2)                   = E (1 + w)^(-1/2) H(sigma), sigma^2 = w / (1 + w)
+// so a coordinate takes two log1p and two exp, where the general routine takes four logarithms,
+// two exponentials and the T_1.  H from the component's table at dof nu2 (FP64: scale unused).
+// cst: the per-dof constants of dof nu+p.
+__device__ __forceinline__ float h_lookup(float sigma, const float4* tab, float scale) { return h32_eval(sigma, tab, scale); }
+__device__ __forceinline__ double h_lookup(double sigma, const double* tab, float) { return h1_eval(sigma, tab); }
+__device__ __forceinline__ float m_log1p(float x) { return log1pf(x); }
+__device__ __forceinline__ double m_log1p(double x) { return log1p(x); }
+__device__ __forceinline__ float m_rsqrt(float x) { return rsqrtf(x); }
+__device__ __forceinline__ double m_rsqrt(double x) { return rsqrt(x); }
+
+template <typename T, typename TAB, typename O>
+__device__ __forceinline__ void pair_assemble_q2(const T* F, const Layout& Ly, int p, const T* c, T d, T logtp,
+                                                 T alpha_s, T alpha, const T* cst, const TAB* tab, float scale, O& o)
+{
+    if (!(alpha_s > T(0))) return pair_null(2, 0, o);
+    // eq (4): log t_p + log alpha_s in T, q log 2 added in FP64
+    o.logf = 2 * 0.6931471805599453 + (double)(logtp + m_log(alpha_s));
+    const T nu = F[Ly.scal + SC_NU], nu1 = nu + T(p), nu2 = nu1 + T(1);
+    const T k0 = (nu + d) / nu1, ia = T(1) / alpha_s;
+    const T u = alpha * ia / k0;  // eq (13)
+    o.u = u;
+    o.elogu = u - m_log(T(0.5) * (nu + d)) - T(1) / k0 + F[Ly.scal + SC_PSI];  // eq (15)
+    T xi[2], H[4];
+#pragma unroll
+    for (int r = 0; r < 2; ++r) {
+        const int b = 1 - r;
+        const T* blk = F + Ly.l1 + r * Ly.l1s;  // m_r, the Schur complement
+        const T mv = blk[0], sch = blk[1];
+        const T Srr = k0 * F[Ly.Lam + 3 * r];
+        const T w0 = c[r] * c[r] / (nu1 * Srr);
+        const T E0 = cst[CST_ET1] * m_rsqrt(Srr) * m_exp(T(-0.5) * (nu1 + T(1)) * m_log1p(w0));
+        const T cp = c[b] - mv * c[r];
+        const T sc1 = (nu1 / nu2) * (T(1) + w0) * k0, V0 = sc1 * sch;
+        const T w = cp * cp / (nu2 * V0);
+        const T E = m_exp(T(-0.5) * (nu2 - T(1)) * m_log1p(w));
+        const T rq = m_rsqrt(T(1) + w);
+        const T Tm = E * rq * h_lookup(m_sqrt(w) * rq, tab, scale);
+        const T t1 = cp > T(0) ? T(1) - Tm : Tm;
+        // V = nu2/(nu2-2) V0
+        const T kq = nu2 / (nu2 - T(2));
+        const T xip = cst[CST_ET1M] * m_rsqrt(kq * V0) * E;
+        xi[r] = E0 * t1;
+        H[3 * r] = c[r] * xi[r];
+        H[2 * r + b] = E0 * (mv * c[r] * t1 - kq * V0 * xip);
+    }
+    const T* Lam = F + Ly.Lam;
+    T Lx[2];
+#pragma unroll
+    for (int a = 0; a < 2; ++a) {
+        Lx[a] = (Lam[2 * a] * xi[0] + Lam[2 * a + 1] * xi[1]) * ia;
+        o.eu[a] = u * c[a] + Lx[a];  // eq (16)
+    }
+#pragma unroll
+    for (int a = 0; a < 2; ++a)
+#pragma unroll
+        for (int b = 0; b <= a; ++b) {  // eq (17), symmetrised
+            const T lh1 = Lam[2 * a] * H[b] + Lam[2 * a + 1] * H[2 + b];
+            const T lh2 = Lam[2 * b] * H[a] + Lam[2 * b + 1] * H[2 + a];
+            const T v = u * c[a] * c[b] + (c[a] * Lx[b] + Lx[a] * c[b]) + Lam[2 * a + b] - T(0.5) * (lh1 + lh2) * ia;
+            o.euu[2 * a + b] = v;
+            o.euu[2 * b + a] = v;
+        }
+}
+
 // Mixed precision: the assembly of pair_assemble in FP32 (log f keeps the
 // FP64 log t_p and adds log alpha_s computed in FP32).
 // F: the component's FP32 factor block, cst its FP32 per-dof constants (conversions from

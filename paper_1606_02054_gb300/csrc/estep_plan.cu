@@ -236,15 +236,24 @@ __global__ void __launch_bounds__(128) combine_mixed_kernel(CombineArgs a)
         const float alpha = a.density_only ? 0.0f : a.L0.res32 ? a.L0.res32[r1] : (float)a.L0.res[r1];
         const float* F32 = a.F32 + (size_t)h * a.Ly.stride;
         float tq1[CF_MAXQ], tq2[Q == 2 ? 1 : CF_MAXQ * CF_MAXQ];
+        PairOutF of;
+        if (Q == 2 && a.fuse_l1 && !a.density_only && !isinf(F32[a.Ly.scal + SC_NU])) {
+            // the level-1 T_1 (dof nu+p+1, table 4h + 1) formed inside the assembly
+            pair_assemble_q2<float>(F32, a.Ly, p, c, d, logtp, alpha_s, alpha, a.cst32 + (size_t)(3 * h) * CST_STRIDE,
+                                    a.h32tab + (size_t)(4 * h + 1) * H32_CELLS, a.h32scale[4 * h + 1], of);
+            a.logf[pid] = of.logf;
+            if (a.se) a.se[pid] = se;
+            if (!(of.logf < INFINITY)) atomicOr(a.flags, KF_NAN);  // NaN or +inf; -inf is a null pair
+            store_pr32(a.pr32 + pid * pr32_width(2), 2, of);
+            continue;
+        }
         if (!a.density_only) {
             if (Q == 2 && a.fuse_l1) {
-                // the level-1 T_1 at dof nu+p+1 (table 3h holds T_1 at that dof; the normal
-                // limit takes Phi), from the same FP32 limits the records would carry
-                const bool nrm = isinf(F32[a.Ly.scal + SC_NU]);
+                // the normal limit: the level-1 records' Phi from the same FP32 limits
                 for (int r = 0; r < 2; ++r) {
                     float bt1[CF_MAXQ];
                     limits_l1<float>(F32, a.Ly, p, 2, c, d, r, bt1);
-                    tq1[r] = nrm ? m_ncdf(bt1[0]) : t1cdf_table(bt1[0], a.t1tab + (size_t)(3 * h) * T1TAB_N);
+                    tq1[r] = m_ncdf(bt1[0]);
                 }
             } else {
                 for (int r = 0; r < q && q1 > 0; ++r) tq1[r] = (float)a.L1.res[pid * q + r];
@@ -252,7 +261,6 @@ __global__ void __launch_bounds__(128) combine_mixed_kernel(CombineArgs a)
             if (Q != 2 && q1 > 1)
                 for (int i = 0; i < q * q1; ++i) tq2[i] = (float)a.L2.res[pid * q * q1 + i];
         }
-        PairOutF of;
         pair_assemble_f32(F32, a.Ly, p, q, c, d, logtp, alpha_s, alpha, tq1, tq2,
                           a.density_only, a.cst32 + (size_t)(3 * h) * CST_STRIDE, of);
         a.logf[pid] = of.logf;
@@ -323,10 +331,8 @@ __global__ void __launch_bounds__(128) combine_kernel(CombineArgs a)
     }
 }
 
-// FP32 with the T_1 tables (a.t1tab) and a record of table index 3h + 1 (dof nu + p + 1,
-// the q = 2 moments' level 1): T_1 by interpolation in the table 3h, which holds T_1 at
-// that dof (see t1cdf_table), instead of the continued fraction.  FP64 with the tables of H
-// (a.h1tab): T_1 at dof nu_h + p + e, table index 3h + e, from the table 4h + e.
+// With the tables of H (FP32: a.h32tab, FP64: a.h1tab): T_1 at dof nu_h + p + e, table index
+// 3h + e, from the table 4h + e instead of the continued fraction.
 template <typename R>
 __global__ void __launch_bounds__(128) t1_records_kernel(RecSet r, IntegArgs a)
 {
@@ -335,11 +341,12 @@ __global__ void __launch_bounds__(128) t1_records_kernel(RecSet r, IntegArgs a)
          i += (long long)gridDim.x * blockDim.x) {
         const R dof = (R)r.dof[i];  // infinite: the normal limit, Phi
         const int tab = r.tab[i];
-        if (sizeof(R) == sizeof(float) && a.t1tab && tab % 3 == 1 && !isinf(dof)) {
-            r.res[i] = (double)t1cdf_table((float)r.bt[i], a.t1tab + (size_t)(tab - 1) * T1TAB_N);
+        const int ti = tab / 3 * 4 + tab % 3;
+        if (sizeof(R) == sizeof(float) && a.h32tab && !isinf(dof)) {
+            r.res[i] = (double)t1cdf_h32((float)r.bt[i], (float)dof, a.h32tab + (size_t)ti * H32_CELLS, a.h32scale[ti]);
         } else if (sizeof(R) == sizeof(double) && a.h1tab && dof <= R(H1_DOF_MAX)) {
             const double x = r.bt[i], v = r.dof[i], rr = rsqrt(v + x * x);
-            const double t = h1_tail(sqrt(v) * rr, fabs(x) * rr, v, a.h1tab + (size_t)(tab / 3 * 4 + tab % 3) * H1_SIZE);
+            const double t = h1_tail(sqrt(v) * rr, fabs(x) * rr, v, a.h1tab + (size_t)ti * H1_SIZE);
             r.res[i] = x > 0.0 ? 1.0 - t : t;
         } else
             r.res[i] = isinf(dof) ? (double)m_ncdf((R)r.bt[i])

@@ -28,13 +28,14 @@ __global__ void __launch_bounds__(256) t2_records_kernel(RecSet r, IntegArgs a)
             omr2 = (R)((1.0 - rho64) * (1.0 + rho64));
             cr = (R)(h64 * (rho64 > 0.0 ? rho64 : -rho64) - (rho64 > 0.0 ? k64 : -k64));
         }
-        const float2* tab = f32 && a.t1tab ? a.t1tab + (size_t)r.tab[i] * T1TAB_N : nullptr;
+        const int ti = a.h32_case ? r.tab[i] : r.tab[i] / 3 * 4 + r.tab[i] % 3 + 1;
+        const float4* tab = f32 && a.h32tab ? a.h32tab + (size_t)ti * H32_CELLS : nullptr;
         int nn = 2 * a.t2n;
         const double v = isinf(nu) ? phi2_warp<R>(h, k, rho, a.t2n, glx, glw, lane)
                                    : t2cdf_warp<R>(h, k, rho, nu, omr2, cr, c[CST_LGB], c[CST_LGB1], c[CST_C2], a.t2n,
                                        glx, glw, f32 ? T2_NH : a.t2n,
                                        f32 ? (const R*)a.glx32h : glx, f32 ? (const R*)a.glw32h : glw,
-                                       lane, tab, &nn, f32 ? a.t2n_lo : 0, f32 ? (const R*)a.glx32l : nullptr,
+                                       lane, tab, tab ? a.h32scale[ti] : 0.0f, &nn, f32 ? a.t2n_lo : 0, f32 ? (const R*)a.glx32l : nullptr,
                                        f32 ? (const R*)a.glw32l : nullptr);
         nodes += (unsigned long long)nn;
         if (lane == 0) {
@@ -47,7 +48,7 @@ __global__ void __launch_bounds__(256) t2_records_kernel(RecSet r, IntegArgs a)
 }
 
 // FP32 T_2 records (finite dof), scheduled by quadrature piece.  A warp takes a chunk of
-// 64 records; lane l sets up records l and l + 32 (the angles of the split, the pieces'
+// up to 128 records; lane l sets up records l, l + 32, ... (the angles of the split, the pieces'
 // lengths and node counts, once per record), the chunk's pieces (one or two per record,
 // 8 to 64 nodes each) are ordered by node set and dealt to the warp's 32/L groups of L
 // lanes, a group sums its piece's nodes (lane sub takes nodes sub, sub + L, ...), and the
@@ -56,23 +57,33 @@ __global__ void __launch_bounds__(256) t2_records_kernel(RecSet r, IntegArgs a)
 // lanes while a neighbour's second piece runs.  The same L gives the same bits.
 namespace {
 constexpr int T2P_WARPS = 8;
-constexpr int T2P_CH = 2 * CF_WARP;  // records per warp chunk
+constexpr int T2P_R = 4;                 // records per lane of a warp's chunk
+constexpr int T2P_CH = T2P_R * CF_WARP;  // records per warp chunk
 // a record's set-up fields, one array per field (consecutive records in distinct banks)
-enum { T2F_ANC0, T2F_PHIS, T2F_L0, T2F_L1, T2F_D0, T2F_ZS, T2F_NU, T2F_LGB1, T2F_N };
+enum { T2F_ANC, T2F_L0, T2F_L1, T2F_D0, T2F_SC, T2F_NU, T2F_LGB1, T2F_N };
 constexpr int T2P_NMAX = 64;  // nodes per piece at most (t2_nodes <= 64, T2_NH = 64)
 // node sets: the classes 0-4 of t2_lo_class, then t2n nodes, then the graded pieces' T2_NH
 constexpr int T2P_NK = T2_LO_NCLS + 2, T2P_KN = T2_LO_NCLS, T2P_KG = T2_LO_NCLS + 1;
 }  // namespace
 
-// TAB: the inner T_1 from the per-dof tables (a.t1tab), else by its continued fraction
+// TAB: the inner T_1 from the per-dof tables of H (a.h32tab), else by its continued fraction.
+// With c = zs^2/(nu + 1), r = 1/sqrt(1 + c sin^2(phi - phi*)) and sigma = sqrt(c)
+// |sin(phi - phi*)| r the node's T_1(-|z|) is T = r^(nu+1) H(sigma), and z's sign is one per
+// piece: the integrand is sin^(nu-1)(phi) (0 + T) or (1 - T).  A lane takes two neighbouring
+// nodes at a time in packed FP32.  The kernel was bound by instruction issue: 77 instructions a
+// node (two folded sines, two lg2, two ex2, a Hermite interpolation) are about 40, and a record's set-up
+// takes two arctangents (cf_atan2_f32) instead of three from the library.
+// p = 16, q = 2, g = 8, n = 2,000,000 (3.2e7 records, 25 nodes each) on a GB300: 2.66 -> 2.1 ms;
+// a node is 60 cycles of a scheduler (FMA about 40, MUFU 32), a record's set-up, ordering and
+// rounds about 15 nodes' worth.
 template <int L, bool TAB>
-__global__ void __launch_bounds__(T2P_WARPS * CF_WARP, 4) t2_pieces_kernel(RecSet r, IntegArgs a)
+__global__ void __launch_bounds__(T2P_WARPS * CF_WARP, 4) t2_pieces_kernel(RecSet r, IntegArgs a, int rows)
 {
     constexpr int G = CF_WARP / L;
     __shared__ float srf[T2P_WARPS][T2F_N][T2P_CH];
-    __shared__ int srt[T2P_WARPS][T2P_CH];                     // table index
+    __shared__ int srt[T2P_WARPS][T2P_CH];                     // 2 table index + sign bit
     __shared__ unsigned char srk[T2P_WARPS][2 * T2P_CH];       // node set of piece (record << 1) | pc
-    __shared__ float sgx[T2P_NK][T2P_NMAX], sgw[T2P_NK][T2P_NMAX];  // the node sets
+    __shared__ __align__(8) float sgx[T2P_NK][T2P_NMAX], sgw[T2P_NK][T2P_NMAX];  // the node sets
     __shared__ float spsum[T2P_WARPS][T2P_CH][2];
     __shared__ unsigned char sitem[T2P_WARPS][2 * T2P_CH];  // (record << 1) | piece
     const int lane = threadIdx.x & (CF_WARP - 1), wib = threadIdx.x >> 5;
@@ -93,24 +104,26 @@ __global__ void __launch_bounds__(T2P_WARPS * CF_WARP, 4) t2_pieces_kernel(RecSe
         } else if (kd == T2P_KN) {
             if (i < a.t2n) { x = a.glx32[i]; w = a.glw32[i]; }
         } else if (i < T2_NH) {
-            x = a.glx32h[i]; w = a.glw32h[i];
+            const float u = a.glx32h[i];
+            x = u * u * u; w = a.glw32h[i] * (3.0f * u * u);
         }
         sgx[kd][i] = x;
         sgw[kd][i] = w;
     }
     __syncthreads();
     unsigned long long nodes = 0;  // this lane's records' quadrature nodes (profiler count)
-    for (long long base = warp * T2P_CH; base < r.nrec; base += nwarps * T2P_CH) {
-        // phase 1: set-up of records lane and lane + 32
-        int np[2], kind[2][2];
-        float C2[2], lim[2];
-        bool limit[2];
+    const int chunk = rows * CF_WARP;  // records of a warp's chunk, at most T2P_CH
+    for (long long base = warp * chunk; base < r.nrec; base += nwarps * chunk) {
+        // phase 1: set-up of records lane, lane + 32, ...
+        int np[T2P_R], kind[T2P_R][2];
+        float C2[T2P_R], lim[T2P_R];
+        bool limit[T2P_R];
 #pragma unroll
-        for (int m = 0; m < 2; ++m) {
+        for (int m = 0; m < T2P_R; ++m) {
             const int rr = lane + m * CF_WARP;
             const long long i = base + rr;
             np[m] = 0; kind[m][0] = kind[m][1] = T2P_KN; C2[m] = 0.0f; lim[m] = 0.0f; limit[m] = false;
-            if (i >= r.nrec) continue;
+            if (m >= rows || i >= r.nrec) continue;
             const float* c = a.cst32 + r.tab[i] * CST_STRIDE;
             float h, k, rho, nu, omr2, cr;
             if (r.t2f) {  // FP32 record fields written by the plan
@@ -138,50 +151,55 @@ __global__ void __launch_bounds__(T2P_WARPS * CF_WARP, 4) t2_pieces_kernel(RecSe
             // fewer nodes where the integrand is smooth enough (t2_lo_class, per piece)
             const bool lo = a.t2n_lo > 0 && !graded && fabsf(rho) < T2_LO_RHO && nu >= T2_LO_DOF_MIN &&
                             nu <= T2_LO_DOF_MAX;
-            const T2Setup<float> S = t2_setup<float>(h, k, rho, nu, omr2, cr);
-            np[m] = S.split ? 2 : 1;
-            kind[m][0] = graded ? T2P_KG : lo ? t2_lo_class(S.L0, nu, S.zs) : T2P_KN;
-            kind[m][1] = graded ? T2P_KG : lo ? t2_lo_class(S.L1, nu, S.zs) : T2P_KN;
-            nodes += (unsigned long long)(count(kind[m][0]) + (S.split ? count(kind[m][1]) : 0));
-            Rf[T2F_ANC0][rr] = S.anc0; Rf[T2F_PHIS][rr] = S.phis;
-            Rf[T2F_L0][rr] = S.L0; Rf[T2F_L1][rr] = S.L1;
-            Rf[T2F_D0][rr] = S.d0; Rf[T2F_ZS][rr] = S.zs;
+            // the angles of t2_setup: D = phi_h - phi*, and phi* or phi_h as the pieces' anchor
+            const float sg = rho > 0.0f ? 1.0f : -1.0f, ar = fabsf(rho), sn = sqrt_approx(nu);
+            const float D = cf_atan2_f32(sn * cr, fmaf(sg * h, k, ar * nu));
+            const bool split = rho != 0.0f && D > 0.0f;
+            const float anc = cf_atan2_f32(split ? ar * sn : sn, split ? -sg * k : -h);
+            const float c1 = fmaf(rho * rho, nu, k * k) * ptx_rcp_approx(omr2 * nu);  // zs^2 / (nu + 1)
+            np[m] = split ? 2 : 1;
+            kind[m][0] = graded ? T2P_KG : lo ? t2_lo_class(anc, nu, c1 * (nu + 1.0f)) : T2P_KN;
+            kind[m][1] = graded ? T2P_KG : lo ? t2_lo_class(D, nu, c1 * (nu + 1.0f)) : T2P_KN;
+            nodes += (unsigned long long)(count(kind[m][0]) + (split ? count(kind[m][1]) : 0));
+            Rf[T2F_ANC][rr] = anc;
+            Rf[T2F_L0][rr] = -anc; Rf[T2F_L1][rr] = D;
+            Rf[T2F_D0][rr] = split ? 0.0f : D;
+            Rf[T2F_SC][rr] = sqrt_approx(c1);
             Rf[T2F_NU][rr] = nu; Rf[T2F_LGB1][rr] = c[CST_LGB1];
-            Rt[rr] = r.tab[i];
+            // z > 0 on the first piece: bit 0 (the second piece's sign is the opposite)
+            const bool pos0 = rho == 0.0f ? k > 0.0f : sg > 0.0f;
+            const int ti = a.h32_case ? r.tab[i] : r.tab[i] / 3 * 4 + r.tab[i] % 3 + 1;
+            Rt[rr] = 2 * ti + (pos0 ? 1 : 0);
             Rk[2 * rr] = (unsigned char)kind[m][0];
             Rk[2 * rr + 1] = (unsigned char)kind[m][1];
         }
-        // the chunk's pieces, grouped by node set (the sets present in the chunk, in order)
-        int M = 0;
-        unsigned present = 0;
+        // the chunk's pieces, grouped by node set: a counting sort with the seven sets' counts (at most
+        // 256 each) in 9-bit fields of one 64-bit word, scanned over the lanes once for all sets
+        unsigned long long mine = 0;
 #pragma unroll
-        for (int m = 0; m < 2; ++m)
+        for (int m = 0; m < T2P_R; ++m)
 #pragma unroll
             for (int pc = 0; pc < 2; ++pc)
-                if (pc < np[m]) present |= 1u << kind[m][pc];
-        present = __reduce_or_sync(CF_FULL, present);
-        while (present) {
-            const int kd = __ffs(present) - 1;
-            present &= present - 1;
-            int cnt = 0;
+                if (pc < np[m]) mine += 1ull << (9 * kind[m][pc]);
+        unsigned long long incl = mine;
 #pragma unroll
-            for (int m = 0; m < 2; ++m)
-#pragma unroll
-                for (int pc = 0; pc < 2; ++pc) cnt += pc < np[m] && kind[m][pc] == kd;
-            int incl = cnt;
-#pragma unroll
-            for (int o = 1; o < CF_WARP; o <<= 1) {
-                const int v = __shfl_up_sync(CF_FULL, incl, o);
-                if (lane >= o) incl += v;
-            }
-            int pos = M + incl - cnt;
-#pragma unroll
-            for (int m = 0; m < 2; ++m)
-#pragma unroll
-                for (int pc = 0; pc < 2; ++pc)
-                    if (pc < np[m] && kind[m][pc] == kd) items[pos++] = (unsigned char)(((lane + m * CF_WARP) << 1) | pc);
-            M += __shfl_sync(CF_FULL, incl, CF_WARP - 1);
+        for (int o = 1; o < CF_WARP; o <<= 1) {
+            const unsigned long long v = __shfl_up_sync(CF_FULL, incl, o);
+            if (lane >= o) incl += v;
         }
+        const unsigned long long total = __shfl_sync(CF_FULL, incl, CF_WARP - 1);
+        // field k of this product is the number of pieces in sets 0..k
+        const unsigned long long upto = total * 0x0040201008040201ull;
+        const int M = (int)(upto >> 54) & 511;  // field 6: the last set
+        unsigned long long pos = (upto << 9) + incl - mine;  // field k: this lane's next place in set k
+#pragma unroll
+        for (int m = 0; m < T2P_R; ++m)
+#pragma unroll
+            for (int pc = 0; pc < 2; ++pc)
+                if (pc < np[m]) {
+                    items[(pos >> (9 * kind[m][pc])) & 511] = (unsigned char)(((lane + m * CF_WARP) << 1) | pc);
+                    pos += 1ull << (9 * kind[m][pc]);
+                }
         __syncwarp();
         // phase 2: rounds of G pieces, one per group
         for (int it0 = 0; it0 < M; it0 += G) {
@@ -195,30 +213,59 @@ __global__ void __launch_bounds__(T2P_WARPS * CF_WARP, 4) t2_pieces_kernel(RecSe
                 const int nn = count(kd);
                 const float* gx = sgx[kd];
                 const float* gw = sgw[kd];
-                const bool graded = kd == T2P_KG;
-                const float anc = pc ? Rf[T2F_PHIS][rr] : Rf[T2F_ANC0][rr];
+                const float anc = Rf[T2F_ANC][rr];
                 const float Lp = pc ? Rf[T2F_L1][rr] : Rf[T2F_L0][rr];
                 const float d0 = pc ? 0.0f : Rf[T2F_D0][rr];
-                const float zs = Rf[T2F_ZS][rr], nu = Rf[T2F_NU][rr], lgb1 = Rf[T2F_LGB1][rr];
+                const float sc = Rf[T2F_SC][rr], nu = Rf[T2F_NU][rr];
                 const float num1 = nu - 1.0f, nu1 = nu + 1.0f;
-                const float2* tab = TAB ? a.t1tab + (size_t)Rt[rr] * T1TAB_N : nullptr;
-                // the node's integrand; the piece's sum is scaled by |L| once, below
-                auto node = [&](float off) {
-                    const float sp = cf_sin_pi(anc + off);  // both arguments lie in [-pi, pi]
-                    const float sd = cf_sin_pi(d0 + off);
-                    const float z = zs * sd;
-                    float t1;
-                    if constexpr (TAB) t1 = t1cdf_table(z, tab);
-                    else t1 = t1cdf_dev<float>(z, nu1, lgb1);
-                    return ptx_ex2_approx(num1 * ptx_lg2_approx(sp)) * t1;
-                };
-                if (graded) {  // nodes anchor + L u^3, weights 3 u^2
-                    for (int t = sub; t < nn; t += L) {
-                        const float u = gx[t];
-                        acc = fmaf(gw[t] * (3.0f * u * u), node(Lp * (u * u * u)), acc);
+                const bool pos = ((Rt[rr] ^ pc) & 1) != 0;
+                // the nodes' sum is scaled by |L| once, below; graded sets are stored as u^3, 3 u^2 w
+                if constexpr (TAB) {
+                    const int ti = Rt[rr] >> 1;
+                    const float4* __restrict__ tab = a.h32tab + (size_t)ti * H32_CELLS;
+                    const float scale = __ldg(a.h32scale + ti);
+                    const float A = pos ? 1.0f : 0.0f, B = pos ? -1.0f : 1.0f;
+                    f32x2 acc2 = 0ull;
+                    for (int t = 2 * sub; t < nn; t += 2 * L) {  // an odd count is padded with weight 0
+                        const f32x2 off = mul2(*reinterpret_cast<const f32x2*>(gx + t), pk2(Lp));
+                        const f32x2 sp = sin2_signed(add2(off, pk2(anc)));
+                        const f32x2 q = mul2(sin2_signed(add2(off, pk2(d0))), pk2(sc));
+                        float D0, D1, s0, s1;
+                        up2(fma2(q, q, pk2(1.0f)), D0, D1);
+                        up2(mul2(sp, sp), s0, s1);
+                        const float r0 = rsqrt_approx(D0), r1 = rsqrt_approx(D1);
+                        const f32x2 rr2 = pk2(r0, r1);
+                        float e0, e1, g0, g1, u0, u1;
+                        // the powers through the logarithms of the squares: lg2's absolute error near 1
+                        // enters with (nu - 1)/2
+                        up2(mul2(pk2(ptx_lg2_approx(s0), ptx_lg2_approx(s1)), pk2(0.5f * num1)), e0, e1);
+                        up2(mul2(pk2(ptx_lg2_approx(D0), ptx_lg2_approx(D1)), pk2(-0.5f * num1)), g0, g1);
+                        // H(sigma) as h32_eval
+                        up2(fma2(mul2(q & 0x7fffffff7fffffffull, rr2), pk2(scale), pk2(-0.5f)), u0, u1);
+                        const f32x2 u = pk2(fminf(u0, (float)H32_CELLS - 0.51f), fminf(u1, (float)H32_CELLS - 0.51f));
+                        const f32x2 mm = add2(u, pk2(12582912.0f));
+                        float m0, m1, t0, t1;
+                        up2(mm, m0, m1);
+                        up2(fma2(add2(mm, pk2(-12582912.0f)), pk2(-1.0f), u), t0, t1);
+                        const float4 c0 = __ldg(tab + (__float_as_int(m0) & (H32_CELLS - 1)));
+                        const float4 c1 = __ldg(tab + (__float_as_int(m1) & (H32_CELLS - 1)));
+                        const f32x2 H = pk2(fmaf(fmaf(fmaf(c0.w, t0, c0.z), t0, c0.y), t0, c0.x),
+                                            fmaf(fmaf(fmaf(c1.w, t1, c1.z), t1, c1.y), t1, c1.x));
+                        const f32x2 T = mul2(mul2(pk2(ptx_ex2_approx(g0), ptx_ex2_approx(g1)), mul2(rr2, rr2)), H);
+                        const f32x2 f = mul2(pk2(ptx_ex2_approx(e0), ptx_ex2_approx(e1)), fma2(T, pk2(B), pk2(A)));
+                        acc2 = fma2(*reinterpret_cast<const f32x2*>(gw + t), f, acc2);
                     }
+                    float a0, a1;
+                    up2(acc2, a0, a1);
+                    acc = a0 + a1;
                 } else {
-                    for (int t = sub; t < nn; t += L) acc = fmaf(gw[t], node(Lp * gx[t]), acc);
+                    const float lgb1 = Rf[T2F_LGB1][rr], zs = sc * sqrtf(nu1);
+                    for (int t = sub; t < nn; t += L) {
+                        const float off = Lp * gx[t];
+                        const float sp = cf_sin_pi(anc + off), sd = cf_sin_pi(d0 + off);
+                        const float t1 = t1cdf_dev<float>(pos ? fabsf(zs * sd) : -fabsf(zs * sd), nu1, lgb1);
+                        acc = fmaf(gw[t], ptx_ex2_approx(num1 * ptx_lg2_approx(sp)) * t1, acc);
+                    }
                 }
                 acc *= fabsf(Lp);
             }
@@ -226,12 +273,12 @@ __global__ void __launch_bounds__(T2P_WARPS * CF_WARP, 4) t2_pieces_kernel(RecSe
             if (it < M && sub == 0) P[rr][pc] = acc;
         }
         __syncwarp();
-        // phase 3: records lane and lane + 32
+        // phase 3: records lane, lane + 32, ...
 #pragma unroll
-        for (int m = 0; m < 2; ++m) {
+        for (int m = 0; m < T2P_R; ++m) {
             const int rr = lane + m * CF_WARP;
             const long long i = base + rr;
-            if (i >= r.nrec) continue;
+            if (m >= rows || i >= r.nrec) continue;
             float v;
             if (limit[m]) v = lim[m];
             else v = C2[m] * (np[m] == 2 ? P[rr][0] + P[rr][1] : P[rr][0]);
@@ -276,7 +323,7 @@ static __device__ __noinline__ double t2_general_f64(const RecSet& r, const Inte
     const double h = r.bt[2 * i], k = r.bt[2 * i + 1], rho = a.F[r.fac[i] + 2];
     return t2cdf_warp<double>(h, k, rho, r.dof[i], (1.0 - rho) * (1.0 + rho),
                               h * (rho > 0.0 ? rho : -rho) - (rho > 0.0 ? k : -k), c[CST_LGB], c[CST_LGB1], c[CST_C2],
-                              a.t2n, a.glx64, a.glw64, a.t2n, a.glx64, a.glw64, lane, nullptr, nn);
+                              a.t2n, a.glx64, a.glw64, a.t2n, a.glx64, a.glw64, lane, nullptr, 0.0f, nn);
 }
 
 // chunk: records per warp, 1..32
@@ -394,13 +441,18 @@ __global__ void __launch_bounds__(T2D_WARPS * CF_WARP, 2) t2_records_h1_kernel(R
 // Lanes per FP32 T_2 piece (finite dof), a.t2_group in {2, 4, 8, 16}; 32 (or 0: the CFUSN
 // model's records) = the warp-per-record kernel.
 template <int L>
-static void go_group(const RecSet& r, const IntegArgs& a, int blocks, cudaStream_t st)
+static void go_group(const RecSet& r, const IntegArgs& a, int nsm, cudaStream_t st)
 {
-    const long long per_block = (long long)T2P_WARPS * T2P_CH;
-    const long long need = (r.nrec + per_block - 1) / per_block;
-    const int gb = (int)(need < blocks ? need : blocks);
-    if (a.t1tab) t2_pieces_kernel<L, true><<<gb > 0 ? gb : 1, T2P_WARPS * CF_WARP, 0, st>>>(r, a);
-    else t2_pieces_kernel<L, false><<<gb > 0 ? gb : 1, T2P_WARPS * CF_WARP, 0, st>>>(r, a);
+    // records per lane of a chunk: as many as leave every SM its 32 resident warps (longer
+    // chunks lose less in the rounds where node counts change and in the last one: p = 16, q = 2,
+    // 6.4e6 records 0.472 ms at 2, 0.432 at 3, 0.424 at 4)
+    const long long fill = 4LL * T2P_WARPS * nsm * CF_WARP;
+    const int rows = (int)(r.nrec <= fill ? 1 : r.nrec >= T2P_R * fill ? T2P_R : (r.nrec + fill - 1) / fill);
+    const long long per_block = (long long)T2P_WARPS * CF_WARP * rows;
+    const long long need = (r.nrec + per_block - 1) / per_block, cap = 16LL * nsm;
+    const int gb = (int)(need < cap ? need : cap);
+    if (a.h32tab) t2_pieces_kernel<L, true><<<gb, T2P_WARPS * CF_WARP, 0, st>>>(r, a, rows);
+    else t2_pieces_kernel<L, false><<<gb, T2P_WARPS * CF_WARP, 0, st>>>(r, a, rows);
 }
 
 cudaError_t launch_t2(const RecSet& r, const IntegArgs& a, int fp32, int blocks, int nsm, cudaStream_t st)
@@ -417,10 +469,10 @@ cudaError_t launch_t2(const RecSet& r, const IntegArgs& a, int fp32, int blocks,
         return cudaGetLastError();
     }
     const int L = a.t2_group;
-    if (fp32 && L == 2) go_group<2>(r, a, blocks, st);
-    else if (fp32 && L == 4) go_group<4>(r, a, blocks, st);
-    else if (fp32 && L == 8) go_group<8>(r, a, blocks, st);
-    else if (fp32 && L == 16) go_group<16>(r, a, blocks, st);
+    if (fp32 && L == 2) go_group<2>(r, a, nsm, st);
+    else if (fp32 && L == 4) go_group<4>(r, a, nsm, st);
+    else if (fp32 && L == 8) go_group<8>(r, a, nsm, st);
+    else if (fp32 && L == 16) go_group<16>(r, a, nsm, st);
     else if (fp32) {
         t2_records_kernel<float><<<blocks, 256, 0, st>>>(r, a);
     } else {

@@ -15,6 +15,8 @@ mapped variable t in [-1, 1]:
   Phi^-1(p), pm = min(p, 1 - p) in [1e-37, 1/2]:
       x = log2(-log2 pm) in [0, 7],  Phi^-1(pm) = x Q(t), t = affine(x)
       (the factor x makes Phi^-1(1/2) = 0 exactly);  Phi^-1(p) = -x Q for p > 1/2.
+  atan(a), 0 <= a <= 1:  a R(a^2), R fitted on [0, 1] (relative error of atan(a)/a)
+      (cf_atan2_f32 folds the other octants onto it).
   sin(x), |x| <= pi:  r = |x| folded to [0, pi/2] (pi - |x| beyond pi/2),
       sin(r) = r S(r^2) with S fitted on [0, (pi/2)^2] (relative error of sin/r),
       then the sign of x.
@@ -73,6 +75,14 @@ def fit_sin(deg=4):
     return coef, err
 
 
+def fit_atan(deg=8):
+    a = np.linspace(1e-6, 1.0, 400001)
+    m, _ = lawson(a * a, np.arctan(a) / a, deg, 0.0, 1.0)
+    coef = sum(c * Pm.Polynomial([-1.0, 2.0]) ** k for k, c in enumerate(m)).coef
+    err = np.abs(Pm.polyval(a * a, coef) / (np.arctan(a) / a) - 1.0).max()
+    return coef, err
+
+
 if __name__ == "__main__":
     m, A, B, e = fit_ncdf()
     print(f"// Phi: max |error of the log2 exponent| {e:.2e}")
@@ -85,3 +95,6 @@ if __name__ == "__main__":
     coef, e = fit_sin()
     print(f"// sin: max |error| {e:.2e}  (value = r * S(r^2), S in powers of r^2)")
     print("S =", ", ".join(f"{c:.9e}f" for c in coef))
+    coef, e = fit_atan()
+    print(f"// atan: max relative |error| {e:.2e}  (value = a * R(a^2), R in powers of a^2)")
+    print("R =", ", ".join(f"{c:.9e}f" for c in coef))

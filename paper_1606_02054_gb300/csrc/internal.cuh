@@ -158,7 +158,8 @@ struct PlanArgs {
 //   [3] lgamma((v+1)/2) - lgamma(v/2) - log(v pi)/2    (log t_1 density at dof v)
 //   [4] the same at dof v - 1
 //   [5] lgamma(v/2)                                    (chi-square quantile at dof v)
-enum { CST_LGB = 0, CST_LGB1 = 1, CST_C2 = 2, CST_LT1 = 3, CST_LT1M = 4, CST_LGA = 5, CST_STRIDE = 8 };
+//   [6], [7] the exponentials of [3] and [4]
+enum { CST_LGB = 0, CST_LGB1 = 1, CST_C2 = 2, CST_LT1 = 3, CST_LT1M = 4, CST_LGA = 5, CST_ET1 = 6, CST_ET1M = 7, CST_STRIDE = 8 };
 
 struct IntegArgs {
     const double* cst64;   // [tab][CST_STRIDE]
@@ -182,10 +183,12 @@ struct IntegArgs {
     int t2n_lo;
     const float* glx32l;
     const float* glw32l;
-    // FP32 T_2: per tab, log2 T_1(-|z|; dof + 1) on the grid of T1TAB_N points
-    // uniform in v = log2(1 + |z|) over [0, T1TAB_V], with d/dv (float2 each);
-    // NULL: the continued fraction is used instead
-    const float2* t1tab;
+    // FP32 T_1 and T_2: the tables of H32_* below (else null: the continued fraction).  The
+    // inner T_1 of a T_2 record of table index t is in table 4 (t / 3) + t % 3 + 1 (E-step) or t
+    // (h32_case: cfust_tk_eval, one table per case).
+    const float4* h32tab;
+    const float* h32scale;  // per table: cells per unit of sigma
+    int h32_case;
     // FP32 single-pass moments at q <= 4 (else null): per shift m and lattice point i, the
     // baker-transformed coordinates w_d = 1 - |2 frac(i z_d / N + shift_md) - 1|, d = 1..q,
     // in one float4 (computed in FP64 at creation; they are the same for every record)
@@ -221,7 +224,13 @@ constexpr int H1_CELLS = 64, H1_D = 9, H1_NC = H1_D + 1;
 constexpr int H1_SIZE = H1_CELLS * H1_NC;  // doubles per table
 constexpr double H1_DOF_MAX = 250.0;
 
-constexpr int T1TAB_N = 2048;
+// The FP32 tables of the same H: cubic polynomials (one float4) on H32_CELLS equal cells of
+// [0, sigma_max], sigma_max = 1 up to dof 250 and beyond it the sigma where T_1 leaves FP32's
+// range (16 / sqrt(v + 256)), so the cells stay fine enough at any dof: 1.4e-8 relative
+// (against 30-digit values, dof 1.5 to 5000).
+constexpr int H32_CELLS = 256;
+__host__ __device__ __forceinline__ double h32_sigma_max(double v) { return v <= 250.0 ? 1.0 : 16.0 / sqrt(v + 256.0); }
+
 constexpr int T2_NH = 64;
 // FP32 T_2 pieces where 4 <= dof <= 64 and |rho| < 0.9: Gauss-Legendre with 8, 12, 16, 20,
 // 24 or t2n (32) nodes by the piece's length L in units of the integrand's two widths: the
@@ -249,10 +258,10 @@ constexpr float T2_LO_ZW = 0.2f;
 constexpr float T2_LO_DOF_MIN = 4.0f, T2_LO_DOF_MAX = 64.0f, T2_LO_RHO = 0.9f;
 
 // class of an FP32 T_2 piece of length L (either sign) in the region above: 0-4, or 5 for
-// the t2n nodes
-__device__ __forceinline__ int t2_lo_class(float L, float nu, float zs)
+// the t2n nodes; zs2 = zs^2
+__device__ __forceinline__ int t2_lo_class(float L, float nu, float zs2)
 {
-    const float s2 = L * L * fmaf(T2_LO_ZW * zs, zs, nu - 1.0f);
+    const float s2 = L * L * fmaf(T2_LO_ZW, zs2, nu - 1.0f);
     return (s2 <= T2_LO_S2_0 && nu <= T2_LO_DMAX_0)   ? 0
            : (s2 <= T2_LO_S2_1 && nu <= T2_LO_DMAX_1) ? 1
            : s2 <= T2_LO_S2_2                         ? 2
@@ -260,8 +269,6 @@ __device__ __forceinline__ int t2_lo_class(float L, float nu, float zs)
            : s2 <= T2_LO_S2_4                         ? 4
                                                       : T2_LO_NCLS;
 }
-
-constexpr float T1TAB_V = 48.0f;
 
 struct CombineArgs {
     Dims D;
@@ -274,7 +281,8 @@ struct CombineArgs {
     const double* pc;
     const float* pd32;     // mixed form: d, log t_p and c in FP32 (read instead of pd, pc)
     const float* pc32;
-    const float2* t1tab;   // mixed form at q = 2 with fuse_l1: the level-1 T_1 from the tables
+    const float4* h32tab;  // mixed form at q = 2 with fuse_l1: the level-1 T_1 from the FP32 tables of H
+    const float* h32scale;
     int fuse_l1;
     RecSet L0, L1, L2, LM;
     int density_only;

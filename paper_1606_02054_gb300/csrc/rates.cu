@@ -17,7 +17,7 @@
 //     rate an implementation of the same algorithm could reach if it did nothing
 //     else;
 //   - one node of the FP32 T_2 quadrature (two sines, the sin^(nu-1) weight, the
-//     inner T_1 from its table), 1, 2 or 4 independent nodes per thread (the best).
+//     inner T_1 through its table), 1 or 2 packed pairs of nodes per thread (the better).
 // Every kernel runs a full grid (8 blocks of 256 threads per SM) for a fixed
 // number of iterations; rates are operations (or points) per second of
 // CUDA-event time after one warm-up launch, and the SM clock is read with
@@ -164,42 +164,54 @@ __global__ void __launch_bounds__(kThreads) mix_rate_kernel(float* out, int iter
     out[(size_t)blockIdx.x * blockDim.x + threadIdx.x] = s0 + s1;
 }
 
-// One node of the FP32 T_2 quadrature, per node: the two sines of the angle
-// (cf_sin_pi), the weight sin^(nu-1) (lg2, ex2), the inner T_1 from a per-dof table
-// (t1cdf_table: log2(1 + |z|) by lg2, cubic Hermite, ex2) and the weighted sum; two
-// independent nodes per thread, angles advancing by a fixed step, the table L1-resident.
+// Two neighbouring nodes of the FP32 T_2 quadrature in packed FP32, as t2_pieces_kernel
+// computes them: the two sines, the powers (lg2, ex2), the table's cubic and the weighted sum; P
+// pairs per thread, angles advancing by a fixed step, the table L1-resident.
 template <int P>
-__global__ void __launch_bounds__(kThreads) t2node_rate_kernel(float* out, const float2* __restrict__ tab, int iters)
+__global__ void __launch_bounds__(kThreads) t2node_rate_kernel(float* out, const float4* __restrict__ tab, int iters)
 {
     const float t0 = threadIdx.x * (1.0f / 8192.0f);
-    float th[P], acc[P];
+    f32x2 th[P], acc[P];
 #pragma unroll
     for (int p = 0; p < P; ++p) {
-        th[p] = 0.1f + 0.7f * (p & 3) + 0.05f * (p >> 2) + t0;
-        acc[p] = 0.f;
+        th[p] = pk2(0.1f + 0.7f * p + t0, 0.4f + 0.7f * p + t0);
+        acc[p] = 0ull;
     }
-    const float dth = 0.00613f, zs = -2.3f, d0 = 0.4f, num1 = 7.5f, wgt = 0.01f;
+    const float sc = 0.7f, num1 = 7.5f;
     for (int i = 0; i < iters; ++i) {
 #pragma unroll
         for (int p = 0; p < P; ++p) {
-            const float sp = cf_sin_pi(th[p]);
-            const float sd = cf_sin_pi(d0 - th[p]);
-            const float f = ptx_ex2_approx(num1 * ptx_lg2_approx(sp)) * t1cdf_table(zs * sd, tab);
-            acc[p] = fmaf(wgt, f, acc[p]);
-            const float t = th[p] + dth;
-            th[p] = t >= 3.0f ? t - 2.9f : t;
+            float D0, D1, s0, s1, e0, e1, g0, g1, u0, u1;
+            const f32x2 sp = sin2_signed(th[p]);
+            up2(mul2(sp, sp), s0, s1);
+            const f32x2 q = mul2(sin2_signed(add2(th[p], pk2(-0.4f))), pk2(sc));
+            up2(fma2(q, q, pk2(1.0f)), D0, D1);
+            const float r0 = rsqrt_approx(D0), r1 = rsqrt_approx(D1);
+            const f32x2 rr = pk2(r0, r1);
+            up2(mul2(pk2(ptx_lg2_approx(s0), ptx_lg2_approx(s1)), pk2(0.5f * num1)), e0, e1);
+            up2(mul2(pk2(ptx_lg2_approx(D0), ptx_lg2_approx(D1)), pk2(-0.5f * num1)), g0, g1);
+            up2(mul2(q & 0x7fffffff7fffffffull, rr), u0, u1);
+            const f32x2 H = pk2(h32_eval(u0, tab, (float)H32_CELLS), h32_eval(u1, tab, (float)H32_CELLS));
+            const f32x2 T = mul2(mul2(pk2(ptx_ex2_approx(g0), ptx_ex2_approx(g1)), mul2(rr, rr)), H);
+            acc[p] = fma2(mul2(pk2(ptx_ex2_approx(e0), ptx_ex2_approx(e1)), T), pk2(0.01f), acc[p]);
+            const f32x2 t = add2(th[p], pk2(0.00613f));
+            up2(t, u0, u1);
+            th[p] = pk2(u0 >= 3.0f ? u0 - 2.9f : u0, u1 >= 3.0f ? u1 - 2.9f : u1);
         }
     }
     float sum = 0.f;
 #pragma unroll
-    for (int p = 0; p < P; ++p) sum += acc[p];
+    for (int p = 0; p < P; ++p) {
+        float a0, a1;
+        up2(acc[p], a0, a1);
+        sum += a0 + a1;
+    }
     out[(size_t)blockIdx.x * blockDim.x + threadIdx.x] = sum;
 }
 
-__global__ void fill_t1tab_kernel(float2* tab)
+__global__ void fill_h32_kernel(float4* tab)
 {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < T1TAB_N) tab[i] = make_float2(-1.0f - 3.0f * i * (T1TAB_V / (T1TAB_N - 1)), -3.0f);
+    if (threadIdx.x < H32_CELLS) tab[threadIdx.x] = make_float4(0.5f - 0.001f * threadIdx.x, -0.001f, 1e-6f, 1e-9f);
 }
 
 __global__ void clock_kernel(long long* out, long long spin)
@@ -277,13 +289,13 @@ cudaError_t mix_rate(Timer& t, float* out, int blocks, double target, double* ra
 }
 
 template <int P>
-cudaError_t t2node_rate(Timer& t, float* out, const float2* tab, int blocks, double target, double* rate)
+cudaError_t t2node_rate(Timer& t, float* out, const float4* tab, int blocks, double target, double* rate)
 {
     int it = 0;
     double s = 0.0;
     cudaError_t e = calibrate(t, [&](int n) { t2node_rate_kernel<P><<<blocks, kThreads>>>(out, tab, n); }, 64, target, &it, &s);
     if (e == cudaSuccess) {
-        const double r = (double)P * blocks * kThreads * it / s;
+        const double r = 2.0 * P * blocks * kThreads * it / s;
         if (r > *rate) *rate = r;
     }
     return e;
@@ -309,14 +321,15 @@ extern "C" cfust_status cfust_measure_rates(int device, double seconds, cfust_ra
     const size_t nthr = (size_t)blocks * kThreads;
     void* buf = nullptr;
     if ((e = cudaMalloc(&buf, nthr * sizeof(double) + (size_t)nsm * sizeof(long long) +
-                                  T1TAB_N * sizeof(float2))) != cudaSuccess) {
+                                  (H32_CELLS + 1) * sizeof(float4))) != cudaSuccess) {
         cf_set_global_error(std::string("cfust_measure_rates: ") + cudaGetErrorString(e));
         return CFUST_ENOMEM;
     }
     float* f32 = (float*)buf;
     double* f64 = (double*)buf;
     long long* clk = (long long*)((char*)buf + nthr * sizeof(double));
-    float2* t1tab = (float2*)((char*)buf + nthr * sizeof(double) + (size_t)nsm * sizeof(long long));
+    // behind the clock counts, on a 16-byte boundary
+    float4* h32tab = (float4*)((char*)buf + nthr * sizeof(double) + ((size_t)nsm * sizeof(long long) + 15) / 16 * 16);
     Timer t;
     const double tgt = seconds / 13.0;  // 13 measurements share the budget
     int it = 0;
@@ -352,10 +365,9 @@ extern "C" cfust_status cfust_measure_rates(int device, double seconds, cfust_ra
         if ((e = mix_rate<6>(t, f32, blocks, tgt, &out->mix_points[6])) != cudaSuccess) break;
         if ((e = mix_rate<7>(t, f32, blocks, tgt, &out->mix_points[7])) != cudaSuccess) break;
         if ((e = mix_rate<8>(t, f32, blocks, tgt, &out->mix_points[8])) != cudaSuccess) break;
-        fill_t1tab_kernel<<<(T1TAB_N + 255) / 256, 256>>>(t1tab);
-        if ((e = t2node_rate<1>(t, f32, t1tab, blocks, tgt / 3, &out->t2_nodes)) != cudaSuccess) break;
-        if ((e = t2node_rate<2>(t, f32, t1tab, blocks, tgt / 3, &out->t2_nodes)) != cudaSuccess) break;
-        if ((e = t2node_rate<4>(t, f32, t1tab, blocks, tgt / 3, &out->t2_nodes)) != cudaSuccess) break;
+        fill_h32_kernel<<<1, 256>>>(h32tab);
+        if ((e = t2node_rate<1>(t, f32, h32tab, blocks, tgt / 2, &out->t2_nodes)) != cudaSuccess) break;
+        if ((e = t2node_rate<2>(t, f32, h32tab, blocks, tgt / 2, &out->t2_nodes)) != cudaSuccess) break;
     } while (0);
     cudaFree(buf);
     if (e != cudaSuccess) {

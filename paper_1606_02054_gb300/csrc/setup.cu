@@ -247,7 +247,7 @@ __global__ void dof_consts_kernel(Dims D, Layout Ly, const double* __restrict__ 
         const double ltm = lgamma(0.5 * v) - lgamma(0.5 * (v - 1.0)) - 0.5 * log((v - 1.0) * CF_PI);
         const double c[CST_STRIDE] = {t1_lgb(v), t1_lgb(v + 1.0),
                                       cf_t_const(v),
-                                      lt, v > 1.0 ? ltm : 0.0, lgamma(0.5 * v), 0.0, 0.0};
+                                      lt, v > 1.0 ? ltm : 0.0, lgamma(0.5 * v), exp(lt), v > 1.0 ? exp(ltm) : 0.0};
         for (int k = 0; k < CST_STRIDE; ++k) {
             c64[t * CST_STRIDE + k] = c[k];
             c32[t * CST_STRIDE + k] = (float)c[k];
@@ -277,52 +277,6 @@ __global__ void narrow_kernel(const double* __restrict__ src, Dims D, float* __r
         dst[t] = (float)src[t];
 }
 
-// log T_1(-w; nu) for w >= 0 in FP64, without underflow: with x = nu/(nu+w^2),
-// T_1(-w) = I_x(nu/2, 1/2)/2 from the continued fraction in log form; lbeta =
-// lgamma((nu+1)/2) - lgamma(nu/2) - lgamma(1/2), the table's constant.
-static __device__ double log_t1_lower(double w, double nu, double lbeta)
-{
-    if (w == 0.0) return -CF_LN2;
-    const double w2 = w * w, den = nu + w2;
-    const double x = nu / den, y = w2 / den;
-    const double a = 0.5 * nu, b = 0.5;
-    const double lbt = lbeta + a * log(x) + b * log(y);
-    if (x < (a + 1.0) / (a + b + 2.0))
-        return lbt + log(betacf_dev<double>(a, b, x)) - log(a) - CF_LN2;
-    return log1p(-exp(lbt) * betacf_dev<double>(b, a, y) / b) - CF_LN2;
-}
-
-// Tables of log2 T_1(-|z|; dofs[t] + 1) and d/dv on the grid uniform in v = log2(1 + |z|)
-// (see IntegArgs::t1tab).
-// jmask: the tables t with bit (t mod 3) set are built (E-step tables t = 3h + j; the
-// others are left as they are: no record reads them); 7 builds every table.
-// cst: the per-dof constants of dof_consts_kernel (CST_LGB1: lbeta at dofs[t] + 1).
-__global__ void t1_table_kernel(int ndof, const double* __restrict__ dofs, const double* __restrict__ cst,
-                                float2* __restrict__ tab, int jmask)
-{
-    const long long total = (long long)ndof * T1TAB_N;
-    const double hv = (double)T1TAB_V / (T1TAB_N - 1);
-    for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < total;
-         e += (long long)gridDim.x * blockDim.x) {
-        const int t = (int)(e / T1TAB_N), i = (int)(e % T1TAB_N);
-        if (!((jmask >> (t % 3)) & 1)) continue;
-        const double nu = dofs[t] + 1.0;
-        if (isinf(nu)) {  // the normal limit evaluates Phi_2 directly, not through this table
-            tab[e] = make_float2(0.0f, 0.0f);
-            continue;
-        }
-        const double v = i * hv;
-        const double w = expm1(v * CF_LN2);
-        const double lbeta = cst[t * CST_STRIDE + CST_LGB1];
-        const double lT = log_t1_lower(w, nu, lbeta);
-        // d/dv log2 T_1(-w(v)) = -t_nu(w) (1 + w) / T_1(-w)   (dw/dv = (1 + w) ln 2); the
-        // density's constant lgamma((nu+1)/2) - lgamma(nu/2) - log(nu pi)/2 is lbeta - log(nu)/2
-        const double lt = lbeta - 0.5 * log(nu) - 0.5 * (nu + 1.0) * log1p(w * w / nu);
-        const double d = -exp(lt - lT) * (1.0 + w);
-        tab[e] = make_float2((float)(lT / CF_LN2), (float)d);
-    }
-}
-
 // Tables of H for the dofs v = nu_h + p + e (internal.cuh, H1_*): per cell, H at the H1_NC
 // Chebyshev nodes (from the continued fraction: with y = 1 - sigma^2 and a = v/2,
 // H = sigma C betacf(a, 1/2, y) / v where that one converges fast, else
@@ -338,6 +292,15 @@ __constant__ double h1_cheb[H1_NC][H1_NC] = {  // powers of x in T_n(x)
     {-1, 0, 18, 0, -48, 0, 32, 0, 0, 0},  {0, -7, 0, 56, 0, -112, 0, 64, 0, 0},
     {1, 0, -32, 0, 160, 0, -256, 0, 128, 0}, {0, 9, 0, -120, 0, 432, 0, -576, 0, 256}};
 
+// H(sigma) at dof v, C = cf_t_const(v)
+static __device__ double h1_value(double sg, double v, double C)
+{
+    const double a = 0.5 * v, y = (1.0 - sg) * (1.0 + sg);
+    const bool direct = y < (a + 1.0) / (a + 2.5);
+    const double cf = betacf_dev<double>(direct ? a : 0.5, direct ? 0.5 : a, direct ? y : sg * sg);
+    return direct ? sg * C * cf / v : 0.5 * exp(-a * log1p(-sg * sg)) - sg * C * cf;
+}
+
 __global__ void __launch_bounds__(H1_TC * H1_NC) h1_table_kernel(const double* __restrict__ dofs,
                                                                  double* __restrict__ tab, int emask)
 {
@@ -350,12 +313,7 @@ __global__ void __launch_bounds__(H1_TC * H1_NC) h1_table_kernel(const double* _
     const int cell = blockIdx.x * H1_TC + lc;
     if (threadIdx.x < 4 * H1_NC) cosv[threadIdx.x] = cospi(threadIdx.x / (2.0 * H1_NC));
     __syncthreads();
-    const double C = cf_t_const(v), a = 0.5 * v;
-    const double sg = (cell + 0.5 + 0.5 * cosv[2 * j + 1]) * (1.0 / H1_CELLS);
-    const double y = (1.0 - sg) * (1.0 + sg);
-    const bool direct = y < (a + 1.0) / (a + 2.5);
-    const double cf = betacf_dev<double>(direct ? a : 0.5, direct ? 0.5 : a, direct ? y : sg * sg);
-    f[lc][j] = direct ? sg * C * cf / v : 0.5 * exp(-a * log1p(-sg * sg)) - sg * C * cf;
+    f[lc][j] = h1_value((cell + 0.5 + 0.5 * cosv[2 * j + 1]) * (1.0 / H1_CELLS), v, cf_t_const(v));
     __syncthreads();
     const double f0 = f[lc][H1_NC / 2];
     double s = 0.0;
@@ -366,4 +324,35 @@ __global__ void __launch_bounds__(H1_TC * H1_NC) h1_table_kernel(const double* _
     for (int n = H1_NC - 1; n >= j; --n) s += cn[lc][n] * h1_cheb[n][j];
     s *= (double)(1 << j);  // x = 2 t
     tab[(size_t)blockIdx.y * H1_SIZE + cell * H1_NC + j] = j ? s : s + f0;
+}
+
+// The FP32 tables (internal.cuh, H32_*): cubics through H at the 4 Chebyshev nodes of each cell.
+// Blocks of 32 cells (blockIdx.x), a thread per node.  Table blockIdx.y: 4h + e at dof
+// nu_h + p + e where emask has bit e (emask > 0), else case blockIdx.y at dofs[blockIdx.y] + 1.
+__global__ void __launch_bounds__(128) h32_table_kernel(const double* __restrict__ dofs, float4* __restrict__ tab,
+                                                        float* __restrict__ scale, int emask)
+{
+    __shared__ double f[32][4];
+    const int e = blockIdx.y & 3;
+    if (emask && !((emask >> e) & 1)) return;
+    const double v = emask ? dofs[3 * (blockIdx.y >> 2)] + e : dofs[blockIdx.y] + 1.0;
+    if (!(v < INFINITY)) return;  // the normal limit reads no table
+    const int lc = threadIdx.x >> 2, j = threadIdx.x & 3;
+    const int cell = blockIdx.x * 32 + lc;
+    const double h = h32_sigma_max(v) / H32_CELLS;
+    const double x4[2] = {0.9238795325112867, 0.3826834323650898};  // cos(pi/8), cos(3 pi/8)
+    const double x = j == 0 ? x4[0] : j == 1 ? x4[1] : j == 2 ? -x4[1] : -x4[0];
+    f[lc][j] = h1_value((cell + 0.5 + 0.5 * x) * h, v, cf_t_const(v));
+    __syncthreads();
+    if (threadIdx.x < 32) {
+        const double* g = f[threadIdx.x];
+        // even and odd parts in x = 2 t at x4[0], x4[1]: a + b x^2 and x (c + d x^2)
+        const double e0 = 0.5 * (g[0] + g[3]), e1 = 0.5 * (g[1] + g[2]);
+        const double o0 = 0.5 * (g[0] - g[3]) / x4[0], o1 = 0.5 * (g[1] - g[2]) / x4[1];
+        const double q0 = x4[0] * x4[0], q1 = x4[1] * x4[1];
+        const double b = (e0 - e1) / (q0 - q1), d = (o0 - o1) / (q0 - q1);
+        tab[(size_t)blockIdx.y * H32_CELLS + blockIdx.x * 32 + threadIdx.x] =
+            make_float4((float)(e1 - b * q1), (float)(2.0 * (o1 - d * q1)), (float)(4.0 * b), (float)(8.0 * d));
+    }
+    if (blockIdx.x == 0 && threadIdx.x == 0) scale[blockIdx.y] = (float)(1.0 / h);
 }
