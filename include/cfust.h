@@ -386,8 +386,8 @@ cfust_status cfust_tk_eval(cfust_ctx* ctx, int k, int count, const double* b, co
  * address in the current context (the address belongs to the context, so a
  * context created after cudaDeviceReset gets its own); the first call in a
  * context also loads the library's device code there, so make the first
- * call on each device before any stream capture.  The block size is chosen
- * without raising the default shared-memory limit, so the statistics equal
+ * call on each device before any stream capture.  The block size is
+ * smaller than that of cfust_estep for some sizes, so the statistics equal
  * those of cfust_estep to rounding, not bit for bit.  All calls share the scratch and it
  * keeps the last call's contents: calls that overlap on the GPU (other
  * streams, other host threads) race and must be serialised by the caller.

@@ -231,14 +231,15 @@ static cfust_status check_flags(cfust_ctx* c, int f, const char* where)
 // Observations per block of the statistics reduction: rows of 4 + p + q + q^2 values
 // (FP32 in the mixed form) plus g posterior weights staged in at most ~64 KB of
 // shared memory, chunk <= 256.  Depends on the sizes and the precision only, not on n.
-// values per staged row of the statistics kernel (FP32 rows also hold tau u r: p more, and
-// an odd length, so that the threads of a warp staging consecutive rows write to distinct
-// shared-memory banks)
-static int reduce_row(int p, int q, bool mixed) { return mixed ? (4 + 2 * p + q + q * q) | 1 : 4 + p + q + q * q; }
+// values per staged row of the statistics kernel (an odd length, so that the threads of a warp
+// staging consecutive rows write to distinct shared-memory banks)
+static int reduce_row(int p, int q) { return (4 + 2 * p + q + q * q) | 1; }
 
 static int reduce_chunk(int p, int q, int g, bool mixed)
 {
-    const int row = reduce_row(p, q, mixed);
+    // the FP64 rows count without tau u r here: the chunk, and with it the rows of a segment, is
+    // that of rows of 4 + p + q + q^2 values (the block then takes at most 112 KB)
+    const int row = mixed ? reduce_row(p, q) : 4 + p + q + q * q;
     const size_t rowbytes = mixed ? sizeof(float) : sizeof(double);
     int chunk = 256;
     while (chunk > 32 && (size_t)chunk * ((row + g) * rowbytes + sizeof(double)) + CF_MAXG * sizeof(double) > 64 * 1024)
@@ -321,6 +322,9 @@ extern "C" const char* cfust_last_error(const cfust_ctx* c)
 
 extern "C" int64_t cfust_launch_count(const cfust_ctx* c) { return c ? c->launches : 0; }
 
+static int fuses_l1(const cfust_ctx* c);
+static cudaError_t fill_level1(cfust_ctx* c);
+
 extern "C" cfust_status cfust_debug_read(cfust_ctx* c, int what, void* dst, int64_t bytes,
                                          int64_t* written)
 {
@@ -346,6 +350,7 @@ extern "C" cfust_status cfust_debug_read(cfust_ctx* c, int what, void* dst, int6
     }
     const size_t nb = std::min(avail, (size_t)bytes);
     CU(cudaSetDevice(c->opts.device));
+    if ((what == 4 || what == 7) && !c->mixed && fuses_l1(c) && c->have_data && c->have_params) CU(fill_level1(c));
     if (nb) CU(cudaMemcpyAsync(dst, src, nb, cudaMemcpyDeviceToHost, c->st));
     CU(cudaStreamSynchronize(c->st));
     if (written) *written = (int64_t)nb;
@@ -371,6 +376,21 @@ extern "C" cfust_status cfust_profile_work(cfust_ctx* c, double* units)
     if (!c->opts.profile) return fail(c, CFUST_ESTATE, "cfust_profile_work: context created without opts.profile");
     for (int k = 0; k < CFUST_NPROF; ++k) units[k] = c->prof_units[k];
     return CFUST_OK;
+}
+
+static IntegArgs integ_args(const cfust_ctx* c);
+
+// The level-1 records of a context whose E-step does not write them (FP64 and plain FP32 forms at
+// q = 2), from the last E-step's factors: for the diagnostic read-back.
+static cudaError_t fill_level1(cfust_ctx* c)
+{
+    PlanArgs pa{};
+    pa.D = c->D; pa.Ly = c->Ly; pa.y = c->y; pa.F = c->F;
+    pa.L0 = c->rec[0]; pa.L1 = c->rec[1]; pa.L2 = c->rec[2]; pa.LM = c->rec[3];
+    pa.only_l1 = 1;
+    cudaError_t e = launch_plan(pa, c->st, &c->launches);
+    if (e != cudaSuccess) return e;
+    return launch_integrals(c->rec[1], integ_args(c), c->opts.precision != CFUST_PREC_FP64, c->nsm, c->st, &c->launches);
 }
 
 static void free_all(cfust_ctx* c)
@@ -493,7 +513,7 @@ extern "C" cfust_status cfust_create(cfust_ctx** out, int p, int q, int g, int64
     const int S = stats_per_comp(p, q);
     // reduction staging: rows of 4 + p + q + q^2 doubles, chunk <= 256 observations,
     // at most ~64 KB of shared memory
-    c->row = reduce_row(p, q, c->mixed);
+    c->row = reduce_row(p, q);
     const int chunk = reduce_chunk(p, q, g, c->mixed);
     c->chunk = chunk;
     c->nblocks_red = (int)((n + chunk - 1) / chunk);
@@ -669,7 +689,7 @@ extern "C" cfust_status cfust_create(cfust_ctx** out, int p, int q, int g, int64
         delete c;
         return s;
     }
-    reduce_set_smem_limits(96 * 1024);
+    reduce_set_smem_limits(128 * 1024);
     if (o.profile &&
         (cudaMalloc((void**)&c->work_dev, sizeof(unsigned long long) * CFUST_NPROF) != cudaSuccess ||
          cudaMemset(c->work_dev, 0, sizeof(unsigned long long) * CFUST_NPROF) != cudaSuccess)) {
@@ -867,6 +887,14 @@ static IntegArgs integ_args(const cfust_ctx* c)
     return ia;
 }
 
+// q = 2, recursion moments: combine evaluates the level-1 T_1s from the tables of H (the mixed form
+// also in the normal limit, where they are Phi)
+static int fuses_l1(const cfust_ctx* c)
+{
+    return c->q == 2 && !c->single_pass && (c->h32tab || c->h1tab) &&
+           (c->mixed || c->opts.model == CFUST_MODEL_CFUST);
+}
+
 // S2-S7: plan, integrals of each level, combine, FP64 fix-up of far-tail pairs.
 static cfust_status launch_pairs(cfust_ctx* c, int density_only)
 {
@@ -879,8 +907,8 @@ static cfust_status launch_pairs(cfust_ctx* c, int density_only)
     pa.single_pass = sp;
     pa.pd = c->pd; pa.pc = c->pc;
     pa.pd32 = c->mixed ? c->pd32 : nullptr; pa.pc32 = c->mixed ? c->pc32 : nullptr;
-    // mixed form at q = 2: the level-1 T_1s are table lookups done by combine, not records
-    const int fuse_l1 = c->mixed && c->q == 2 && !c->single_pass && c->h32tab != nullptr;
+    // q = 2: the level-1 T_1s are table lookups done by combine, not records
+    const int fuse_l1 = fuses_l1(c);
     pa.fuse_l1 = fuse_l1;
     pa.blocks = 16 * c->nsm;
     pa.L0 = c->rec[0]; pa.L1 = c->rec[1]; pa.L2 = c->rec[2]; pa.LM = c->rec[3];
@@ -970,7 +998,7 @@ static cfust_status launch_pairs(cfust_ctx* c, int density_only)
     CombineArgs ca;
     ca.D = c->D; ca.Ly = c->Ly; ca.cst64 = c->cst64; ca.cst32 = c->cst32; ca.F = c->F; ca.pd = c->pd; ca.pc = c->pc;
     ca.pd32 = c->mixed ? c->pd32 : nullptr; ca.pc32 = c->mixed ? c->pc32 : nullptr;
-    ca.h32tab = c->h32tab; ca.h32scale = c->h32scale; ca.fuse_l1 = fuse_l1;
+    ca.h32tab = c->h32tab; ca.h32scale = c->h32scale; ca.h1tab = c->h1tab; ca.fuse_l1 = fuse_l1;
     ca.F32 = c->mixed ? c->F32 : nullptr;
     ca.L0 = pa.L0; ca.L1 = c->rec[1]; ca.L2 = c->rec[2]; ca.LM = c->rec[3];
     ca.density_only = density_only; ca.single_pass = sp; ca.fp32 = fp32;
@@ -1027,7 +1055,7 @@ static cfust_status enqueue_estep_segments(cfust_ctx* c, double* seg, long long 
     r.y32 = c->y32;
     r.small_only = c->tc_stats ? 1 : 0;
     const size_t smem = (c->mixed ? sizeof(float) : sizeof(double)) * ((size_t)c->chunk * c->row + (size_t)c->g * c->chunk) +
-                        sizeof(double) * ((size_t)c->chunk + CF_MAXG);
+                        sizeof(double) * ((size_t)c->chunk + CF_MAXG + (c->mixed ? 0 : 256));
     prof_begin(c, CFUST_PROF_REDUCE);
     if (c->mixed) launch_reduce_f32(r, c->nblocks_red, smem, c->st);
     else estep_reduce_kernel<<<c->nblocks_red, 256, smem, c->st>>>(r);

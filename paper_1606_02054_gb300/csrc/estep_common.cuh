@@ -334,15 +334,21 @@ __device__ inline void pair_assemble_sp(const double* F, const Layout& Ly, int p
 }
 
 // q = 2: the assembly with the level-1 T_1 inside, in T = float (the mixed form) or double.
-// With w0 = c_r^2 / (nu1 S_rr) and w = the T_1's argument squared over its dof nu2 = nu1 + 1,
-// the t densities and that T_1 are powers of 1 + w0 and 1 + w,
-//   t_1(c_r; S_rr, nu1)              = K (S_rr)^(-1/2) (1 + w0)^(-(nu1+1)/2)
-//   t_1(c'; V, nu2 - 2)              = K' V^(-1/2) E,   E = (1 + w)^(-(nu2-1)/2)
-//   T_1(-|b|; nu2)                   = E (1 + w)^(-1/2) H(sigma), sigma^2 = w / (1 + w)
-// so a coordinate takes two log1p and two exp, where the general routine takes four logarithms,
-// two exponentials and the T_1.  H from the component's table at dof nu2 (FP64: scale unused).
-// cst: the per-dof constants of dof nu+p.
+// With S = ((nu+d)/nu1) Lambda and s_r the Schur complement of Lambda at r,
+//   w0 = c_r^2 / (nu1 S_rr) = (c_r dq_r)^2 / (nu+d)
+//   w  = c'^2 / (s_r (nu+d) (1 + w0)),   c' = c_b - m_r c_r,
+// the t densities and the level-1 T_1 (dof nu2 = nu1 + 1) are powers of 1 + w0 and 1 + w:
+//   t_1(c_r; S_rr, nu1)  = e^lt1 (S_rr)^(-1/2) (1 + w0)^(-(nu1+1)/2)
+//   t_1(c'; V, nu2 - 2)  = e^lt1m V^(-1/2) E,   E = (1 + w)^(-nu1/2),  V = (1 + w0)(nu+d) s_r / (nu1-1)
+//   T_1(-|b|; nu2)       = E (1 + w)^(-1/2) H(sigma),   sigma^2 = w / (1 + w)
+// so a coordinate takes two log1p, two exp and two rsqrt, no division and no T_1 record, where the
+// general routine takes four logarithms, two exponentials, five divisions and the T_1.  H from
+// the component's table at dof nu2.  cst: the per-dof constants of dof nu+p.
 __device__ __forceinline__ float h_lookup(float sigma, const float4* tab, float scale) { return h32_eval(sigma, tab, scale); }
+__device__ __forceinline__ double h_lookup(double sigma, const float4* tab, float scale)
+{
+    return (double)h32_eval((float)sigma, tab, scale);  // the FP32 integrals of the plain FP32 form
+}
 __device__ __forceinline__ double h_lookup(double sigma, const double* tab, float) { return h1_eval(sigma, tab); }
 __device__ __forceinline__ float m_log1p(float x) { return log1pf(x); }
 __device__ __forceinline__ double m_log1p(double x) { return log1p(x); }
@@ -356,33 +362,29 @@ __device__ __forceinline__ void pair_assemble_q2(const T* F, const Layout& Ly, i
     if (!(alpha_s > T(0))) return pair_null(2, 0, o);
     // eq (4): log t_p + log alpha_s in T, q log 2 added in FP64
     o.logf = 2 * 0.6931471805599453 + (double)(logtp + m_log(alpha_s));
-    const T nu = F[Ly.scal + SC_NU], nu1 = nu + T(p), nu2 = nu1 + T(1);
-    const T k0 = (nu + d) / nu1, ia = T(1) / alpha_s;
-    const T u = alpha * ia / k0;  // eq (13)
+    const T nu = F[Ly.scal + SC_NU], nu1 = nu + T(p), nud = nu + d;
+    const T rs = m_rsqrt(nud), ia = T(1) / alpha_s;
+    const T ik0 = nu1 * (rs * rs);  // (nu+p)/(nu+d)
+    const T u = ik0 * alpha * ia;   // eq (13)
     o.u = u;
-    o.elogu = u - m_log(T(0.5) * (nu + d)) - T(1) / k0 + F[Ly.scal + SC_PSI];  // eq (15)
+    o.elogu = u - m_log(T(0.5) * nud) - ik0 + F[Ly.scal + SC_PSI];  // eq (15)
     T xi[2], H[4];
 #pragma unroll
     for (int r = 0; r < 2; ++r) {
         const int b = 1 - r;
-        const T* blk = F + Ly.l1 + r * Ly.l1s;  // m_r, the Schur complement
-        const T mv = blk[0], sch = blk[1];
-        const T Srr = k0 * F[Ly.Lam + 3 * r];
-        const T w0 = c[r] * c[r] / (nu1 * Srr);
-        const T E0 = cst[CST_ET1] * m_rsqrt(Srr) * m_exp(T(-0.5) * (nu1 + T(1)) * m_log1p(w0));
-        const T cp = c[b] - mv * c[r];
-        const T sc1 = (nu1 / nu2) * (T(1) + w0) * k0, V0 = sc1 * sch;
-        const T w = cp * cp / (nu2 * V0);
-        const T E = m_exp(T(-0.5) * (nu2 - T(1)) * m_log1p(w));
+        const T* blk = F + Ly.l1 + r * Ly.l1s;  // m_r, the Schur complement, its 1/sqrt
+        const T mv = blk[0], sch = blk[1], dsc = blk[2], dq = F[Ly.dq + r];
+        const T b0 = c[r] * dq * rs, w0 = b0 * b0, r0 = m_rsqrt(T(1) + w0);
+        const T E0 = cst[CST_ET1] * (dq * rs) * m_exp(T(-0.5) * (nu1 + T(1)) * m_log1p(w0));
+        const T sd = dsc * rs * r0, b1 = (c[b] - mv * c[r]) * sd, w = b1 * b1;
+        const T E = m_exp(T(-0.5) * nu1 * m_log1p(w));
         const T rq = m_rsqrt(T(1) + w);
-        const T Tm = E * rq * h_lookup(m_sqrt(w) * rq, tab, scale);
-        const T t1 = cp > T(0) ? T(1) - Tm : Tm;
-        // V = nu2/(nu2-2) V0
-        const T kq = nu2 / (nu2 - T(2));
-        const T xip = cst[CST_ET1M] * m_rsqrt(kq * V0) * E;
+        const T Tm = E * rq * h_lookup(m_abs(b1) * rq, tab, scale);
+        const T t1 = b1 > T(0) ? T(1) - Tm : Tm;
         xi[r] = E0 * t1;
         H[3 * r] = c[r] * xi[r];
-        H[2 * r + b] = E0 * (mv * c[r] * t1 - kq * V0 * xip);
+        // V t_1(c'; V, nu2 - 2), V^(1/2) = (1 + w0) (nu+d) s_r sd / sqrt(nu1 - 1)
+        H[2 * r + b] = E0 * (mv * c[r] * t1 - cst[CST_ET1M] * E * ((T(1) + w0) * nud * sch * sd));
     }
     const T* Lam = F + Ly.Lam;
     T Lx[2];

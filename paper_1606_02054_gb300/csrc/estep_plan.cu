@@ -137,9 +137,12 @@ static void launch_plan_f32(const PlanArgs& a, int gb, cudaStream_t st)
     else plan_kernel_f32<P, 0><<<gb, 128, sh, st>>>(a);
 }
 
+// Q = 2: q = 2 without level-1 records (fuse_l1), the two level-0 scalings from one division and
+// one square root; 0: any q
+template <int Q>
 __global__ void __launch_bounds__(128) plan_kernel(PlanArgs a)
 {
-    const int p = a.D.p, q = a.D.q;
+    const int p = a.D.p, q = Q > 0 ? Q : a.D.q;
     const long long np = a.D.n * a.D.g;
     const int m0 = (a.density_only || a.single_pass) ? 1 : 2;
     for (long long pid = blockIdx.x * (long long)blockDim.x + threadIdx.x; pid < np;
@@ -151,20 +154,31 @@ __global__ void __launch_bounds__(128) plan_kernel(PlanArgs a)
         const double nu1 = F[a.Ly.scal + SC_NU] + p;
         double c[CF_MAXQ], d, logtp;
         pair_whiten(F, a.Ly, p, q, a.y + (size_t)j * p, &d, c, &logtp);
-        a.pd[2 * pid] = d;
-        a.pd[2 * pid + 1] = logtp;
-        for (int k = 0; k < q; ++k) a.pc[pid * q + k] = c[k];
+        if (Q == 2 || !a.only_l1) {
+            a.pd[2 * pid] = d;
+            a.pd[2 * pid + 1] = logtp;
+            for (int k = 0; k < q; ++k) a.pc[pid * q + k] = c[k];
+        }
         double bt[CF_MAXQ];
-        for (int w = 0; w < m0; ++w) {
+        double f = 0.0;
+        if (Q == 2) f = sqrt(nu1 / (F[a.Ly.scal + SC_NU] + d));
+        for (int w = 0; w < (Q != 2 && a.only_l1 ? 0 : m0); ++w) {
             const long long rec = pid * m0 + w;
-            limits_l0(F, a.Ly, p, q, c, d, w, bt);
+            if (Q == 2) {
+                // sqrt((nu+p+2)/(nu+d)) from the component's sqrt((nu+p+2)/(nu+p))
+                if (w) f *= F[a.Ly.scal + SC_RL0];
+                bt[0] = c[0] * f * F[a.Ly.dq];
+                bt[1] = c[1] * f * F[a.Ly.dq + 1];
+            } else {
+                limits_l0(F, a.Ly, p, q, c, d, w, bt);
+            }
             for (int k = 0; k < q; ++k) a.L0.bt[rec * q + k] = bt[k];
             a.L0.fac[rec] = foff + fac_l0(a.Ly);
             a.L0.tab[rec] = 3 * h + 2 * w;
             a.L0.dof[rec] = nu1 + 2.0 * w;
             if (q == 2) put_t2f(a.L0, rec, bt, F, fac_l0(a.Ly), nu1 + 2.0 * w);
         }
-        if (a.density_only) continue;
+        if (a.density_only || Q == 2) continue;
         if (a.single_pass) {
             // alpha and the moments at dof nu+p+2 (eqs 13, 16, 17) from the pass of
             // alpha_s: its limits and chi table, points weighted by W/(nu+p)
@@ -267,6 +281,47 @@ __global__ void __launch_bounds__(128) combine_mixed_kernel(CombineArgs a)
         if (a.se) a.se[pid] = se;
         if (!(of.logf < INFINITY)) atomicOr(a.flags, KF_NAN);  // NaN or +inf; -inf is a null pair
         if (!a.density_only) store_pr32(a.pr32 + pid * pr32_width(q), q, of);
+    }
+}
+
+// FP64 and plain FP32 forms at q = 2 with the level-1 T_1 inside the assembly (finite nu): H from
+// the FP64 tables, or in the plain FP32 form from the FP32 ones.  Bound by the FP64 pipe; p = 16,
+// g = 8, n = 200,000 on a GB300: 2.16 -> 1.38 ms (541 FP64 slots
+// a pair), with the level-1 records' plan (1.26 -> 0.91 ms) and launch gone.
+template <bool F32>
+__global__ void __launch_bounds__(128) combine_q2_kernel(CombineArgs a)
+{
+    const long long np = a.D.n * a.D.g;
+    for (long long pid = blockIdx.x * (long long)blockDim.x + threadIdx.x; pid < np;
+         pid += (long long)gridDim.x * blockDim.x) {
+        const int h = (int)(pid / a.D.n);
+        const double* F = a.F + (size_t)h * a.Ly.stride;
+        const double2 dl = reinterpret_cast<const double2*>(a.pd)[pid];
+        const double2 c2 = reinterpret_cast<const double2*>(a.pc)[pid];
+        const double2 al = reinterpret_cast<const double2*>(a.L0.res)[pid];
+        const double c[2] = {c2.x, c2.y};
+        if (F32 && !(al.x >= 1e-35)) {
+            // outside the FP32 range of the lattice products: redo in FP64
+            const int slot = atomicAdd(a.fix_count, 1);
+            a.fix_list[slot] = (int)pid;
+            continue;
+        }
+        PairOut o;
+        const double* cst = a.cst64 + (size_t)(3 * h) * CST_STRIDE;
+        if (F32)
+            pair_assemble_q2<double>(F, a.Ly, a.D.p, c, dl.x, dl.y, al.x, al.y, cst,
+                                     a.h32tab + (size_t)(4 * h + 1) * H32_CELLS, a.h32scale[4 * h + 1], o);
+        else
+            pair_assemble_q2<double>(F, a.Ly, a.D.p, c, dl.x, dl.y, al.x, al.y, cst,
+                                     a.h1tab + (size_t)(4 * h + 1) * H1_SIZE, 0.0f, o);
+        a.logf[pid] = o.logf;
+        if (a.se) a.se[pid] = 0.0;  // quadrature
+        if (!(o.logf < INFINITY)) atomicOr(a.flags, KF_NAN);  // NaN or +inf; -inf is a null pair
+        a.u[pid] = o.u;
+        a.elogu[pid] = o.elogu;
+        reinterpret_cast<double2*>(a.eu)[pid] = make_double2(o.eu[0], o.eu[1]);
+        reinterpret_cast<double2*>(a.euu)[2 * pid] = make_double2(o.euu[0], o.euu[1]);
+        reinterpret_cast<double2*>(a.euu)[2 * pid + 1] = make_double2(o.euu[2], o.euu[3]);
     }
 }
 
@@ -378,7 +433,8 @@ cudaError_t launch_plan(const PlanArgs& a, cudaStream_t st, long long* launches)
         default: launch_plan_f32<0>(a, gf, st); break;
         }
     }
-    else plan_kernel<<<gb, 128, 0, st>>>(a);
+    else if (a.fuse_l1) plan_kernel<2><<<gb, 128, 0, st>>>(a);
+    else plan_kernel<0><<<gb, 128, 0, st>>>(a);
     ++*launches;
     return cudaGetLastError();
 }
@@ -392,6 +448,9 @@ cudaError_t launch_combine(const CombineArgs& a, cudaStream_t st, long long* lau
         else combine_mixed_kernel<0><<<gb, 128, 0, st>>>(a);
     } else if (a.mixed) {
         combine_kernel<true><<<gb, 128, 0, st>>>(a);
+    } else if (a.fuse_l1 && !a.density_only) {
+        if (a.fp32) combine_q2_kernel<true><<<gb, 128, 0, st>>>(a);
+        else combine_q2_kernel<false><<<gb, 128, 0, st>>>(a);
     } else {
         combine_kernel<false><<<gb, 128, 0, st>>>(a);
     }

@@ -37,7 +37,7 @@ struct Layout {
     int stride; // doubles per component
 };
 
-enum { SC_NU = 0, SC_LOGTP = 1, SC_PSI = 2, SC_COUNT = 4 };
+enum { SC_NU = 0, SC_LOGTP = 1, SC_PSI = 2, SC_RL0 = 3 /* sqrt((nu+p+2)/(nu+p)) */, SC_COUNT = 4 };
 
 __host__ __device__ inline Layout make_layout(int p, int q)
 {
@@ -144,7 +144,8 @@ struct PlanArgs {
     double* pc;        // per pair: c (q)
     float* pd32;       // mixed form: the same in FP32 (written instead of pd, pc)
     float* pc32;
-    int fuse_l1;       // mixed form at q = 2: no level-1 records (combine evaluates the T_1s)
+    int fuse_l1;       // q = 2, recursion: no level-1 records (combine evaluates the T_1s)
+    int only_l1 = 0;   // FP64 and plain FP32 forms: write the level-1 records only (diagnostic read-back)
     int blocks = 0;    // mixed form: blocks of the plan (resident on the device; each takes
                        // tiles of 128 observations of one component), 0: one per tile
     RecSet L0, L1, L2, LM;
@@ -158,7 +159,7 @@ struct PlanArgs {
 //   [3] lgamma((v+1)/2) - lgamma(v/2) - log(v pi)/2    (log t_1 density at dof v)
 //   [4] the same at dof v - 1
 //   [5] lgamma(v/2)                                    (chi-square quantile at dof v)
-//   [6], [7] the exponentials of [3] and [4]
+//   [6] exp([3]) sqrt(v), [7] exp([4]) / sqrt(v - 1)   (the t densities of pair_assemble_q2)
 enum { CST_LGB = 0, CST_LGB1 = 1, CST_C2 = 2, CST_LT1 = 3, CST_LT1M = 4, CST_LGA = 5, CST_ET1 = 6, CST_ET1M = 7, CST_STRIDE = 8 };
 
 struct IntegArgs {
@@ -281,8 +282,9 @@ struct CombineArgs {
     const double* pc;
     const float* pd32;     // mixed form: d, log t_p and c in FP32 (read instead of pd, pc)
     const float* pc32;
-    const float4* h32tab;  // mixed form at q = 2 with fuse_l1: the level-1 T_1 from the FP32 tables of H
+    const float4* h32tab;  // q = 2 with fuse_l1: the level-1 T_1 from the tables of H
     const float* h32scale;
+    const double* h1tab;
     int fuse_l1;
     RecSet L0, L1, L2, LM;
     int density_only;

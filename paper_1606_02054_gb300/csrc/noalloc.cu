@@ -45,13 +45,12 @@ extern "C" cfust_status cfust_reduce_stats_noalloc(int p, int q, int g, int64_t 
         return nerr(CFUST_EINVAL, "cfust_reduce_stats_noalloc: sizes out of range");
     if (!y || !pi || !mu || !logf || !u || !elogu || !eu || !euu || !stats)
         return nerr(CFUST_EINVAL, "cfust_reduce_stats_noalloc: NULL device pointer");
-    // rows of 4 + p + q + q^2 doubles, chunk <= 256 observations, at most 48 KB of
-    // shared memory per block (the default limit: no attribute is set here).  The
-    // allocating path raises its limit to 64 KB and may stage more observations per
-    // block, so the two agree to rounding, not bit for bit.
-    const int row = 4 + p + q + q * q;
+    // chunk <= 256 observations: those whose values (4 + p + q + q^2 doubles a row without the
+    // weighted vectors, and the weights) take at most 48 KB.  The allocating path lets them take
+    // 64 KB and may stage more observations per block, so the two agree to rounding, not bit for bit.
     int chunk = 256;
-    while (chunk > 32 && ((size_t)chunk * (row + g + 1) + CF_MAXG) * sizeof(double) > 48 * 1024) chunk -= 32;
+    while (chunk > 32 && ((size_t)chunk * (4 + p + q + q * q + g + 1) + CF_MAXG) * sizeof(double) > 48 * 1024) chunk -= 32;
+    const int row = (4 + 2 * p + q + q * q) | 1;  // as staged (reduce.cu)
     const int nblocks = (int)((n + chunk - 1) / chunk);
     const int width = g * stats_per_comp(p, q) + 1;
     if ((long long)nblocks * width > CF_NOALLOC_PARTIAL_DOUBLES)
@@ -86,7 +85,10 @@ extern "C" cfust_status cfust_reduce_stats_noalloc(int p, int q, int g, int64_t 
     r.y32 = nullptr;
     r.pr32 = nullptr;
     r.small_only = 0;
-    const size_t smem = sizeof(double) * ((size_t)chunk * row + (size_t)g * chunk + chunk + CF_MAXG);
+    const size_t smem = sizeof(double) * ((size_t)chunk * row + (size_t)g * chunk + chunk + CF_MAXG + 256);
+    // the staged rows take up to 84 KB (no allocation: a limit of the kernel in this context)
+    if ((e = cudaFuncSetAttribute(estep_reduce_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 128 * 1024)) != cudaSuccess)
+        return nerr(CFUST_ECUDA, std::string("cfust_reduce_stats_noalloc: ") + cudaGetErrorString(e));
     estep_reduce_kernel<<<nblocks, 256, smem, st>>>(r);
     if ((e = cudaGetLastError()) != cudaSuccess)
         return nerr(CFUST_ECUDA, std::string("cfust_reduce_stats_noalloc: ") + cudaGetErrorString(e));

@@ -14,10 +14,10 @@
 
 
 
-// Staged FP64 row of one observation for component h:
-//   [0] tau, [1] tau*u, [2] elogu - u, [3] 1, [4..4+p) r, then eu (q), euu (q*q).
-// Each statistic is the sum over the chunk of row[ia]*row[ib]*row[ic] (the FP32 rows:
-// stat_operands_w below).  The
+// Staged row of one observation for component h, with the weighted vectors beside r:
+//   [0] tau, [1] tau u, [2] tau (elogu - u), [3] 1, then r (p), tau u r (p), tau eu (q),
+//   tau euu (q*q),
+// so that every statistic is the sum over the chunk of row[ia] * row[ib].  The
 // symmetric See and Srr are computed for their lower triangles only
 // (stats_reduced(p, q) statistics) and written to both positions o1, o2 of the
 // full layout (o2 = -1 when there is one).
@@ -26,42 +26,6 @@ __device__ inline int stats_reduced(int p, int q)
     return 3 + p + q + p * q + q * (q + 1) / 2 + p * (p + 1) / 2;
 }
 
-__device__ inline void stat_operands(int e, int p, int q, int& ia, int& ib, int& ic, int& o1, int& o2)
-{
-    const int R0 = 4, E0 = 4 + p, EE0 = 4 + p + q;
-    const int fSee = 3 + p + q + p * q, fSrr = fSee + q * q;
-    o2 = -1;
-    if (e == 0) { ia = 0; ib = 3; ic = 3; o1 = 0; return; }                   // N
-    if (e == 1) { ia = 1; ib = 3; ic = 3; o1 = 1; return; }                   // U
-    if (e == 2) { ia = 0; ib = 2; ic = 3; o1 = 2; return; }                   // Snu
-    o1 = e;
-    e -= 3;
-    if (e < p) { ia = 1; ib = R0 + e; ic = 3; return; }                       // Sr
-    e -= p;
-    if (e < q) { ia = 0; ib = E0 + e; ic = 3; return; }                       // Se
-    e -= q;
-    if (e < p * q) { ia = 0; ib = R0 + e / q; ic = E0 + e % q; return; }      // Sre
-    e -= p * q;
-    int a = 0;
-    if (e < q * (q + 1) / 2) {                                                // See (lower)
-        while ((a + 1) * (a + 2) / 2 <= e) ++a;
-        const int b = e - a * (a + 1) / 2;
-        ia = 0; ib = EE0 + a * q + b; ic = 3;
-        o1 = fSee + a * q + b;
-        if (a != b) o2 = fSee + b * q + a;
-        return;
-    }
-    e -= q * (q + 1) / 2;
-    while ((a + 1) * (a + 2) / 2 <= e) ++a;                                   // Srr (lower)
-    const int b = e - a * (a + 1) / 2;
-    ia = 1; ib = R0 + a; ic = R0 + b;
-    o1 = fSrr + a * p + b;
-    if (a != b) o2 = fSrr + b * p + a;
-}
-
-// The FP32 rows hold the weighted vectors too: [0] tau, [1] tau u, [2] tau (elogu - u),
-// [3] 1, then r (p), tau u r (p), tau eu (q), tau euu (q*q), so that every statistic is the
-// sum over the chunk of row[ia] * row[ib] (two operands instead of three).
 __device__ inline void stat_operands_w(int e, int p, int q, int& ia, int& ib, int& o1, int& o2)
 {
     const int R0 = 4, WR0 = 4 + p, E0 = 4 + 2 * p, EE0 = 4 + 2 * p + q;
@@ -242,7 +206,7 @@ __device__ void estep_reduce_body(const ReduceArgs& a, T* rows)
                     const double uv = a.u[pid];
                     rw[0] = (T)tv;
                     rw[1] = (T)(tv * uv);
-                    rw[2] = (T)(a.elogu[pid] - uv);
+                    rw[2] = (T)(tv * (a.elogu[pid] - uv));
                 }
                 rw[3] = T(1);
                 if (a.small_only) {
@@ -256,13 +220,17 @@ __device__ void estep_reduce_body(const ReduceArgs& a, T* rows)
                     }
                 } else {
                     const double* yj = a.y + (size_t)(j0 + t) * p;
-                    for (int i = 0; i < p; ++i) rw[4 + i] = (T)(yj[i] - a.mu[(size_t)h * p + i]);
+                    for (int i = 0; i < p; ++i) {
+                        const T ri = (T)(yj[i] - a.mu[(size_t)h * p + i]);
+                        rw[4 + i] = ri;
+                        rw[4 + p + i] = rw[1] * ri;
+                    }
                 }
                 if (pr) {
                     for (int k = 0; k < q + q * q; ++k) rw[4 + 2 * p + k] = rw[0] * (T)pr[2 + k];
                 } else {
-                    for (int k = 0; k < q; ++k) rw[4 + p + k] = (T)a.eu[pid * q + k];
-                    for (int k = 0; k < q * q; ++k) rw[4 + p + q + k] = (T)a.euu[pid * q * q + k];
+                    for (int k = 0; k < q; ++k) rw[4 + 2 * p + k] = rw[0] * (T)a.eu[pid * q + k];
+                    for (int k = 0; k < q * q; ++k) rw[4 + 2 * p + q + k] = rw[0] * (T)a.euu[pid * q * q + k];
                 }
             } else {
                 for (int i = 0; i < a.row; ++i) rw[i] = T(0);
@@ -281,12 +249,19 @@ __device__ void estep_reduce_body(const ReduceArgs& a, T* rows)
         }
         // small_only: N, U, Snu, Se and See (the tensor-core kernel writes Sr, Sre, Srr)
         const int Sred = a.small_only ? 3 + q + q * (q + 1) / 2 : stats_reduced(p, q);
-        for (int es = t; es < Sred; es += blockDim.x) {
-            const int e = !a.small_only || es < 3 ? es : es < 3 + q ? 3 + p + (es - 3) : 3 + p + q + p * q + (es - 3 - q);
-            int ia, ib, ic, o1, o2;
+        // FP64: where the statistics are few, the threads share out the rows too (nsub groups of
+        // lanes threads, each every nsub-th row, added in order at the end)
+        int lanes = blockDim.x;
+        if (sizeof(T) == sizeof(double))
+            while (lanes >= 2 * Sred && lanes > 32) lanes >>= 1;
+        const int nsub = blockDim.x / lanes, sub = t / lanes;
+        for (int es = t - sub * lanes; es < (nsub > 1 ? lanes : Sred); es += lanes) {
+            const bool on = es < Sred;
+            const int e = !on ? 0 : !a.small_only || es < 3 ? es : es < 3 + q ? 3 + p + (es - 3) : 3 + p + q + p * q + (es - 3 - q);
+            int ia, ib, o1, o2;
             T acc = T(0), comp = T(0);
+            stat_operands_w(e, p, q, ia, ib, o1, o2);
             if (sizeof(T) == sizeof(float)) {
-                stat_operands_w(e, p, q, ia, ib, o1, o2);
                 // two compensated sums, even and odd rows (independent chains), added at the end
                 T acc1 = T(0), comp1 = T(0);
                 const T* ra = rows + ia;
@@ -315,10 +290,13 @@ __device__ void estep_reduce_body(const ReduceArgs& a, T* rows)
                     acc = tt;
                 }
             } else {
-                stat_operands(e, p, q, ia, ib, ic, o1, o2);
-                for (int jj = 0; jj < cnt; ++jj) {
-                    const T* rw = rows + (size_t)jj * a.row;
-                    acc += rw[ia] * rw[ib] * rw[ic];
+                for (int jj = sub; jj < cnt; jj += nsub) acc += rows[(size_t)jj * a.row + ia] * rows[(size_t)jj * a.row + ib];
+                if (nsub > 1) {
+                    T* part = rows + (size_t)a.chunk * a.row + (size_t)g * a.chunk + a.chunk + CF_MAXG;  // behind lpi
+                    part[t] = acc;
+                    __syncthreads();
+                    if (sub > 0 || !on) break;
+                    for (int k = 1; k < nsub; ++k) acc += part[k * lanes + t];
                 }
             }
             out[h * S + o1] = (double)acc;

@@ -154,7 +154,7 @@ __global__ void __launch_bounds__(32) setup_components_kernel(Dims D, Layout Ly,
                                    - 0.5 * logdet;
             Fh[Ly.scal + SC_PSI] = cf_digamma(0.5 * (v + p));
         }
-        Fh[Ly.scal + 3] = 0.0;
+        Fh[Ly.scal + SC_RL0] = isinf(v) ? 1.0 : sqrt((v + p + 2.0) / (v + p));
         if (!corr_chol_dev(q, Lam, Fh + Ly.dq, Fh + Ly.Lq)) atomicOr(flags, KF_NOTPD_LAMBDA);
     }
     // level 1: Schur complement of Lambda at each r (lane r), level 2 inside
@@ -247,7 +247,7 @@ __global__ void dof_consts_kernel(Dims D, Layout Ly, const double* __restrict__ 
         const double ltm = lgamma(0.5 * v) - lgamma(0.5 * (v - 1.0)) - 0.5 * log((v - 1.0) * CF_PI);
         const double c[CST_STRIDE] = {t1_lgb(v), t1_lgb(v + 1.0),
                                       cf_t_const(v),
-                                      lt, v > 1.0 ? ltm : 0.0, lgamma(0.5 * v), exp(lt), v > 1.0 ? exp(ltm) : 0.0};
+                                      lt, v > 1.0 ? ltm : 0.0, lgamma(0.5 * v), exp(lt) * sqrt(v), v > 1.0 ? exp(ltm) / sqrt(v - 1.0) : 0.0};
         for (int k = 0; k < CST_STRIDE; ++k) {
             c64[t * CST_STRIDE + k] = c[k];
             c32[t * CST_STRIDE + k] = (float)c[k];

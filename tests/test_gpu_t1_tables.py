@@ -97,3 +97,21 @@ def test_t1_records(cf, oracle, p, q, n, nu):
         err = np.abs(got[k] - o[k])[ok] / np.maximum(1.0 if k == "logf" else 0.0, np.abs(o[k][ok]))
         print(f"p={p} q={q} n={n} {k}: worst {err.max():.2e}")
         assert err.max() <= rtol
+
+
+@pytest.mark.parametrize("precision,rtol", [(0, 1e-12), (1, 5e-5)])
+def test_level1_read_back(cf, oracle, precision, rtol):
+    """At q = 2 the E-step forms the level-1 T_1 inside combine; the diagnostic read-back still
+    gives their limits and values."""
+    ctx, y, par, _ = _setup(cf, 2, 2, 41, (1.0, 6.0, 60.0, 150.0))
+    if precision:
+        ctx = cf.cfust_create(2, 2, 4, 41, cf.cfust_default_opts(precision=precision))
+        cf.cfust_set_data(ctx, y)
+        cf.cfust_set_params(ctx, par)
+    cf.cfust_estep(ctx)
+    before = cf.cfust_debug_read(ctx, 6).copy()
+    bt = cf.cfust_debug_read(ctx, 4).reshape(4, 41, 2)
+    got = cf.cfust_debug_read(ctx, 7).reshape(4, 41, 2)
+    ref = np.array([[[oracle.t1cdf(b, par["nu"][h] + 3) for b in row] for row in bt[h]] for h in range(4)])
+    assert np.abs(got / ref - 1.0).max() <= rtol
+    assert np.array_equal(before, cf.cfust_debug_read(ctx, 6))
