@@ -67,6 +67,7 @@ struct cfust_ctx {
     float *glx32 = nullptr, *glw32 = nullptr;
     float *glx32h = nullptr, *glw32h = nullptr;  // T2_NH nodes for graded T_2 pieces
     float *glx32l = nullptr, *glw32l = nullptr;  // node sets of the FP32 T_2 piece classes (t2_lo_class)
+    double *glx64l = nullptr, *glw64l = nullptr;  // FP64: 32 nodes (t2_lo_f64)
     int t2n_lo = 0;
     double *logf = nullptr, *u = nullptr, *elogu = nullptr, *eu = nullptr, *euu = nullptr,
            *se = nullptr, *tau = nullptr;
@@ -398,7 +399,7 @@ static void free_all(cfust_ctx* c)
     sur_free(c->sur);
     void* bufs[] = {c->y, c->pi, c->mu, c->Sigma, c->Delta, c->nu, c->pi_n, c->mu_n, c->Sigma_n,
                     c->Delta_n, c->nu_n, c->F, c->dofs, c->cst64, c->cst32, c->chi64, c->chi32, c->shf64, c->shf32, c->wtab,
-                    c->glx64, c->glw64, c->glx32, c->glw32, c->glx32h, c->glw32h, c->glx32l, c->glw32l,
+                    c->glx64, c->glw64, c->glx32, c->glw32, c->glx32h, c->glw32h, c->glx32l, c->glw32l, c->glx64l, c->glw64l,
                     c->logf, c->u, c->elogu, c->eu,
                     c->euu, c->se, c->tau, c->partial, c->stats, c->flags, c->comp_status,
                     c->stage32, c->pd, c->pc, c->fix_count, c->fix_list, c->y32, c->F32, c->pr32, c->pd32, c->pc32, c->res32_l0, c->h32tab, c->h32scale,
@@ -501,7 +502,7 @@ extern "C" cfust_status cfust_create(cfust_ctx** out, int p, int q, int g, int64
     c->t2n = o.t2_nodes ? o.t2_nodes : (o.precision == CFUST_PREC_FP64 ? 64 : 32);
     // FP32 modes by default: 8-24 nodes by t2_lo_class where the integrand is smooth enough
     // (a node count set in the options holds for every piece)
-    c->t2n_lo = (o.precision != CFUST_PREC_FP64 && o.t2_nodes == 0) ? 1 : 0;
+    c->t2n_lo = o.t2_nodes == 0 ? 1 : 0;  // FP64: 32 of 64 nodes where those lose nothing (t2_lo_f64)
     cudaDeviceProp prop;
     if ((e = cudaGetDeviceProperties(&prop, o.device)) != cudaSuccess) {
         cfust_status s = fail(nullptr, CFUST_ECUDA, std::string("cfust_create: ") + cudaGetErrorString(e));
@@ -551,6 +552,7 @@ extern "C" cfust_status cfust_create(cfust_ctx** out, int p, int q, int g, int64
     ALLOC(glx64, c->t2n); ALLOC(glw64, c->t2n); ALLOC(glx32, c->t2n); ALLOC(glw32, c->t2n);
     ALLOC(glx32h, T2_NH); ALLOC(glw32h, T2_NH);
     ALLOC(glx32l, T2_LO_TOTAL); ALLOC(glw32l, T2_LO_TOTAL);
+    ALLOC(glx64l, 32); ALLOC(glw64l, 32);
     ALLOC(logf, ng); ALLOC(u, ng); ALLOC(elogu, ng); ALLOC(se, ng); ALLOC(tau, ng);
     ALLOC(eu, ng * q); ALLOC(euu, ng * q * q);
     ALLOC(partial, part);
@@ -677,6 +679,12 @@ extern "C" cfust_status cfust_create(cfust_ctx** out, int p, int q, int g, int64
         cp(c->wtab, wt.data(), sizeof(float) * wt.size());
     }
     cp(c->glx64, gx.data(), sizeof(double) * gx.size());
+    {
+        std::vector<double> gx32n, gw32n;
+        gauss_legendre01(32, gx32n, gw32n);
+        cp(c->glx64l, gx32n.data(), sizeof(double) * 32);
+        cp(c->glw64l, gw32n.data(), sizeof(double) * 32);
+    }
     cp(c->glw64, gw.data(), sizeof(double) * gw.size());
     cp(c->glx32, gx32.data(), sizeof(float) * gx32.size());
     cp(c->glw32, gw32.data(), sizeof(float) * gw32.size());
@@ -870,7 +878,7 @@ static IntegArgs integ_args(const cfust_ctx* c)
     ia.glx64 = c->glx64; ia.glw64 = c->glw64; ia.glx32 = c->glx32; ia.glw32 = c->glw32;
     ia.t2n = c->t2n;
     ia.glx32h = c->glx32h; ia.glw32h = c->glw32h;
-    ia.t2n_lo = c->t2n_lo; ia.glx32l = c->glx32l; ia.glw32l = c->glw32l;
+    ia.t2n_lo = c->t2n_lo; ia.glx64l = c->glx64l; ia.glw64l = c->glw64l; ia.glx32l = c->glx32l; ia.glw32l = c->glw32l;
     ia.h32tab = c->h32tab;
     ia.h32scale = c->h32scale;
     ia.h32_case = 0;

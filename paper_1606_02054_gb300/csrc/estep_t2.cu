@@ -308,13 +308,72 @@ __global__ void __launch_bounds__(T2P_WARPS * CF_WARP, 4) t2_pieces_kernel(RecSe
 // near phi_h), the factor 1 - T_1(-z) is formed at the nodes, a second logarithm and exponential.
 //
 // Bound by the FP64 pipe (1/64 of the FP32 rate): a node was a continued fraction with six
-// divisions an iteration, about 1460 FP64 slots, and is about 100.  A warp takes up to 32
+// divisions an iteration, about 1460 FP64 slots, and is about 80.  A warp takes up to 32
 // records: lane l sets up record l (two arctangents, three square roots, the univariate
 // part), then the warp runs each record's nodes over its lanes.  Measured on a GB300:
-// p = 16, q = 2, g = 8, n = 20,000 (3.2e5 records of 97 nodes): 72.1 -> 7.6 ms;
-// p = q = g = 2, n = 1000 (4000 records): 1.48 -> 0.22 ms.
+// p = 16, q = 2, g = 8, n = 20,000 (3.2e5 records): 72.1 ms with the continued fraction and 97
+// nodes a record, 7.5 through H with log() and exp(), 3.8 with node_log, node_exp and 57 nodes
+// (t2_lo_f64); p = q = g = 2, n = 1000 (4000 records): 1.48 -> 0.12 ms.
 constexpr int T2D_WARPS = 8;
 enum { T2D_ANC0, T2D_PHIS, T2D_L0, T2D_L1, T2D_D0, T2D_SC, T2D_NU, T2D_N };
+
+// log v (v > 0, normal) and e^x (x <= 0) for the nodes, by tables in shared memory: v = 2^e m with
+// c = 1/m at the middle of m's 128th rounded to FP32, log v = e ln 2 - log c + log1p(m c - 1), the
+// halves above m = sqrt 2 counted below the next power of two, so that nothing cancels near
+// v = 1; e^x = 2^(k/64) e^r.  Series to r^6 (|r| < 2^-8) and r^5 (|r| < 0.0055): 10 FP64 operations
+// each, about an ulp, where log() and exp() measured 28 and 15.
+struct NodeTables {
+    double2 lg[128];
+    double ex[64];
+};
+__device__ __forceinline__ void node_tables_init(NodeTables& nt)
+{
+    for (int t = threadIdx.x; t < 128; t += blockDim.x) {
+        const double c = (double)(float)(128.0 / (t + 128.5));
+        nt.lg[t] = make_double2(c, -log(c) - (t >= 53 ? CF_LN2 : 0.0));
+        if (t < 64) nt.ex[t] = exp2(t / 64.0);
+    }
+    __syncthreads();
+}
+__device__ __forceinline__ double node_log(double v, const NodeTables& nt)
+{
+    const int hi = __double2hiint(v), i = (hi >> 13) & 127;
+    const int e = (hi >> 20) - 1023 + (i >= 53 ? 1 : 0);
+    const double ed = __hiloint2double(0x43300000, e ^ 0x80000000) - 4503601774854144.0;  // 2^52 + 2^31
+    const double2 c = nt.lg[i];
+    const double r = fma(__hiloint2double((hi & 0xfffff) | 0x3ff00000, __double2loint(v)), c.x, -1.0);
+    double q = -1.0 / 6;
+    q = fma(q, r, 1.0 / 5);
+    q = fma(q, r, -1.0 / 4);
+    q = fma(q, r, 1.0 / 3);
+    q = fma(q, r, -1.0 / 2);
+    return fma(ed, CF_LN2, c.y) + fma(r * r, q, r);
+}
+__device__ __forceinline__ double node_exp(double x, const NodeTables& nt)
+{
+    const double magic = 6755399441055744.0;  // 3 * 2^51
+    const double m = fma(x, 92.33248261689366, magic);  // 64 / ln 2
+    const int k = __double2loint(m);
+    const double kd = m - magic;
+    // ln 2 / 64 in two parts, the first with 32 zero low bits
+    double r = fma(kd, -0.010830417275428772, x);
+    r = fma(kd, -7.420820373486988e-09, r);
+    double q = 1.0 / 120;
+    q = fma(q, r, 1.0 / 24);
+    q = fma(q, r, 1.0 / 6);
+    q = fma(q, r, 0.5);
+    q = fma(q, r, 1.0);
+    q = fma(q, r, 1.0) * nt.ex[k & 63];
+    return x < -690.0 ? 0.0 : __hiloint2double(__double2hiint(q) + ((k >> 6) << 20), __double2loint(q));
+}
+
+// The t2n = 64 nodes of a piece are 32 (one round of the warp instead of two) where the
+// Gauss-Legendre error of 32 stays below 1e-16 of the record's T_2: 10 <= dof <= 64,
+// |rho| < 0.9 and L^2 (dof - 1 + 0.5 zs^2) <= 90.  Measured in 80-bit arithmetic on 24,000 records of the
+// two distributions of fit_t2_classes.py: below 1e-16 up to a root of 10.2 (kept: 9.5),
+// 67 % of the pieces there.  Only without a node count in the options (a.t2n_lo).
+constexpr int T2D_NLO = 32;
+__device__ __forceinline__ bool t2_lo_f64(double L, double nu, double zs2) { return L * L * (nu - 1.0 + 0.5 * zs2) <= 90.0; }
 
 // records outside the tables (|rho| = 1, dof above H1_DOF_MAX): the general routine
 static __device__ __noinline__ double t2_general_f64(const RecSet& r, const IntegArgs& a, long long i, int lane, int* nn)
@@ -329,17 +388,19 @@ static __device__ __noinline__ double t2_general_f64(const RecSet& r, const Inte
 // chunk: records per warp, 1..32
 __global__ void __launch_bounds__(T2D_WARPS * CF_WARP, 2) t2_records_h1_kernel(RecSet r, IntegArgs a, int chunk)
 {
+    __shared__ NodeTables nt;
     __shared__ double sf[T2D_WARPS][T2D_N][CF_WARP];
     const int lane = threadIdx.x & (CF_WARP - 1), wib = threadIdx.x >> 5;
     const long long warp = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const long long nwarps = ((long long)gridDim.x * blockDim.x) >> 5;
     double (*R)[CF_WARP] = sf[wib];
-    const int n = a.t2n;
+    node_tables_init(nt);
     unsigned long long nodes = 0;  // this warp's quadrature nodes (profiler count)
     for (long long base = warp * chunk; base < r.nrec; base += nwarps * chunk) {
         const int cnt = r.nrec - base < chunk ? (int)(r.nrec - base) : chunk;
         // bits: 0 split, 1 the first piece's z > 0 (the second one's is the opposite), 2 graded,
-        // 3 general routine, 4 the second piece's factor 1 - T_1(-z) at the nodes
+        // 3 general routine, 4 the second piece's factor 1 - T_1(-z) at the nodes, 5 and 6 the first
+        // and second piece with T2D_NLO nodes
         int kind = 0, tab = 0;
         double C2 = 0.0, part = 0.0;
         if (lane < cnt) {
@@ -366,7 +427,10 @@ __global__ void __launch_bounds__(T2D_WARPS * CF_WARP, 2) t2_records_h1_kernel(R
                 R[T2D_L0][lane] = -anc;
                 R[T2D_L1][lane] = D;
                 R[T2D_D0][lane] = split ? 0.0 : D;
-                R[T2D_SC][lane] = sqrt(R2 / (omr2 * nu));  // |zs| / sqrt(nu + 1)
+                const double c1 = R2 / (omr2 * nu);  // zs^2 / (nu + 1)
+                R[T2D_SC][lane] = sqrt(c1);
+                if (a.t2n_lo && nu >= 10.0 && nu <= 64.0 && ar < 0.9)
+                    kind |= (t2_lo_f64(anc, nu, c1 * (nu + 1.0)) ? 32 : 0) | (t2_lo_f64(D, nu, c1 * (nu + 1.0)) ? 64 : 0);
                 R[T2D_NU][lane] = nu;
                 if (pos0 || split) {  // a piece with z > 0: its part of T_1(.; nu)
                     const double* t1 = a.h1tab + (size_t)tab * H1_SIZE;
@@ -405,9 +469,14 @@ __global__ void __launch_bounds__(T2D_WARPS * CF_WARP, 2) t2_records_h1_kernel(R
                 const double anc = pc ? R[T2D_PHIS][l] : R[T2D_ANC0][l], d0 = pc ? 0.0 : R[T2D_D0][l];
                 const double L = pc ? R[T2D_L1][l] : R[T2D_L0][l];
                 double s = 0.0;
+                const bool lo = (kd >> (5 + pc)) & 1;
+                const int n = lo ? T2D_NLO : a.t2n;
+                const double* __restrict__ gx = lo ? a.glx64l : a.glx64;
+                const double* __restrict__ gw = lo ? a.glw64l : a.glw64;
+                nodes += (unsigned long long)n;
                 for (int t = lane; t < n; t += CF_WARP) {
-                    const double u = a.glx64[t];
-                    double w = a.glw64[t], um = u;
+                    const double u = gx[t];
+                    double w = gw[t], um = u;
                     if (kd & 4) {  // nodes anchor + L u^3, weights 3 u^2
                         um = u * u * u;
                         w *= 3.0 * u * u;
@@ -418,13 +487,12 @@ __global__ void __launch_bounds__(T2D_WARPS * CF_WARP, 2) t2_records_h1_kernel(R
                     const double rr = rsqrt(fma(q, q, 1.0));
                     const double H = h1_eval(fabs(q) * rr, t2);
                     if (kd & pc << 4)
-                        s = fma(w * exp(num1 * log(fabs(sp))), 1.0 - exp(num1 * log(rr)) * (rr * rr) * H, s);
+                        s = fma(w * node_exp(num1 * node_log(fabs(sp), nt), nt), 1.0 - node_exp(num1 * node_log(rr, nt), nt) * (rr * rr) * H, s);
                     else
-                        s = fma(w * (rr * rr), exp(num1 * log(fabs(sp) * rr)) * H, s);
+                        s = fma(w * (rr * rr), node_exp(num1 * node_log(fabs(sp) * rr, nt), nt) * H, s);
                 }
                 acc = fma(((kd >> 1) ^ pc) & !(kd & pc << 4) ? -fabs(L) : fabs(L), s, acc);
             }
-            nodes += (unsigned long long)(n << (kd & 1));
             acc = warp_sum(acc);
             if (lane == l) mine = acc;
         }

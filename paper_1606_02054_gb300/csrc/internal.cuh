@@ -209,8 +209,11 @@ struct IntegArgs {
     // exact E[log W] (else null): log(s^2) at every point of the chi tables, same layout
     const double* lchi64;
     const float* lchi32;
-    // FP64 T_1 and T_2 (else null): the tables of H1_* below, index 4 h + e
+    // FP64 T_1 and T_2 (else null): the tables of H1_* below, index 4 h + e; 32 nodes for the
+    // pieces of t2_lo_f64
     const double* h1tab;
+    const double* glx64l;
+    const double* glw64l;
 };
 
 // FP64 univariate t CDFs through a table per dof.  With sin phi = sqrt(v/(v + x^2)) and
