@@ -20,6 +20,10 @@ __global__ void setup_components_kernel(Dims, Layout, const double*, const doubl
                                         const double*, double*, int*);
 __global__ void chi_table_kernel(int, int, const double*, const double*, Lattice, const double*, double, double*,
                                  float*, double*, float*);
+__global__ void chi_score_kernel(Lattice, const double*, double*);
+__global__ void chi_poly_kernel(int, double, const double*, const double*, double*);
+__global__ void chi_eval_kernel(int, int, double, const double*, const double*, Lattice, const double*, const double*,
+                                const double*, double*, float*, double*, float*);
 __global__ void dof_consts_kernel(Dims, Layout, const double*, int, double*, double*, float*);
 __global__ void h32_table_kernel(const double*, float4*, float*, int);
 __global__ void h1_table_kernel(const double*, double*, int);
@@ -57,6 +61,9 @@ struct cfust_ctx {
     float* cst32 = nullptr;
     double* chi64 = nullptr;
     float* chi32 = nullptr;
+    double* chi_z = nullptr;     // FP32 modes: normal scores of coordinate 0, and the tables' coefficients
+    double* chi_coef = nullptr;  //   (chi_eval_kernel)
+    double chi_zr = 8.0;         // the scores' range that the coefficients cover
     double* lchi64 = nullptr;  // exact E[log W]: log(s^2) beside the chi tables
     float* lchi32 = nullptr;
     double* shf64 = nullptr;
@@ -403,7 +410,7 @@ static void free_all(cfust_ctx* c)
                     c->logf, c->u, c->elogu, c->eu,
                     c->euu, c->se, c->tau, c->partial, c->stats, c->flags, c->comp_status,
                     c->stage32, c->pd, c->pc, c->fix_count, c->fix_list, c->y32, c->F32, c->pr32, c->pd32, c->pc32, c->res32_l0, c->h32tab, c->h32scale,
-                    c->work_dev, c->seg, c->lchi64, c->lchi32, c->h1tab, c->fix_part, c->fix_done, c->latu};
+                    c->work_dev, c->seg, c->lchi64, c->lchi32, c->h1tab, c->fix_part, c->fix_done, c->latu, c->chi_z, c->chi_coef};
     for (void* b : bufs)
         if (b) cudaFree(b);
     for (RecSet& r : c->rec) {
@@ -542,6 +549,11 @@ extern "C" cfust_status cfust_create(cfust_ctx** out, int p, int q, int g, int64
     ALLOC(cst32, 3 * g * CST_STRIDE);
     ALLOC(chi64, ntab * NM);
     ALLOC(chi32, ntab * NM);
+    const bool chi_poly = q >= 3 && o.precision != CFUST_PREC_FP64;
+    if (chi_poly) {
+        ALLOC(chi_z, NM);
+        ALLOC(chi_coef, (size_t)ntab * 32 * 10);
+    }
     if (o.elogw == CFUST_ELOGW_EXACT) {
         ALLOC(lchi64, ntab * NM);
         ALLOC(lchi32, ntab * NM);
@@ -657,6 +669,21 @@ extern "C" cfust_status cfust_create(cfust_ctx** out, int p, int q, int g, int64
     }
     cp(c->shf64, s64.data(), sizeof(double) * s64.size());
     cp(c->shf32, s32.data(), sizeof(float) * s32.size());
+    if (chi_poly) {  // before the copies below, which wait for it (legacy stream)
+        // the smaller tail of every coordinate 0 is at least pm, so |z| <= sqrt(-2 ln(2 pm))
+        double pm = 0.5;
+        for (int m = 0; m < o.qmc_shifts; ++m)
+            for (int i = 0; i < o.qmc_points; ++i) {
+                double x = (double)i / o.qmc_points + s64[m * CF_MAXDIM];
+                if (x >= 1.0) x -= 1.0;
+                const double wc = std::fabs(2.0 * x - 1.0);
+                pm = std::min(pm, std::min(wc, 1.0 - wc));
+            }
+        c->chi_zr = pm > 1e-14 ? std::min(8.0, std::sqrt(-2.0 * std::log(2.0 * pm)) + 0.05) : 8.0;
+        chi_score_kernel<<<(int)std::min<size_t>((NM + 255) / 256, 8 * (size_t)c->nsm), 256>>>(c->lat, c->shf64, c->chi_z);
+        if ((e = cudaGetLastError()) != cudaSuccess && s == CFUST_OK)
+            s = fail(nullptr, CFUST_ECUDA, std::string("cfust_create: ") + cudaGetErrorString(e));
+    }
     if (c->single_pass && o.precision != CFUST_PREC_FP64 && q <= 4) {
         // baker-transformed lattice coordinates d = 1..q of every (shift, point), FP64 -> FP32
         // (read by the FP32 moment pass at q <= 4)
@@ -856,15 +883,20 @@ static cfust_status launch_setup(cfust_ctx* c, int density_only)
         prof_begin(c, CFUST_PROF_CHI);
         // the single-pass E-step reads only the dof nu+p tables (index 3h)
         const int every = c->single_pass ? 3 : 1;
-        const long long total = 3LL * c->g / every * c->lat.N * c->lat.M;
+        const int ntab = 3 * c->g / every;
+        const long long total = (long long)ntab * c->lat.N * c->lat.M;
         const int blocks = (int)std::min<long long>((total + 127) / 128, 64LL * c->nsm);
-        // the FP64 table serves the FP64 integrators; in the FP32 modes only the rare FP64
-        // fix-up reads it, and 1e-9 is far inside what a pair sent there needs
-        const double rtol = c->opts.precision == CFUST_PREC_FP64 ? 1e-15 : 1e-9;
-        chi_table_kernel<<<blocks, 128, 0, c->st>>>(3 * c->g, every, c->dofs, c->cst64, c->lat, c->shf64, rtol,
-                                                     c->chi64, c->chi32, c->lchi64, c->lchi32);
+        if (c->chi_z) {  // FP32 modes (the FP64 table serves the rare FP64 fix-up there)
+            chi_poly_kernel<<<dim3(ntab, 32), 32, 0, c->st>>>(every, c->chi_zr, c->dofs, c->cst64, c->chi_coef);
+            LAUNCHED();
+            chi_eval_kernel<<<blocks, 128, 0, c->st>>>(ntab, every, c->chi_zr, c->dofs, c->cst64, c->lat, c->shf64, c->chi_z,
+                                                       c->chi_coef, c->chi64, c->chi32, c->lchi64, c->lchi32);
+        } else {
+            chi_table_kernel<<<blocks, 128, 0, c->st>>>(3 * c->g, every, c->dofs, c->cst64, c->lat, c->shf64, 1e-15,
+                                                        c->chi64, c->chi32, c->lchi64, c->lchi32);
+        }
         LAUNCHED();
-        prof_end(c, CFUST_PROF_CHI, 1);
+        prof_end(c, CFUST_PROF_CHI, c->chi_z ? 2 : 1);
     }
     return CFUST_OK;
 }

@@ -317,56 +317,6 @@ __global__ void __launch_bounds__(T2P_WARPS * CF_WARP, 4) t2_pieces_kernel(RecSe
 constexpr int T2D_WARPS = 8;
 enum { T2D_ANC0, T2D_PHIS, T2D_L0, T2D_L1, T2D_D0, T2D_SC, T2D_NU, T2D_N };
 
-// log v (v > 0, normal) and e^x (x <= 0) for the nodes, by tables in shared memory: v = 2^e m with
-// c = 1/m at the middle of m's 128th rounded to FP32, log v = e ln 2 - log c + log1p(m c - 1), the
-// halves above m = sqrt 2 counted below the next power of two, so that nothing cancels near
-// v = 1; e^x = 2^(k/64) e^r.  Series to r^6 (|r| < 2^-8) and r^5 (|r| < 0.0055): 10 FP64 operations
-// each, about an ulp, where log() and exp() measured 28 and 15.
-struct NodeTables {
-    double2 lg[128];
-    double ex[64];
-};
-__device__ __forceinline__ void node_tables_init(NodeTables& nt)
-{
-    for (int t = threadIdx.x; t < 128; t += blockDim.x) {
-        const double c = (double)(float)(128.0 / (t + 128.5));
-        nt.lg[t] = make_double2(c, -log(c) - (t >= 53 ? CF_LN2 : 0.0));
-        if (t < 64) nt.ex[t] = exp2(t / 64.0);
-    }
-    __syncthreads();
-}
-__device__ __forceinline__ double node_log(double v, const NodeTables& nt)
-{
-    const int hi = __double2hiint(v), i = (hi >> 13) & 127;
-    const int e = (hi >> 20) - 1023 + (i >= 53 ? 1 : 0);
-    const double ed = __hiloint2double(0x43300000, e ^ 0x80000000) - 4503601774854144.0;  // 2^52 + 2^31
-    const double2 c = nt.lg[i];
-    const double r = fma(__hiloint2double((hi & 0xfffff) | 0x3ff00000, __double2loint(v)), c.x, -1.0);
-    double q = -1.0 / 6;
-    q = fma(q, r, 1.0 / 5);
-    q = fma(q, r, -1.0 / 4);
-    q = fma(q, r, 1.0 / 3);
-    q = fma(q, r, -1.0 / 2);
-    return fma(ed, CF_LN2, c.y) + fma(r * r, q, r);
-}
-__device__ __forceinline__ double node_exp(double x, const NodeTables& nt)
-{
-    const double magic = 6755399441055744.0;  // 3 * 2^51
-    const double m = fma(x, 92.33248261689366, magic);  // 64 / ln 2
-    const int k = __double2loint(m);
-    const double kd = m - magic;
-    // ln 2 / 64 in two parts, the first with 32 zero low bits
-    double r = fma(kd, -0.010830417275428772, x);
-    r = fma(kd, -7.420820373486988e-09, r);
-    double q = 1.0 / 120;
-    q = fma(q, r, 1.0 / 24);
-    q = fma(q, r, 1.0 / 6);
-    q = fma(q, r, 0.5);
-    q = fma(q, r, 1.0);
-    q = fma(q, r, 1.0) * nt.ex[k & 63];
-    return x < -690.0 ? 0.0 : __hiloint2double(__double2hiint(q) + ((k >> 6) << 20), __double2loint(q));
-}
-
 // The t2n = 64 nodes of a piece are 32 (one round of the warp instead of two) where the
 // Gauss-Legendre error of 32 stays below 1e-16 of the record's T_2: 10 <= dof <= 64,
 // |rho| < 0.9 and L^2 (dof - 1 + 0.5 zs^2) <= 90.  Measured in 80-bit arithmetic on 24,000 records of the

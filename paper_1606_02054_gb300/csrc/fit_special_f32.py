@@ -15,6 +15,7 @@ mapped variable t in [-1, 1]:
   Phi^-1(p), pm = min(p, 1 - p) in [1e-37, 1/2]:
       x = log2(-log2 pm) in [0, 7],  Phi^-1(pm) = x Q(t), t = affine(x)
       (the factor x makes Phi^-1(1/2) = 0 exactly);  Phi^-1(p) = -x Q for p > 1/2.
+      The start of the FP64 inverse (ncdfinv_tab): x in [0, 10], degree 9.
   atan(a), 0 <= a <= 1:  a R(a^2), R fitted on [0, 1] (relative error of atan(a)/a)
       (cf_atan2_f32 folds the other octants onto it).
   sin(x), |x| <= pi:  r = |x| folded to [0, pi/2] (pi - |x| beyond pi/2),
@@ -56,7 +57,8 @@ def fit_ncdf(deg=8, zmax=9.5):
 def fit_ncdfinv(deg=8, xmax=7.0):
     x = np.linspace(1e-6, xmax, 400001)
     pm = 2.0 ** (-(2.0 ** x))
-    target = sp.ndtri(pm)
+    ok = pm > 1e-301  # x = 10 is beyond the FP64 range
+    x, target = x[ok], sp.ndtri(pm[ok])
     m, _ = lawson(x, target / x, deg, 0.0, xmax)
     err = np.abs(x * Pm.polyval(2.0 * x / xmax - 1.0, m) - target).max()
     return m, 2.0 / xmax, -1.0, err
@@ -90,6 +92,10 @@ if __name__ == "__main__":
     print("P =", ", ".join(f"{c:.9e}f" for c in m))
     m, A, B, e = fit_ncdfinv()
     print(f"// Phi^-1: max |error| {e:.2e}  (value = x * Q(t))")
+    print(f"t = x * {A!r}f + {B!r}f")
+    print("Q =", ", ".join(f"{c:.9e}f" for c in m))
+    m, A, B, e = fit_ncdfinv(9, 10.0)
+    print(f"// start of the FP64 Phi^-1: max |error| {e:.2e}")
     print(f"t = x * {A!r}f + {B!r}f")
     print("Q =", ", ".join(f"{c:.9e}f" for c in m))
     coef, e = fit_sin()

@@ -220,6 +220,99 @@ __global__ void chi_table_kernel(int ndof, int every, const double* __restrict__
     }
 }
 
+// The same tables in the FP32 modes.  The lattice coordinate w_0 of a point never changes, so its
+// normal score z = Phi^-1(w_0) is kept (chi_score_kernel, once per context), and log s is a smooth
+// function of z (nearly linear for a large dof): degree CHI_D polynomials on CHI_CELLS cells of
+// [-zr, zr] through quantiles at the cells' Chebyshev nodes, 320 quantiles a dof instead of
+// N x M = 8192.  zr <= 8 covers the lattice's own scores (4.4 at 1024 x 8 points; the extreme
+// quantiles are the longest chains); points beyond it take the quantile itself.  Interpolation
+// below 3e-14 of s for dof 1 to 1000 at zr = 8 (against scipy; a dof here is nu + p + j > 1), where
+// the full table's quantiles were taken to 1e-9 in these modes.  One E-step's tables on a GB300,
+// 8192 points, single pass: p = q = g = 4 1.1 -> 0.19 ms, p = q = g = 6 1.4 -> 0.19 ms; what is left
+// is a serial chain (a few Newton steps, each an incomplete gamma function).
+constexpr int CHI_CELLS = 32, CHI_D = 9, CHI_NC = CHI_D + 1;
+
+__global__ void chi_score_kernel(Lattice lat, const double* __restrict__ shf, double* __restrict__ z)
+{
+    const int total = lat.M * lat.N;
+    for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < total; t += gridDim.x * blockDim.x) {
+        const int i = t % lat.N, m = t / lat.N;
+        double x = (double)(((long long)i * lat.z[0]) % lat.N) / (double)lat.N + shf[m * CF_MAXDIM];
+        if (x >= 1.0) x -= 1.0;
+        const double wc = fabs(2.0 * x - 1.0), w = 1.0 - wc;
+        z[t] = w < 0.5 ? normcdfinv(w) : -normcdfinv(wc);
+    }
+}
+
+// table k = every * blockIdx.x, cell blockIdx.y (a warp of its own: a quantile is a long serial
+// chain of FP64 operations, so they are spread over the SMs): the coefficients of log s in powers
+// of t in [-1/2, 1/2]
+__global__ void __launch_bounds__(32) chi_poly_kernel(int every, double zr, const double* __restrict__ dofs,
+                                                      const double* __restrict__ cst, double* __restrict__ coef)
+{
+    __shared__ double f[CHI_NC], cn[CHI_NC];
+    const int k = blockIdx.x * every, cell = blockIdx.y, j = threadIdx.x;
+    const double dof = dofs[k];
+    if (isinf(dof)) return;  // the normal limit: s = 1
+    if (j < CHI_NC) {
+        const double z = zr * ((cell + 0.5 + 0.5 * cospi((2 * j + 1) / (2.0 * CHI_NC))) * (2.0 / CHI_CELLS) - 1.0);
+        f[j] = 0.5 * log(cf_chi2_node(z, dof, cst[k * CST_STRIDE + CST_LGA]) / dof);
+    }
+    __syncwarp();
+    const double f0 = f[CHI_NC / 2];
+    if (j < CHI_NC) {
+        double s = 0.0;
+        for (int i = 0; i < CHI_NC; ++i) s += (f[i] - f0) * cospi((j * (2 * i + 1) % (4 * CHI_NC)) / (2.0 * CHI_NC));
+        cn[j] = s * (j ? 2.0 / CHI_NC : 1.0 / CHI_NC);
+    }
+    __syncwarp();
+    if (j < CHI_NC) {
+        double s = 0.0;
+        for (int n = CHI_NC - 1; n >= j; --n) s += cn[n] * h1_cheb[n][j];
+        s *= (double)(1 << j);  // x = 2 t
+        coef[((size_t)k * CHI_CELLS + cell) * CHI_NC + j] = j ? s : s + f0;
+    }
+}
+
+__global__ void chi_eval_kernel(int ntab, int every, double zr, const double* __restrict__ dofs, const double* __restrict__ cst,
+                                Lattice lat, const double* __restrict__ shf, const double* __restrict__ zq,
+                                const double* __restrict__ coef, double* __restrict__ t64, float* __restrict__ t32,
+                                double* __restrict__ l64, float* __restrict__ l32)
+{
+    const long long NM = (long long)lat.M * lat.N;
+    const long long total = ntab * NM;
+    for (long long te = blockIdx.x * (long long)blockDim.x + threadIdx.x; te < total;
+         te += (long long)gridDim.x * blockDim.x) {
+        const int k = (int)(te / NM) * every;
+        const long long at = te % NM, t = k * NM + at;
+        const double dof = dofs[k], z = zq[at];
+        double ls = 0.0;
+        if (!isinf(dof)) {
+            if (fabs(z) < zr) {
+                const double u = (z + zr) * (0.5 * CHI_CELLS / zr);
+                const int c = min((int)u, CHI_CELLS - 1);
+                const double x = u - c - 0.5;
+                const double* q = coef + ((size_t)k * CHI_CELLS + c) * CHI_NC;
+                ls = q[CHI_D];
+                for (int i = CHI_D - 1; i >= 0; --i) ls = fma(ls, x, q[i]);
+            } else {  // as chi_table_kernel
+                const int i = (int)(at % lat.N), m = (int)(at / lat.N);
+                double x = (double)(((long long)i * lat.z[0]) % lat.N) / (double)lat.N + shf[m * CF_MAXDIM];
+                if (x >= 1.0) x -= 1.0;
+                const double wc = fabs(2.0 * x - 1.0);
+                ls = 0.5 * log(cf_chi2_quantile(1.0 - wc, wc, dof, cst[k * CST_STRIDE + CST_LGA], 1e-9) / dof);
+            }
+        }
+        const double s = exp(ls);
+        t64[t] = s;
+        t32[t] = (float)s;
+        if (l64) {  // log(s^2) (exact E[log W])
+            l64[t] = 2.0 * ls;
+            l32[t] = (float)(2.0 * ls);
+        }
+    }
+}
+
 // Degrees of freedom and T_1/T_2 constants for every table index t:
 // E-step tables t = 3h + j have dof nu_h + p + j (j = 0: T_q and T_{q-2},
 // j = 1: T_{q-1}, j = 2: T_q at nu+p+2); with F == nullptr the dofs are
@@ -285,13 +378,6 @@ __global__ void narrow_kernel(const double* __restrict__ src, Dims D, float* __r
 // changes only.  Blocks of 16 cells (blockIdx.x) of table 4h + e (blockIdx.y); a thread per
 // node, then per coefficient.
 constexpr int H1_TC = 16;  // cells per block
-__constant__ double h1_cheb[H1_NC][H1_NC] = {  // powers of x in T_n(x)
-    {1, 0, 0, 0, 0, 0, 0, 0, 0, 0},       {0, 1, 0, 0, 0, 0, 0, 0, 0, 0},
-    {-1, 0, 2, 0, 0, 0, 0, 0, 0, 0},      {0, -3, 0, 4, 0, 0, 0, 0, 0, 0},
-    {1, 0, -8, 0, 8, 0, 0, 0, 0, 0},      {0, 5, 0, -20, 0, 16, 0, 0, 0, 0},
-    {-1, 0, 18, 0, -48, 0, 32, 0, 0, 0},  {0, -7, 0, 56, 0, -112, 0, 64, 0, 0},
-    {1, 0, -32, 0, 160, 0, -256, 0, 128, 0}, {0, 9, 0, -120, 0, 432, 0, -576, 0, 256}};
-
 // H(sigma) at dof v, C = cf_t_const(v)
 static __device__ double h1_value(double sg, double v, double C)
 {
