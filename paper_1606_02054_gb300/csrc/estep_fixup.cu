@@ -11,39 +11,26 @@
 // pairs are therefore cut into tasks, a warp each: an integral of dimension >= 3 into its
 // shifts and those into parts of the points, a lower one whole.  The task sums go to
 // a buffer; the warp that finishes a pair's last task adds them in their order (the
-// same bits whichever warp it is) and assembles the pair.  Longer lists fill the GPU with a
-// warp per pair (FIX_CAP = 1024 pairs are 7 warps per SM).  Fix-up of one E-step on a GB300,
-// parameters with strongly skewed components: p = q = g = 4, n = 200,000, single pass
-// 12.2 -> 4.3 ms; the same with recursion moments, n = 20,000, 26.9 -> 2.0 ms; p = q = g = 6,
-// n = 50,000, single pass 37.9 -> 18.4 ms (there the FP64 pipe is busy: the pass of alpha_s
-// no longer runs twice).
+// same bits whichever warp it is) and assembles the pair.  Longer lists fill the GPU by
+// themselves (FIX_CAP = 1024 pairs are 7 warps per SM): a warp takes a pair and runs its tasks
+// in turn, with a buffer of its own.  Phi and its inverse come from tables (ncdf_tab): the FP64
+// pipe is what a list of hundreds of pairs waits for.  Fix-up of one E-step on a GB300,
+// parameters with strongly skewed components (a warp per pair -> tasks -> tasks and tables):
+// p = q = g = 4, n = 200,000, single pass 12.2 -> 4.3 -> 3.4 ms; the same with recursion
+// moments, n = 20,000, 26.9 -> 2.0 -> 1.7 ms; p = q = g = 6, n = 50,000, single pass
+// 37.9 -> 18.4 -> 11.5 ms.
 #include "estep_common.cuh"
 
-// T_k(bt; 0, corr(Lc Lc^T), nu) in FP64, warp-cooperative; chi = table of this dof.
-__device__ double tk_fp64(int k, const double* bt, const double* Lc, double nu, const double* chi,
-                          const EstepArgs& a, int lane, double* se)
+// T_k(bt; 0, corr(Lc Lc^T), nu), k <= 2, in FP64, warp-cooperative
+__device__ double tk_fp64(int k, const double* bt, const double* Lc, double nu, const EstepArgs& a, int lane)
 {
-    if (se) *se = 0.0;
-    switch (k) {
-    case 0: return 1.0;
-    case 1: return isinf(nu) ? normcdf(bt[0]) : t1cdf_dev<double>(bt[0], nu, t1_lgb(nu));
-    case 2: {
-        const double rho = Lc[2];
-        if (isinf(nu))
-            return phi2_warp<double>(bt[0], bt[1], rho, a.t2n, a.glx64, a.glw64, lane);
-        return t2cdf_warp<double>(bt[0], bt[1], rho, nu, (1.0 - rho) * (1.0 + rho),
-                                  bt[0] * (rho > 0.0 ? rho : -rho) - (rho > 0.0 ? bt[1] : -bt[1]),
-                                  t1_lgb(nu), t1_lgb(nu + 1.0),
-                                  exp(lgamma(0.5 * (nu + 1.0)) - lgamma(0.5 * nu)) / sqrt(CF_PI),
-                                  a.t2n, a.glx64, a.glw64, a.t2n, a.glx64, a.glw64, lane);
-    }
-    case 3: return tk_lattice_warp<double, 3>(bt, Lc, chi, a.shf64, a.lat, lane, se);
-    case 4: return tk_lattice_warp<double, 4>(bt, Lc, chi, a.shf64, a.lat, lane, se);
-    case 5: return tk_lattice_warp<double, 5>(bt, Lc, chi, a.shf64, a.lat, lane, se);
-    case 6: return tk_lattice_warp<double, 6>(bt, Lc, chi, a.shf64, a.lat, lane, se);
-    case 7: return tk_lattice_warp<double, 7>(bt, Lc, chi, a.shf64, a.lat, lane, se);
-    default: return tk_lattice_warp<double, 8>(bt, Lc, chi, a.shf64, a.lat, lane, se);
-    }
+    if (k == 0) return 1.0;
+    if (k == 1) return isinf(nu) ? normcdf(bt[0]) : t1cdf_dev<double>(bt[0], nu, t1_lgb(nu));
+    const double rho = Lc[2];
+    if (isinf(nu)) return phi2_warp<double>(bt[0], bt[1], rho, a.t2n, a.glx64, a.glw64, lane);
+    return t2cdf_warp<double>(bt[0], bt[1], rho, nu, (1.0 - rho) * (1.0 + rho),
+                              bt[0] * (rho > 0.0 ? rho : -rho) - (rho > 0.0 ? bt[1] : -bt[1]), t1_lgb(nu),
+                              t1_lgb(nu + 1.0), cf_t_const(nu), a.t2n, a.glx64, a.glw64, a.t2n, a.glx64, a.glw64, lane);
 }
 
 // Sums over the points i0 <= i < i1 of shift m of the lattice pass of T_K (the points and
@@ -52,7 +39,8 @@ __device__ double tk_fp64(int k, const double* bt, const double* Lc, double nu, 
 // All lanes; lane 0 writes.
 template <int K, bool MOM>
 __device__ void lattice_part(const double* bt, const double* Lc, const EstepArgs& a, const double* crow,
-                             const double* lrow, double rk, int m, int i0, int i1, int lane, double* out)
+                             const double* lrow, double rk, int m, int i0, int i1, int lane, double* out,
+                             const NcdfTables& nq)
 {
     constexpr int K2 = K * (K + 1) / 2, NY = MOM ? K : K - 1;
     double b[K], invd[K], Lf[K][K];
@@ -78,7 +66,7 @@ __device__ void lattice_part(const double* bt, const double* Lc, const EstepArgs
             double t = b[r] * s;
 #pragma unroll
             for (int l = 0; l < r; ++l) t -= Lf[r][l] * y[l];
-            const double e = normcdf(t * invd[r]);
+            const double e = ncdf_tab(t * invd[r], nq);
             f *= e;
             if (r < NY) {
                 double x = (double)(((long long)i * a.lat.z[r + 1]) % N) * invN + a.shf64[m * CF_MAXDIM + r + 1];
@@ -86,7 +74,7 @@ __device__ void lattice_part(const double* bt, const double* Lc, const EstepArgs
                 double v = (1.0 - fabs(2.0 * x - 1.0)) * e;
                 v = v < Lim<double>::vmin() ? Lim<double>::vmin() : v;
                 v = v > Lim<double>::one_minus_ulp() ? Lim<double>::one_minus_ulp() : v;
-                y[r] = normcdfinv(v);
+                y[r] = ncdfinv_tab(v, nq);
             }
             if (e <= Lim<double>::tiny()) f = 0.0;
         }
@@ -125,15 +113,16 @@ __device__ void lattice_part(const double* bt, const double* Lc, const EstepArgs
 
 template <bool MOM>
 __device__ void lattice_part_k(int k, const double* bt, const double* Lc, const EstepArgs& a, const double* crow,
-                               const double* lrow, double rk, int m, int i0, int i1, int lane, double* out)
+                               const double* lrow, double rk, int m, int i0, int i1, int lane, double* out,
+                               const NcdfTables& nq)
 {
     switch (k) {
-    case 3: lattice_part<3, MOM>(bt, Lc, a, crow, lrow, rk, m, i0, i1, lane, out); break;
-    case 4: lattice_part<4, MOM>(bt, Lc, a, crow, lrow, rk, m, i0, i1, lane, out); break;
-    case 5: lattice_part<5, MOM>(bt, Lc, a, crow, lrow, rk, m, i0, i1, lane, out); break;
-    case 6: lattice_part<6, MOM>(bt, Lc, a, crow, lrow, rk, m, i0, i1, lane, out); break;
-    case 7: lattice_part<7, MOM>(bt, Lc, a, crow, lrow, rk, m, i0, i1, lane, out); break;
-    default: lattice_part<8, MOM>(bt, Lc, a, crow, lrow, rk, m, i0, i1, lane, out); break;
+    case 3: lattice_part<3, MOM>(bt, Lc, a, crow, lrow, rk, m, i0, i1, lane, out, nq); break;
+    case 4: lattice_part<4, MOM>(bt, Lc, a, crow, lrow, rk, m, i0, i1, lane, out, nq); break;
+    case 5: lattice_part<5, MOM>(bt, Lc, a, crow, lrow, rk, m, i0, i1, lane, out, nq); break;
+    case 6: lattice_part<6, MOM>(bt, Lc, a, crow, lrow, rk, m, i0, i1, lane, out, nq); break;
+    case 7: lattice_part<7, MOM>(bt, Lc, a, crow, lrow, rk, m, i0, i1, lane, out, nq); break;
+    default: lattice_part<8, MOM>(bt, Lc, a, crow, lrow, rk, m, i0, i1, lane, out, nq); break;
     }
 }
 
@@ -177,7 +166,8 @@ __device__ void fix_store(const EstepArgs& a, long long pid, const PairOut& o, d
 }
 
 // Task t of pair number i of the list (fix_tasks): its sums into the pair's buffer.
-__device__ void fix_task(const EstepArgs& a, const FixArgs& x, long long pid, int t, int lane, double* out)
+__device__ void fix_task(const EstepArgs& a, const FixArgs& x, long long pid, int t, int lane, double* out,
+                         const NcdfTables& nq)
 {
     const int p = a.D.p, q = a.D.q, h = (int)(pid / a.D.n);
     const long long j = pid - (long long)h * a.D.n;
@@ -195,7 +185,7 @@ __device__ void fix_task(const EstepArgs& a, const FixArgs& x, long long pid, in
     fix_integral(a, F, c, d, n, k, dof, tab, fac, bt);
     const double* chi = a.chi64 + (size_t)(3 * h + tab) * NM;
     if (k < 3) {
-        const double v = tk_fp64(k, bt, F + fac, dof, chi, a, lane, nullptr);
+        const double v = tk_fp64(k, bt, F + fac, dof, a, lane);
         if (lane == 0) out[0] = v;
         return;
     }
@@ -205,9 +195,9 @@ __device__ void fix_task(const EstepArgs& a, const FixArgs& x, long long pid, in
     if (a.single_pass && !a.density_only) {
         const double* lrow = a.lchi64 ? a.lchi64 + (size_t)(3 * h) * NM + (size_t)m * a.lat.N : nullptr;
         const double rk = isinf(dof) ? 1.0 : sqrt((dof + 2.0) / dof);
-        lattice_part_k<true>(k, bt, F + fac, a, crow, lrow, rk, m, i0, i1, lane, out);
+        lattice_part_k<true>(k, bt, F + fac, a, crow, lrow, rk, m, i0, i1, lane, out, nq);
     } else {
-        lattice_part_k<false>(k, bt, F + fac, a, crow, nullptr, 1.0, m, i0, i1, lane, out);
+        lattice_part_k<false>(k, bt, F + fac, a, crow, nullptr, 1.0, m, i0, i1, lane, out, nq);
     }
 }
 
@@ -291,20 +281,22 @@ __device__ void fix_assemble(const EstepArgs& a, const FixArgs& x, long long pid
 
 __global__ void __launch_bounds__(128) fixup_kernel(EstepArgs a, FixArgs x, const int* count, const int* list)
 {
+    __shared__ NcdfTables nq;
+    __shared__ double slot[4][CF_MAXQ + CF_MAXQ * (CF_MAXQ + 1) / 2 + 3 + CF_MAXSHIFT];
+    static_assert(sizeof(slot) >= (NCDF_CELLS + 4) * H1_NC * sizeof(double), "scratch of ncdf_tables_init");
+    const int cnt = *count;
+    if (cnt == 0) return;
     const int lane = threadIdx.x & (CF_WARP - 1);
     const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int nwarps = (gridDim.x * blockDim.x) >> 5;
-    const int p = a.D.p, q = a.D.q, q1 = q - 1, q2 = q - 2;
-    const int cnt = *count;
-    const size_t NM = (size_t)a.lat.N * a.lat.M;
-    __shared__ double slot[4][CF_MAXQ + CF_MAXQ * (CF_MAXQ + 1) / 2 + 3 + CF_MAXSHIFT];
-    double* acc = slot[threadIdx.x >> 5];
+    double* sm = slot[threadIdx.x >> 5];
+    ncdf_tables_init(nq, &slot[0][0]);
     if (cnt <= x.cap) {
         const long long total = (long long)cnt * x.ntask;
         for (long long t = warp; t < total; t += nwarps) {
             const int i = (int)(t / x.ntask), k = (int)(t % x.ntask);
             double* part = x.part + (size_t)i * x.ntask * x.nv;
-            fix_task(a, x, list[i], k, lane, part + (size_t)k * x.nv);
+            fix_task(a, x, list[i], k, lane, part + (size_t)k * x.nv, nq);
             int last = 0;
             if (lane == 0) {
                 __threadfence();
@@ -313,62 +305,20 @@ __global__ void __launch_bounds__(128) fixup_kernel(EstepArgs a, FixArgs x, cons
             last = __shfl_sync(CF_FULL, last, 0);
             if (!last) continue;
             __threadfence();
-            fix_assemble(a, x, list[i], part, lane, acc);
+            fix_assemble(a, x, list[i], part, lane, sm);
             if (lane == 0) x.done[i] = 0;  // ready for the next E-step
         }
         return;
     }
-    for (int i = warp; i < cnt; i += nwarps) {
-        const long long pid = list[i];
-        const int h = (int)(pid / a.D.n);
-        const long long j = pid - (long long)h * a.D.n;
-        const double* F = a.F + (size_t)h * a.Ly.stride;
-        const double* chi = a.chi64 + (size_t)(3 * h) * NM;
-        const double nu1 = F[a.Ly.scal + SC_NU] + p;
-        double c[CF_MAXQ], d, logtp, bt[CF_MAXQ], se = 0.0;
-        pair_whiten(F, a.Ly, p, q, a.y + (size_t)j * p, &d, c, &logtp);
-        limits_l0(F, a.Ly, p, q, c, d, 0, bt);
-        const double alpha_s = tk_fp64(q, bt, F + fac_l0(a.Ly), nu1, chi, a, lane, &se);
-        double alpha = 0.0, tq1[CF_MAXQ], tq2[CF_MAXQ * CF_MAXQ];
-        if (a.single_pass && !a.density_only) {
-            double m[CF_MAXQ + CF_MAXQ * (CF_MAXQ + 1) / 2];
-            // the pass of alpha_s (bt still holds its limits) weighted to dof nu+p+2
-            const double* Lq = F + fac_l0(a.Ly);
-            const double rk = isinf(nu1) ? 1.0 : sqrt((nu1 + 2.0) / nu1);
-            double as = 0.0, sej = 0.0, lw = NAN;
-            const double* lchi = a.lchi64 ? a.lchi64 + (size_t)(3 * h) * NM : nullptr;
-            double* lwp = lchi ? &lw : nullptr;
-            switch (q) {
-            case 3: alpha = tk_lattice_mom_warp<double, 3>(bt, Lq, chi, a.shf64, a.lat, lane, acc, rk, &as, &sej, lchi, lwp); break;
-            case 4: alpha = tk_lattice_mom_warp<double, 4>(bt, Lq, chi, a.shf64, a.lat, lane, acc, rk, &as, &sej, lchi, lwp); break;
-            case 5: alpha = tk_lattice_mom_warp<double, 5>(bt, Lq, chi, a.shf64, a.lat, lane, acc, rk, &as, &sej, lchi, lwp); break;
-            case 6: alpha = tk_lattice_mom_warp<double, 6>(bt, Lq, chi, a.shf64, a.lat, lane, acc, rk, &as, &sej, lchi, lwp); break;
-            case 7: alpha = tk_lattice_mom_warp<double, 7>(bt, Lq, chi, a.shf64, a.lat, lane, acc, rk, &as, &sej, lchi, lwp); break;
-            default: alpha = tk_lattice_mom_warp<double, 8>(bt, Lq, chi, a.shf64, a.lat, lane, acc, rk, &as, &sej, lchi, lwp); break;
-            }
-            for (int k = 0; k < q + q * (q + 1) / 2; ++k) m[k] = acc[1 + k];
-            __syncwarp();
-            PairOut o;
-            pair_assemble_sp(F, a.Ly, p, q, c, d, logtp, alpha_s, alpha, m, o, lw);
-            if (lane == 0) fix_store(a, pid, o, se);
-            continue;
-        }
-        if (!a.density_only) {
-            limits_l0(F, a.Ly, p, q, c, d, 1, bt);
-            alpha = tk_fp64(q, bt, F + fac_l0(a.Ly), nu1 + 2.0, chi + 2 * NM, a, lane, nullptr);
-            for (int r = 0; r < q && q1 > 0; ++r) {
-                limits_l1(F, a.Ly, p, q, c, d, r, bt);
-                tq1[r] = tk_fp64(q1, bt, F + fac_l1(a.Ly, q, r), nu1 + 1.0, chi + NM, a, lane, nullptr);
-                for (int s = 0; s < q1 && q2 > 0; ++s) {
-                    limits_l2(F, a.Ly, p, q, c, d, r, s, bt);
-                    tq2[r * q1 + s] = tk_fp64(q2, bt, F + fac_l2(a.Ly, q, r, s), nu1, chi, a, lane, nullptr);
-                }
-            }
-        }
-        PairOut o;
-        pair_assemble(F, a.Ly, p, q, c, d, logtp, alpha_s, alpha, tq1, tq2, a.density_only,
-                      a.cst64 + (size_t)(3 * h) * CST_STRIDE, o);
-        if (lane == 0) fix_store(a, pid, o, se);
+    // a warp per pair, its tasks in turn into a buffer of its own
+    const int use = nwarps < x.cap ? nwarps : x.cap;
+    if (warp >= use) return;
+    double* part = x.part + (size_t)warp * x.ntask * x.nv;
+    for (int i = warp; i < cnt; i += use) {
+        for (int k = 0; k < x.ntask; ++k) fix_task(a, x, list[i], k, lane, part + (size_t)k * x.nv, nq);
+        __syncwarp();
+        fix_assemble(a, x, list[i], part, lane, sm);
+        __syncwarp();  // part is reused
     }
 }
 
