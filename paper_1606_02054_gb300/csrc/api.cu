@@ -123,7 +123,7 @@ struct cfust_ctx {
     // whole-fit CUDA graph (cfust_fit_batch): captured on gst, cached per (max_iter, tol, flags)
     bool capturing = false;
     cudaStream_t gst = nullptr;
-    // the T_1 tables are built on a side stream while the plan runs: forked after the dof
+    // the T_1 (H) tables are built on a side stream while the plan runs: forked after the dof
     // constants, joined before the first kernel that reads them (t1_pending in between)
     cudaStream_t st2 = nullptr;
     cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
