@@ -284,18 +284,52 @@ __global__ void __launch_bounds__(128) combine_mixed_kernel(CombineArgs a)
     }
 }
 
+// A pair at q = 2 by the general assembly with the level-1 T_1 from the continued fraction: the
+// components whose level-1 dof nu + p + 1 is above H1_DOF_MAX (no FP64 table of H; the branch is
+// one per component).  p = 16, g = 8, n = 20,000, nu = 300 on a GB300: combine 1.01 ms, against
+// 2.12 + 0.23 ms by level-1 T_1 records and the general combine.  A function of its own, so that the
+// kernel below runs the other components at 5 blocks an SM without spills (1.46 ms at
+// n = 200,000, as without the branch; inlined registers would leave 4: 5 % at n = 20,000).
+static __device__ __noinline__ void combine_q2_general(const CombineArgs& a, long long pid)
+{
+    const int h = (int)(pid / a.D.n), p = a.D.p;
+    const double* F = a.F + (size_t)h * a.Ly.stride;
+    const double* cst = a.cst64 + (size_t)(3 * h) * CST_STRIDE;
+    const double nu2 = F[a.Ly.scal + SC_NU] + p + 1;
+    const double d = a.pd[2 * pid], c[2] = {a.pc[2 * pid], a.pc[2 * pid + 1]};
+    double tq1[2];
+    for (int r = 0; r < 2; ++r) {
+        double bt[1];
+        limits_l1(F, a.Ly, p, 2, c, d, r, bt);
+        tq1[r] = t1cdf_dev<double>(bt[0], nu2, cst[CST_STRIDE + CST_LGB]);
+    }
+    PairOut o;
+    pair_assemble(F, a.Ly, p, 2, c, d, a.pd[2 * pid + 1], a.L0.res[2 * pid], a.L0.res[2 * pid + 1], tq1, nullptr, 0, cst, o);
+    a.logf[pid] = o.logf;
+    if (a.se) a.se[pid] = 0.0;  // quadrature
+    if (!(o.logf < INFINITY)) atomicOr(a.flags, KF_NAN);  // NaN or +inf; -inf is a null pair
+    a.u[pid] = o.u;
+    a.elogu[pid] = o.elogu;
+    for (int k = 0; k < 2; ++k) a.eu[2 * pid + k] = o.eu[k];
+    for (int k = 0; k < 4; ++k) a.euu[4 * pid + k] = o.euu[k];
+}
+
 // FP64 and plain FP32 forms at q = 2 with the level-1 T_1 inside the assembly (finite nu): H from
-// the FP64 tables, or in the plain FP32 form from the FP32 ones.  Bound by the FP64 pipe; p = 16,
-// g = 8, n = 200,000 on a GB300: 2.16 -> 1.38 ms (541 FP64 slots
+// the FP64 tables (dof nu + p + 1 <= H1_DOF_MAX), or in the plain FP32 form from the FP32 ones.
+// Bound by the FP64 pipe; p = 16, g = 8, n = 200,000 on a GB300: 2.16 -> 1.38 ms (541 FP64 slots
 // a pair), with the level-1 records' plan (1.26 -> 0.91 ms) and launch gone.
 template <bool F32>
-__global__ void __launch_bounds__(128) combine_q2_kernel(CombineArgs a)
+__global__ void __launch_bounds__(128, 5) combine_q2_kernel(const __grid_constant__ CombineArgs a)
 {
     const long long np = a.D.n * a.D.g;
     for (long long pid = blockIdx.x * (long long)blockDim.x + threadIdx.x; pid < np;
          pid += (long long)gridDim.x * blockDim.x) {
         const int h = (int)(pid / a.D.n);
         const double* F = a.F + (size_t)h * a.Ly.stride;
+        if (!F32 && !(F[a.Ly.scal + SC_NU] + a.D.p + 1 <= H1_DOF_MAX)) {
+            combine_q2_general(a, pid);
+            continue;
+        }
         const double2 dl = reinterpret_cast<const double2*>(a.pd)[pid];
         const double2 c2 = reinterpret_cast<const double2*>(a.pc)[pid];
         const double2 al = reinterpret_cast<const double2*>(a.L0.res)[pid];
