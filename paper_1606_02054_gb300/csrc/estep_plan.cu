@@ -161,7 +161,7 @@ __global__ void __launch_bounds__(128) plan_kernel(PlanArgs a)
         }
         double bt[CF_MAXQ];
         double f = 0.0;
-        if (Q == 2) f = sqrt(nu1 / (F[a.Ly.scal + SC_NU] + d));
+        if (Q == 2) f = isinf(nu1) ? 1.0 : sqrt(nu1 / (F[a.Ly.scal + SC_NU] + d));
         for (int w = 0; w < (Q != 2 && a.only_l1 ? 0 : m0); ++w) {
             const long long rec = pid * m0 + w;
             if (Q == 2) {
@@ -285,8 +285,8 @@ __global__ void __launch_bounds__(128) combine_mixed_kernel(CombineArgs a)
 }
 
 // A pair at q = 2 by the general assembly with the level-1 T_1 from the continued fraction: the
-// components whose level-1 dof nu + p + 1 is above H1_DOF_MAX (no FP64 table of H; the branch is
-// one per component).  p = 16, g = 8, n = 20,000, nu = 300 on a GB300: combine 1.01 ms, against
+// components whose level-1 dof nu + p + 1 is above H1_DOF_MAX (no FP64 table of H) or, in both
+// forms, infinite (the normal limit: Phi).  The branch is one per component.  p = 16, g = 8, n = 20,000, nu = 300 on a GB300: combine 1.01 ms, against
 // 2.12 + 0.23 ms by level-1 T_1 records and the general combine.  A function of its own, so that the
 // kernel below runs the other components at 5 blocks an SM without spills (1.46 ms at
 // n = 200,000, as without the branch; inlined registers would leave 4: 5 % at n = 20,000).
@@ -301,7 +301,9 @@ static __device__ __noinline__ void combine_q2_general(const CombineArgs& a, lon
     for (int r = 0; r < 2; ++r) {
         double bt[1];
         limits_l1(F, a.Ly, p, 2, c, d, r, bt);
-        tq1[r] = t1cdf_dev<double>(bt[0], nu2, cst[CST_STRIDE + CST_LGB]);
+        tq1[r] = !isinf(nu2) ? t1cdf_dev<double>(bt[0], nu2, cst[CST_STRIDE + CST_LGB])
+                 : a.fp32    ? (double)m_ncdf((float)bt[0])
+                             : m_ncdf(bt[0]);
     }
     PairOut o;
     pair_assemble(F, a.Ly, p, 2, c, d, a.pd[2 * pid + 1], a.L0.res[2 * pid], a.L0.res[2 * pid + 1], tq1, nullptr, 0, cst, o);
@@ -326,10 +328,6 @@ __global__ void __launch_bounds__(128, 5) combine_q2_kernel(const __grid_constan
          pid += (long long)gridDim.x * blockDim.x) {
         const int h = (int)(pid / a.D.n);
         const double* F = a.F + (size_t)h * a.Ly.stride;
-        if (!F32 && !(F[a.Ly.scal + SC_NU] + a.D.p + 1 <= H1_DOF_MAX)) {
-            combine_q2_general(a, pid);
-            continue;
-        }
         const double2 dl = reinterpret_cast<const double2*>(a.pd)[pid];
         const double2 c2 = reinterpret_cast<const double2*>(a.pc)[pid];
         const double2 al = reinterpret_cast<const double2*>(a.L0.res)[pid];
@@ -338,6 +336,11 @@ __global__ void __launch_bounds__(128, 5) combine_q2_kernel(const __grid_constan
             // outside the FP32 range of the lattice products: redo in FP64
             const int slot = atomicAdd(a.fix_count, 1);
             a.fix_list[slot] = (int)pid;
+            continue;
+        }
+        const double nu = F[a.Ly.scal + SC_NU];
+        if (F32 ? isinf(nu) : !(nu + a.D.p + 1 <= H1_DOF_MAX)) {
+            combine_q2_general(a, pid);
             continue;
         }
         PairOut o;

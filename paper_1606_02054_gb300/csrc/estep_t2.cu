@@ -325,11 +325,15 @@ enum { T2D_ANC0, T2D_PHIS, T2D_L0, T2D_L1, T2D_D0, T2D_SC, T2D_NU, T2D_N };
 constexpr int T2D_NLO = 32;
 __device__ __forceinline__ bool t2_lo_f64(double L, double nu, double zs2) { return L * L * (nu - 1.0 + 0.5 * zs2) <= 90.0; }
 
-// records outside the tables (|rho| = 1, dof above H1_DOF_MAX): the general routine
+// records outside the tables (|rho| = 1, dof above H1_DOF_MAX or infinite): the general routines
 static __device__ __noinline__ double t2_general_f64(const RecSet& r, const IntegArgs& a, long long i, int lane, int* nn)
 {
     const double* c = a.cst64 + r.tab[i] * CST_STRIDE;
     const double h = r.bt[2 * i], k = r.bt[2 * i + 1], rho = a.F[r.fac[i] + 2];
+    if (isinf(r.dof[i])) {
+        *nn = 2 * a.t2n;
+        return phi2_warp<double>(h, k, rho, a.t2n, a.glx64, a.glw64, lane);
+    }
     return t2cdf_warp<double>(h, k, rho, r.dof[i], (1.0 - rho) * (1.0 + rho),
                               h * (rho > 0.0 ? rho : -rho) - (rho > 0.0 ? k : -k), c[CST_LGB], c[CST_LGB1], c[CST_C2],
                               a.t2n, a.glx64, a.glw64, a.t2n, a.glx64, a.glw64, lane, nullptr, 0.0f, nn);

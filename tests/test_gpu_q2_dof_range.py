@@ -1,10 +1,11 @@
 """GPU: FP64 E-steps over the whole range of dofs that a context accepts, where the per-dof
 tables of T_1 and T_2 end (internal.cuh, H1_DOF_MAX = 250): moments and M-step of components
 whose level-1 dof nu + p + 1 lies below and above that limit, nu stepping across it between two
-E-steps, against the oracle.
+E-steps, against the oracle; and components in the normal limit nu = infinity beside finite ones.
 
 Tolerances: those of the parity tests: log f 1e-9, u 1e-8, the moments 1e-7 of the row scale (the
-recursion's formulas cancel in the far tails), one M-step 1e-8.
+recursion's formulas cancel in the far tails), one M-step 1e-8; log-likelihood of the FP32 and mixed
+forms 1e-6.
 """
 import numpy as np
 import pytest
@@ -84,3 +85,21 @@ def test_moments_across_the_table_limit(cf, oracle, p):
     ref, _ = oracle.mstep(y, o, par, nu_max=6000.0, hold=oracle.HOLD_NU)
     for k in ("pi", "mu", "Sigma", "Delta", "nu"):
         assert np.allclose(new[k], ref[k], rtol=1e-8, atol=1e-10), k
+
+
+# one component with the normal limit beside one with a finite nu (nu_max = infinity): the level-0
+# T_2 at q = 2, the level-1 and level-2 ones at q = 3 and 4
+@pytest.mark.parametrize("p,q,precision", [(2, 2, 0), (4, 2, 0), (3, 3, 0), (4, 4, 0), (2, 2, 1), (2, 2, 2)])
+def test_infinite_nu(cf, oracle, p, q, precision):
+    y, par = _inputs(p, q, 41, (np.inf, 7.0))
+    if precision == 2:
+        y = y.astype(np.float32)
+    ctx, qs = _ctx(cf, y, par, nu_max=np.inf, precision=precision)
+    L = cf.cfust_estep(ctx)
+    got = cf.cfust_get_pairs(ctx)
+    o = oracle.estep(y.astype(np.float64), par, oracle.qmc(**qs))
+    assert abs(L - o["loglik"]) <= (1e-6 if precision else 1e-9) * abs(o["loglik"])
+    assert abs(cf.cfust_loglik(ctx) - o["loglik"]) <= (1e-6 if precision else 1e-9) * abs(o["loglik"])
+    if not precision:
+        _check_pairs(got, o)
+    assert np.all(got["u"][0] == 1.0)
