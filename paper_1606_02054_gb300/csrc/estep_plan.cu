@@ -286,10 +286,12 @@ __global__ void __launch_bounds__(128) combine_mixed_kernel(CombineArgs a)
 
 // A pair at q = 2 by the general assembly with the level-1 T_1 from the continued fraction: the
 // components whose level-1 dof nu + p + 1 is above H1_DOF_MAX (no FP64 table of H) or, in both
-// forms, infinite (the normal limit: Phi).  The branch is one per component.  p = 16, g = 8, n = 20,000, nu = 300 on a GB300: combine 1.01 ms, against
-// 2.12 + 0.23 ms by level-1 T_1 records and the general combine.  A function of its own, so that the
-// kernel below runs the other components at 5 blocks an SM without spills (1.46 ms at
-// n = 200,000, as without the branch; inlined registers would leave 4: 5 % at n = 20,000).
+// forms, infinite (the normal limit: Phi), and in the FP64 form pairs whose alpha_s is below
+// 2^-963 = 1e-290 (told by its exponent), where pair_assemble_q2's 1/alpha_s may overflow.
+// p = 16, g = 8, n = 20,000, nu = 300 on a GB300: combine 1.01 ms, against 2.12 + 0.23 ms by
+// level-1 T_1 records and the general combine.  A function of its own, so that the kernel below
+// runs the other components at 5 blocks an SM without spills (1.46 ms at n = 200,000, as
+// without the branch; inlined registers would leave 4: 5 % at n = 20,000).
 static __device__ __noinline__ void combine_q2_general(const CombineArgs& a, long long pid)
 {
     const int h = (int)(pid / a.D.n), p = a.D.p;
@@ -339,7 +341,7 @@ __global__ void __launch_bounds__(128, 5) combine_q2_kernel(const __grid_constan
             continue;
         }
         const double nu = F[a.Ly.scal + SC_NU];
-        if (F32 ? isinf(nu) : !(nu + a.D.p + 1 <= H1_DOF_MAX)) {
+        if (F32 ? isinf(nu) : !(nu + a.D.p + 1 <= H1_DOF_MAX) || __double2hiint(al.x) < (1023 - 963) << 20) {
             combine_q2_general(a, pid);
             continue;
         }

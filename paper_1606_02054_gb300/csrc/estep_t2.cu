@@ -441,9 +441,9 @@ __global__ void __launch_bounds__(T2D_WARPS * CF_WARP, 2) t2_records_h1_kernel(R
                     const double rr = rsqrt(fma(q, q, 1.0));
                     const double H = h1_eval(fabs(q) * rr, t2);
                     if (kd & pc << 4)
-                        s = fma(w * node_exp(num1 * node_log(fabs(sp), nt), nt), 1.0 - node_exp(num1 * node_log(rr, nt), nt) * (rr * rr) * H, s);
+                        s = fma(w * node_exp<true>(num1 * node_log(fabs(sp), nt), nt), 1.0 - node_exp<true>(num1 * node_log(rr, nt), nt) * (rr * rr) * H, s);
                     else
-                        s = fma(w * (rr * rr), node_exp(num1 * node_log(fabs(sp) * rr, nt), nt) * H, s);
+                        s = fma(w * (rr * rr), node_exp<true>(num1 * node_log(fabs(sp) * rr, nt), nt) * H, s);
                 }
                 acc = fma(((kd >> 1) ^ pc) & !(kd & pc << 4) ? -fabs(L) : fabs(L), s, acc);
             }

@@ -1,7 +1,8 @@
 """GPU: FP64 E-steps over the whole range of dofs that a context accepts, where the per-dof
 tables of T_1 and T_2 end (internal.cuh, H1_DOF_MAX = 250): moments and M-step of components
 whose level-1 dof nu + p + 1 lies below and above that limit, nu stepping across it between two
-E-steps, against the oracle; and components in the normal limit nu = infinity beside finite ones.
+E-steps, against the oracle; and components in the normal limit nu = infinity beside finite ones; and T_2
+down to the end of the FP64 range.
 
 Tolerances: those of the parity tests: log f 1e-9, u 1e-8, the moments 1e-7 of the row scale (the
 recursion's formulas cancel in the far tails), one M-step 1e-8; log-likelihood of the FP32 and mixed
@@ -9,6 +10,7 @@ forms 1e-6.
 """
 import numpy as np
 import pytest
+import scipy.stats
 
 from paper_1606_02054_gb300 import synth
 
@@ -103,3 +105,32 @@ def test_infinite_nu(cf, oracle, p, q, precision):
     if not precision:
         _check_pairs(got, o)
     assert np.all(got["u"][0] == 1.0)
+
+
+def test_smallest_t2(cf, oracle):
+    """T_2 between 1e-307 and 1e-290 (the FP64 range ends at 2e-308): log f, u and the moments
+    as elsewhere, no null pair."""
+    p = q = 2
+    par = dict(pi=np.ones(1), mu=np.zeros((1, p)), Sigma=1e-3 * np.eye(p)[None],
+               Delta=np.array([[[1.0, 0.2], [0.3, 1.0]]]), nu=np.array([190.0]))
+    ray = np.concatenate([np.geomspace(5.0, 1e3, 120)[:, None] * np.array([[-1.0, -a]]) for a in (1.0, 0.98)])
+    o = oracle.estep(ray, par, oracle.qmc())
+    Om = par["Sigma"][0] + par["Delta"][0] @ par["Delta"][0].T
+    logtp = scipy.stats.multivariate_t(shape=Om, df=190.0).logpdf(ray)
+    log10 = (o["logf"][0] - logtp - 2.0 * np.log(2.0)) / np.log(10.0)
+    keep = (log10 > -307.0) & (log10 < -290.0)
+    assert keep.sum() >= 20 and np.sum(log10[keep] < -301.0) >= 5, log10
+    y = ray[keep]
+    ctx, qs = _ctx(cf, y, par)
+    L = cf.cfust_estep(ctx)
+    got = cf.cfust_get_pairs(ctx)
+    o = oracle.estep(y, par, oracle.qmc(**qs))
+    assert np.isfinite(L) and np.all(np.isfinite(got["logf"]))
+    _check_pairs(got, o)
+    # subnormal T_2: no null pair, no overflow of 1/T_2
+    y = ray[(log10 > -310.0) & (log10 < -308.0)]
+    assert len(y) >= 5
+    ctx, _ = _ctx(cf, y, par)
+    assert np.isfinite(cf.cfust_estep(ctx))
+    got = cf.cfust_get_pairs(ctx)
+    assert all(np.all(np.isfinite(got[k])) for k in ("logf", "u", "elogu", "eu", "euu"))
