@@ -364,8 +364,12 @@ __device__ __forceinline__ void pair_assemble_q2(const T* F, const Layout& Ly, i
     o.logf = 2 * 0.6931471805599453 + (double)(logtp + m_log(alpha_s));
     const T nu = F[Ly.scal + SC_NU], nu1 = nu + T(p), nud = nu + d;
     const T rs = m_rsqrt(nud), ia = T(1) / alpha_s;
-    const T ik0 = nu1 * (rs * rs);  // (nu+p)/(nu+d)
-    const T u = ik0 * alpha * ia;   // eq (13)
+    // (nu+p)/(nu+d) and eq (13): in FP32 by divisions, whose roundings are half of those of the
+    // products with rs and ia (and as large as T_2's own); in FP64, where a division is 10 operations
+    // and T_2 carries some ten roundings, by those products
+    constexpr bool f32 = sizeof(T) == sizeof(float);
+    const T ik0 = f32 ? nu1 / nud : nu1 * (rs * rs);
+    const T u = f32 ? ik0 * alpha / alpha_s : ik0 * alpha * ia;
     o.u = u;
     o.elogu = u - m_log(T(0.5) * nud) - ik0 + F[Ly.scal + SC_PSI];  // eq (15)
     T xi[2], H[4];
