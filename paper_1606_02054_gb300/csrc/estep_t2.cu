@@ -242,7 +242,7 @@ __global__ void __launch_bounds__(T2P_WARPS * CF_WARP, 4) t2_pieces_kernel(RecSe
                         up2(mul2(pk2(ptx_lg2_approx(D0), ptx_lg2_approx(D1)), pk2(-0.5f * num1)), g0, g1);
                         // H(sigma) as h32_eval
                         up2(fma2(mul2(q & 0x7fffffff7fffffffull, rr2), pk2(scale), pk2(-0.5f)), u0, u1);
-                        const f32x2 u = pk2(fminf(u0, (float)H32_CELLS - 0.51f), fminf(u1, (float)H32_CELLS - 0.51f));
+                        const f32x2 u = pk2(fminf(u0, H32_U_MAX), fminf(u1, H32_U_MAX));
                         const f32x2 mm = add2(u, pk2(12582912.0f));
                         float m0, m1, t0, t1;
                         up2(mm, m0, m1);
