@@ -5,6 +5,9 @@ Bounds:
   h1_eval, h32_eval: exact but for the argument's rounding on tables of a linear function.
   the packed Phi and Phi^-1: those of the scalar forms, whose constants they share
       (tests/test_gpu_special.py); Phi^-1 of p > 1/2 rounds 1 - p once more: 2^-24 over the density there.
+  node_log: half an ulp each for the table's entry, the series' sum and the last addition: 3e-16 of
+      |log v|, and 1e-18 where v is near 1 (entries below 2^-7); node_exp: the reduction, the
+      series and the product: 4e-16 relative; the whole range of exp() with FAR.
   ncdf_tab: the exponential, the polynomial and two products: 1e-15 relative; ncdfinv_tab: 1e-15 of
       max(1, |y|) (the quotient and the difference of Mills ratios of at most 1/2, times sqrt(2 pi)).
 """
@@ -41,7 +44,8 @@ __global__ void __launch_bounds__(128) f64_kernel(int fn, int n, const double* x
     __shared__ double scratch[(NCDF_CELLS + 4) * H1_NC];
     ncdf_tables_init(q, scratch);
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
-        out[i] = fn == 0 ? ncdf_tab(x[i], q) : fn == 1 ? ncdfinv_tab(x[i], q) : h1_eval(x[i], tab);
+        out[i] = fn == 0 ? ncdf_tab(x[i], q) : fn == 1 ? ncdfinv_tab(x[i], q) 
+               : fn == 2 ? h1_eval(x[i], tab) : fn == 3 ? node_log(x[i], q.nt) : node_exp<true>(x[i], q.nt);
 }
 template <typename T> static T* up(const T* h, int n)
 {
@@ -139,6 +143,27 @@ def test_packed_sine(dev):
     err = np.abs(np.abs(dev(2, x).astype(np.float64)) - np.abs(np.sin(x.astype(np.float64))))
     print(f"packed sine: {err.max():.2e}")
     assert err.max() <= 2.5e-7  # the fit 7e-8, the folded angle and the product 1.2e-7
+
+
+def test_node_functions(dev):
+    mp = pytest.importorskip("mpmath")
+    mp.mp.prec = 120
+    rng = np.random.default_rng(3)
+    v = np.concatenate([np.exp(rng.uniform(-700.0, 5.0, 1500)), 1.0 + rng.uniform(-0.5, 0.5, 1500),
+                        1.0 + np.exp(rng.uniform(-40.0, -1.0, 500)), 1.0 - np.exp(rng.uniform(-36.0, -1.0, 500))])
+    ref = [mp.log(mp.mpf(float(t))) for t in v]
+    err = np.array([abs(float(mp.mpf(float(g)) - r)) for g, r in zip(dev(3, v), ref)])
+    lim = 3e-16 * np.abs(np.array([float(r) for r in ref])) + 1e-18
+    print(f"node_log: {np.max(err / lim):.2f} of the bound")
+    assert np.all(err <= lim)
+    x = np.concatenate([-rng.uniform(0.0, 708.0, 3000), -np.exp(rng.uniform(-40.0, 3.0, 1000)), [0.0, -689.9999, -690.0, -690.0001]])
+    ref = [mp.exp(mp.mpf(float(t))) for t in x]
+    err = np.array([abs(float(mp.mpf(float(g)) / r - 1)) for g, r in zip(dev(4, x), ref)])
+    print(f"node_exp: worst {err.max():.2e}")
+    assert err.max() <= 4e-16
+    far = dev(4, np.array([-709.5, -740.0, -746.0, -1e300, -np.inf, np.nan]))
+    assert np.allclose(far[:2], np.exp([-709.5, -740.0]), rtol=1e-12, atol=5e-324)
+    assert np.all(far[2:5] == 0.0) and np.isnan(far[5])
 
 
 def test_tabulated_phi(dev):
