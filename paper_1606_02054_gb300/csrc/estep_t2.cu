@@ -72,8 +72,11 @@ constexpr int T2P_NK = T2_LO_NCLS + 2, T2P_KN = T2_LO_NCLS, T2P_KG = T2_LO_NCLS 
 // piece: the integrand is sin^(nu-1)(phi) (0 + T) or (1 - T).  A lane takes two neighbouring
 // nodes at a time in packed FP32.  The kernel was bound by instruction issue: 77 instructions a
 // node (two folded sines, two lg2, two ex2, a Hermite interpolation) are about 40, and a record's set-up
-// takes two arctangents (cf_atan2_f32) instead of three from the library.
-// p = 16, q = 2, g = 8, n = 2,000,000 (3.2e7 records, 25 nodes each) on a GB300: 2.66 -> 2.1 ms;
+// takes two arctangents (cf_atan2_f32) instead of three from the library.  The set-up keeps full
+// FP32 precision (Newton steps, sqrtf, remainders; 2.19 -> 2.22 ms): u = alpha / alpha_s is as exact as
+// its two records.
+// p = 16, q = 2, g = 8, n = 2,000,000 (3.2e7 records, 25 nodes each) on a GB300: 2.66 -> 2.1 ms
+// (2.2 at the parameters of the comparison above);
 // a node is 60 cycles of a scheduler (FMA about 40, MUFU 32), a record's set-up, ordering and
 // rounds about 15 nodes' worth.
 template <int L, bool TAB>
@@ -152,11 +155,11 @@ __global__ void __launch_bounds__(T2P_WARPS * CF_WARP, 4) t2_pieces_kernel(RecSe
             const bool lo = a.t2n_lo > 0 && !graded && fabsf(rho) < T2_LO_RHO && nu >= T2_LO_DOF_MIN &&
                             nu <= T2_LO_DOF_MAX;
             // the angles of t2_setup: D = phi_h - phi*, and phi* or phi_h as the pieces' anchor
-            const float sg = rho > 0.0f ? 1.0f : -1.0f, ar = fabsf(rho), sn = sqrt_approx(nu);
+            const float sg = rho > 0.0f ? 1.0f : -1.0f, ar = fabsf(rho), sn = sqrt_newton(nu);
             const float D = cf_atan2_f32(sn * cr, fmaf(sg * h, k, ar * nu));
             const bool split = rho != 0.0f && D > 0.0f;
             const float anc = cf_atan2_f32(split ? ar * sn : sn, split ? -sg * k : -h);
-            const float c1 = fmaf(rho * rho, nu, k * k) * ptx_rcp_approx(omr2 * nu);  // zs^2 / (nu + 1)
+            const float c1 = fmaf(rho * rho, nu, k * k) * rcp_newton(omr2 * nu);  // zs^2 / (nu + 1)
             np[m] = split ? 2 : 1;
             kind[m][0] = graded ? T2P_KG : lo ? t2_lo_class(anc, nu, c1 * (nu + 1.0f)) : T2P_KN;
             kind[m][1] = graded ? T2P_KG : lo ? t2_lo_class(D, nu, c1 * (nu + 1.0f)) : T2P_KN;
@@ -164,7 +167,7 @@ __global__ void __launch_bounds__(T2P_WARPS * CF_WARP, 4) t2_pieces_kernel(RecSe
             Rf[T2F_ANC][rr] = anc;
             Rf[T2F_L0][rr] = -anc; Rf[T2F_L1][rr] = D;
             Rf[T2F_D0][rr] = split ? 0.0f : D;
-            Rf[T2F_SC][rr] = sqrt_approx(c1);
+            Rf[T2F_SC][rr] = sqrtf(c1);
             Rf[T2F_NU][rr] = nu; Rf[T2F_LGB1][rr] = c[CST_LGB1];
             // z > 0 on the first piece: bit 0 (the second piece's sign is the opposite)
             const bool pos0 = rho == 0.0f ? k > 0.0f : sg > 0.0f;

@@ -16,7 +16,7 @@ mapped variable t in [-1, 1]:
       x = log2(-log2 pm) in [0, 7],  Phi^-1(pm) = x Q(t), t = affine(x)
       (the factor x makes Phi^-1(1/2) = 0 exactly);  Phi^-1(p) = -x Q for p > 1/2.
       The start of the FP64 inverse (ncdfinv_tab): x in [0, 10], degree 9.
-  atan(a), 0 <= a <= 1:  a R(a^2), R fitted on [0, 1] (relative error of atan(a)/a)
+  atan(a), 0 <= a <= 1:  a + a^3 S(a^2), S fitted on [0, 1] (error relative to atan)
       (cf_atan2_f32 folds the other octants onto it).
   sin(x), |x| <= pi:  r = |x| folded to [0, pi/2] (pi - |x| beyond pi/2),
       sin(r) = r S(r^2) with S fitted on [0, (pi/2)^2] (relative error of sin/r),
@@ -77,11 +77,16 @@ def fit_sin(deg=4):
     return coef, err
 
 
-def fit_atan(deg=8):
-    a = np.linspace(1e-6, 1.0, 400001)
-    m, _ = lawson(a * a, np.arctan(a) / a, deg, 0.0, 1.0)
-    coef = sum(c * Pm.Polynomial([-1.0, 2.0]) ** k for k, c in enumerate(m)).coef
-    err = np.abs(Pm.polyval(a * a, coef) / (np.arctan(a) / a) - 1.0).max()
+def fit_atan(deg=7, iters=80):
+    a = np.linspace(1e-3, 1.0, 200001)
+    x = a * a
+    t, y, w = 2.0 * x - 1.0, (np.arctan(a) / a - 1.0) / x, np.ones_like(x)
+    for _ in range(iters):  # as lawson, the error weighted by x: relative to atan
+        c = Ch.chebfit(t, y, deg, w=np.sqrt(w) * x)
+        w = w * (np.abs(Ch.chebval(t, c) - y) * x + 1e-300)
+        w /= w.sum()
+    coef = sum(m * Pm.Polynomial([-1.0, 2.0]) ** k for k, m in enumerate(Ch.cheb2poly(c))).coef
+    err = np.abs(1.0 + x * Pm.polyval(x, coef) - np.arctan(a) / a).max()
     return coef, err
 
 
@@ -102,5 +107,5 @@ if __name__ == "__main__":
     print(f"// sin: max |error| {e:.2e}  (value = r * S(r^2), S in powers of r^2)")
     print("S =", ", ".join(f"{c:.9e}f" for c in coef))
     coef, e = fit_atan()
-    print(f"// atan: max relative |error| {e:.2e}  (value = a * R(a^2), R in powers of a^2)")
-    print("R =", ", ".join(f"{c:.9e}f" for c in coef))
+    print(f"// atan: max relative |error| {e:.2e}  (value = a + a^3 S(a^2), S in powers of a^2)")
+    print("S =", ", ".join(f"{c:.9e}f" for c in coef))

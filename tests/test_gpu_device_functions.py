@@ -2,6 +2,10 @@
 each evaluated on its own through a small library built from the header here.
 
 Bounds:
+  cf_atan2_f32: 2 ulp (the quotient with its remainder 0.5, the series' last operation 0.5, the
+      octant's addition 0.5, the fit 0.13); sqrt_newton, rcp_newton: 0.6 ulp (a Newton step on an
+      approximation good to 2^-22 leaves 2^-44 before the last rounding; sqrt's remainder is 2^-23 of
+      x and has its own 24 bits from x = 2^-100 on).
   h1_eval, h32_eval: exact but for the argument's rounding on tables of a linear function.
   the packed Phi and Phi^-1: those of the scalar forms, whose constants they share
       (tests/test_gpu_special.py); Phi^-1 of p > 1/2 rounds 1 - p once more: 2^-24 over the density there.
@@ -33,8 +37,10 @@ __global__ void f32_kernel(int fn, int n, const float* x, const float* y, float*
             else if (fn == 1) r = ncdfinv2_abs(pk2(x[i], x[i + 1]));
             else r = sin2_signed(pk2(x[i], x[i + 1]));
             up2(r, out[i], out[i + 1]);
-        } else {  // y: the table
-            for (int k = i; k < i + 2; ++k) out[k] = h32_eval(x[k], reinterpret_cast<const float4*>(y), (float)H32_CELLS);
+        } else {
+            for (int k = i; k < i + 2; ++k)
+                out[k] = fn == 3 ? h32_eval(x[k], reinterpret_cast<const float4*>(y), (float)H32_CELLS)  // y: the table
+                       : fn == 4 ? cf_atan2_f32(y[k], x[k]) : fn == 5 ? sqrt_newton(x[k]) : rcp_newton(x[k]);
         }
     }
 }
@@ -100,6 +106,32 @@ def dev(tmp_path_factory):
         return out
 
     return run
+
+
+def _ulps(got, ref):
+    ref32 = np.abs(ref).astype(np.float32)
+    return np.abs(got.astype(np.float64) - ref) / (np.nextafter(ref32, np.float32(np.inf)) - ref32).astype(np.float64)
+
+
+def test_atan2_f32(dev):
+    rng = np.random.default_rng(1)
+    th, m = rng.uniform(-np.pi, np.pi, 1_000_000), np.exp(rng.uniform(-20.0, 20.0, 1_000_000))
+    y, x = (m * np.sin(th)).astype(np.float32), (m * np.cos(th)).astype(np.float32)
+    e = _ulps(dev(4, x, y), np.arctan2(y.astype(np.float64), x.astype(np.float64)))
+    print(f"atan2: worst {e.max():.2f} ulp, rms {np.sqrt(np.mean(e * e)):.3f}")
+    assert e.max() <= 2.0
+    big, inf = 3e38, np.inf
+    x = np.array([0, 0, 0, 1, -1, big, -big, inf, -inf, 3, -3, big], np.float32)
+    y = np.array([0, 1, -1, 0, 0, 1, 1, 2, 2, inf, -inf, big], np.float32)
+    # beyond 2^126 the quotient counts as 0 (no angle of that size occurs)
+    ref = np.arctan2(y.astype(np.float64), x.astype(np.float64))
+    assert np.all(np.abs(dev(4, x, y) - ref)[:-1] <= 3e-7)
+
+
+def test_newton_f32(dev):
+    x = (2.0 ** np.random.default_rng(2).uniform(-100.0, 100.0, 1_000_000)).astype(np.float32)
+    assert _ulps(dev(5, x), np.sqrt(x.astype(np.float64))).max() <= 0.6
+    assert _ulps(dev(6, x), 1.0 / x.astype(np.float64)).max() <= 0.6
 
 
 def test_table_lookup(dev):
