@@ -165,16 +165,26 @@ __device__ void fix_store(const EstepArgs& a, long long pid, const PairOut& o, d
     for (int k = 0; k < q * q; ++k) a.euu[pid * q * q + k] = o.euu[k];
 }
 
-// Task t of pair number i of the list (fix_tasks): its sums into the pair's buffer.
-__device__ void fix_task(const EstepArgs& a, const FixArgs& x, long long pid, int t, int lane, double* out,
-                         const NcdfTables& nq)
+// A listed pair's factors, squared distance, log t_p and limits' vector
+struct FixPair {
+    const double* F;
+    int h;
+    double c[CF_MAXQ], d, logtp;
+};
+__device__ void fix_pair(const EstepArgs& a, long long pid, FixPair& P)
 {
-    const int p = a.D.p, q = a.D.q, h = (int)(pid / a.D.n);
-    const long long j = pid - (long long)h * a.D.n;
-    const double* F = a.F + (size_t)h * a.Ly.stride;
-    const size_t NM = (size_t)a.lat.N * a.lat.M;
-    double c[CF_MAXQ], d, logtp, bt[CF_MAXQ], dof;
-    pair_whiten(F, a.Ly, p, q, a.y + (size_t)j * p, &d, c, &logtp);
+    P.h = (int)(pid / a.D.n);
+    P.F = a.F + (size_t)P.h * a.Ly.stride;
+    pair_whiten(P.F, a.Ly, a.D.p, a.D.q, a.y + (size_t)(pid - (long long)P.h * a.D.n) * a.D.p, &P.d, P.c, &P.logtp);
+}
+
+// Task t of a pair: its sums to out.  LAT: with integrals of dimension >= 3.
+template <bool LAT>
+__device__ void fix_task(const EstepArgs& a, const FixArgs& x, const FixPair& P, int t, int lane, double* out,
+                         const NcdfTables* nq)
+{
+    const int q = a.D.q;
+    double bt[CF_MAXQ], dof;
     // the integral's number: 2 of dimension q, q of q - 1, the rest of q - 2
     int n = 0, k, tab, fac;
     for (;; ++n) {
@@ -182,22 +192,24 @@ __device__ void fix_task(const EstepArgs& a, const FixArgs& x, long long pid, in
         if (t < w) break;
         t -= w;
     }
-    fix_integral(a, F, c, d, n, k, dof, tab, fac, bt);
-    const double* chi = a.chi64 + (size_t)(3 * h + tab) * NM;
-    if (k < 3) {
-        const double v = tk_fp64(k, bt, F + fac, dof, a, lane);
+    fix_integral(a, P.F, P.c, P.d, n, k, dof, tab, fac, bt);
+    if (!LAT || k < 3) {
+        const double v = tk_fp64(k, bt, P.F + fac, dof, a, lane);
         if (lane == 0) out[0] = v;
         return;
     }
-    const int m = t / x.parts, part = t % x.parts;
-    const int i0 = (int)((long long)a.lat.N * part / x.parts), i1 = (int)((long long)a.lat.N * (part + 1) / x.parts);
-    const double* crow = chi + (size_t)m * a.lat.N;
-    if (a.single_pass && !a.density_only) {
-        const double* lrow = a.lchi64 ? a.lchi64 + (size_t)(3 * h) * NM + (size_t)m * a.lat.N : nullptr;
-        const double rk = isinf(dof) ? 1.0 : sqrt((dof + 2.0) / dof);
-        lattice_part_k<true>(k, bt, F + fac, a, crow, lrow, rk, m, i0, i1, lane, out, nq);
-    } else {
-        lattice_part_k<false>(k, bt, F + fac, a, crow, nullptr, 1.0, m, i0, i1, lane, out, nq);
+    if constexpr (LAT) {
+        const size_t NM = (size_t)a.lat.N * a.lat.M;
+        const int m = t / x.parts, part = t % x.parts;
+        const int i0 = (int)((long long)a.lat.N * part / x.parts), i1 = (int)((long long)a.lat.N * (part + 1) / x.parts);
+        const double* crow = a.chi64 + (size_t)(3 * P.h + tab) * NM + (size_t)m * a.lat.N;
+        if (a.single_pass && !a.density_only) {
+            const double* lrow = a.lchi64 ? a.lchi64 + (size_t)(3 * P.h) * NM + (size_t)m * a.lat.N : nullptr;
+            const double rk = isinf(dof) ? 1.0 : sqrt((dof + 2.0) / dof);
+            lattice_part_k<true>(k, bt, P.F + fac, a, crow, lrow, rk, m, i0, i1, lane, out, *nq);
+        } else {
+            lattice_part_k<false>(k, bt, P.F + fac, a, crow, nullptr, 1.0, m, i0, i1, lane, out, *nq);
+        }
     }
 }
 
@@ -221,14 +233,13 @@ __device__ double fix_value(const EstepArgs& a, const FixArgs& x, int k, const d
 }
 
 // The pair from its tasks' sums; all lanes, sm: CF_MAXQ + CF_MAXQ (CF_MAXQ + 1) / 2 + 3 doubles
-__device__ void fix_assemble(const EstepArgs& a, const FixArgs& x, long long pid, const double* part, int lane,
-                             double* sm)
+__device__ void fix_assemble(const EstepArgs& a, const FixArgs& x, long long pid, const FixPair& P, const double* part,
+                             int lane, double* sm)
 {
-    const int p = a.D.p, q = a.D.q, q1 = q - 1, h = (int)(pid / a.D.n);
-    const long long j = pid - (long long)h * a.D.n;
-    const double* F = a.F + (size_t)h * a.Ly.stride;
-    double c[CF_MAXQ], d, logtp, se = 0.0;
-    pair_whiten(F, a.Ly, p, q, a.y + (size_t)j * p, &d, c, &logtp);
+    const int p = a.D.p, q = a.D.q, q1 = q - 1, h = P.h;
+    const double *F = P.F, *c = P.c;
+    const double d = P.d, logtp = P.logtp;
+    double se = 0.0;
     const double alpha_s = fix_value(a, x, q, part, &se);
     PairOut o;
     if (a.single_pass && !a.density_only) {
@@ -279,9 +290,15 @@ __device__ void fix_assemble(const EstepArgs& a, const FixArgs& x, long long pid
     if (lane == 0) fix_store(a, pid, o, se);
 }
 
-__global__ void __launch_bounds__(128) fixup_kernel(EstepArgs a, FixArgs x, const int* count, const int* list)
+// LAT: q >= 3.  At q <= 2 no integral needs the tables of Phi, which take about 50 us to build
+// (longer than a short list), nor the lattice code's registers, and a pair's few values fit in
+// shared memory, so that every warp of a long list has a pair.  One kernel for every q ->
+// without them at q <= 2, normal limit (CFUSN) on a GB300: p = 16, q = 2, g = 4, n = 2000 (a few
+// pairs listed) E-step 104 -> 56 us, density 88 -> 39; g = 8, n = 200,000 (long list) 46.8 -> 23.9 ms,
+// 14.2 -> 8.1 (a warp per pair with all of a pair's integrals in one function: 86, 37 us; 28.3, 8.2 ms).
+template <bool LAT>
+__global__ void __launch_bounds__(128, LAT ? 2 : 4) fixup_kernel(EstepArgs a, FixArgs x, const int* count, const int* list)
 {
-    __shared__ NcdfTables nq;
     __shared__ double slot[4][CF_MAXQ + CF_MAXQ * (CF_MAXQ + 1) / 2 + 3 + CF_MAXSHIFT];
     static_assert(sizeof(slot) >= (NCDF_CELLS + 4) * H1_NC * sizeof(double), "scratch of ncdf_tables_init");
     const int cnt = *count;
@@ -290,13 +307,20 @@ __global__ void __launch_bounds__(128) fixup_kernel(EstepArgs a, FixArgs x, cons
     const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int nwarps = (gridDim.x * blockDim.x) >> 5;
     double* sm = slot[threadIdx.x >> 5];
-    ncdf_tables_init(nq, &slot[0][0]);
+    const NcdfTables* nq = nullptr;
+    if constexpr (LAT) {
+        __shared__ NcdfTables tables;
+        ncdf_tables_init(tables, &slot[0][0]);
+        nq = &tables;
+    }
+    FixPair P;
     if (cnt <= x.cap) {
         const long long total = (long long)cnt * x.ntask;
         for (long long t = warp; t < total; t += nwarps) {
             const int i = (int)(t / x.ntask), k = (int)(t % x.ntask);
             double* part = x.part + (size_t)i * x.ntask * x.nv;
-            fix_task(a, x, list[i], k, lane, part + (size_t)k * x.nv, nq);
+            fix_pair(a, list[i], P);
+            fix_task<LAT>(a, x, P, k, lane, part + (size_t)k * x.nv, nq);
             int last = 0;
             if (lane == 0) {
                 __threadfence();
@@ -305,19 +329,21 @@ __global__ void __launch_bounds__(128) fixup_kernel(EstepArgs a, FixArgs x, cons
             last = __shfl_sync(CF_FULL, last, 0);
             if (!last) continue;
             __threadfence();
-            fix_assemble(a, x, list[i], part, lane, sm);
+            fix_assemble(a, x, list[i], P, part, lane, sm);
             if (lane == 0) x.done[i] = 0;  // ready for the next E-step
         }
         return;
     }
-    // a warp per pair, its tasks in turn into a buffer of its own
-    const int use = nwarps < x.cap ? nwarps : x.cap;
+    // a warp per pair, its tasks in turn into a buffer of its own: shared memory at q <= 2 (2 + 2 q
+    // values), else a pair's place in the sums' buffer
+    const int use = !LAT || nwarps < x.cap ? nwarps : x.cap;
     if (warp >= use) return;
-    double* part = x.part + (size_t)warp * x.ntask * x.nv;
+    double* part = LAT ? x.part + (size_t)warp * x.ntask * x.nv : sm;
     for (int i = warp; i < cnt; i += use) {
-        for (int k = 0; k < x.ntask; ++k) fix_task(a, x, list[i], k, lane, part + (size_t)k * x.nv, nq);
+        fix_pair(a, list[i], P);
+        for (int k = 0; k < x.ntask; ++k) fix_task<LAT>(a, x, P, k, lane, part + (size_t)k * x.nv, nq);
         __syncwarp();
-        fix_assemble(a, x, list[i], part, lane, sm);
+        fix_assemble(a, x, list[i], P, part, lane, sm);
         __syncwarp();  // part is reused
     }
 }
@@ -339,7 +365,8 @@ FixArgs fix_args(int q, int single, int density, const Lattice& lat)
 cudaError_t launch_fixup(const EstepArgs& a, const FixArgs& x, const int* count, const int* list, int nsm,
                          cudaStream_t st, long long* launches)
 {
-    fixup_kernel<<<4 * nsm, 128, 0, st>>>(a, x, count, list);
+    if (a.D.q >= 3) fixup_kernel<true><<<4 * nsm, 128, 0, st>>>(a, x, count, list);
+    else fixup_kernel<false><<<4 * nsm, 128, 0, st>>>(a, x, count, list);
     ++*launches;
     return cudaGetLastError();
 }
