@@ -67,7 +67,7 @@ struct cfust_ctx {
     double* lchi64 = nullptr;  // exact E[log W]: log(s^2) beside the chi tables
     float* lchi32 = nullptr;
     double* shf64 = nullptr;
-    float* shf32 = nullptr;
+    char* consts = nullptr;    // one buffer of the constants below (shf64 to t2n_lo's node sets, fix_done)
     unsigned* latu = nullptr;  // lattice coordinates as 32-bit fractions (IntegArgs::latu)
     float4* wtab = nullptr;  // FP32 single pass: lattice coordinates of every (shift, point)
     double *glx64 = nullptr, *glw64 = nullptr;
@@ -405,12 +405,11 @@ static void free_all(cfust_ctx* c)
 {
     sur_free(c->sur);
     void* bufs[] = {c->y, c->pi, c->mu, c->Sigma, c->Delta, c->nu, c->pi_n, c->mu_n, c->Sigma_n,
-                    c->Delta_n, c->nu_n, c->F, c->dofs, c->cst64, c->cst32, c->chi64, c->chi32, c->shf64, c->shf32, c->wtab,
-                    c->glx64, c->glw64, c->glx32, c->glw32, c->glx32h, c->glw32h, c->glx32l, c->glw32l, c->glx64l, c->glw64l,
+                    c->Delta_n, c->nu_n, c->F, c->dofs, c->cst64, c->cst32, c->chi64, c->chi32, c->consts, c->wtab,
                     c->logf, c->u, c->elogu, c->eu,
                     c->euu, c->se, c->tau, c->partial, c->stats, c->flags, c->comp_status,
-                    c->stage32, c->pd, c->pc, c->fix_count, c->fix_list, c->y32, c->F32, c->pr32, c->pd32, c->pc32, c->res32_l0, c->h32tab, c->h32scale,
-                    c->work_dev, c->seg, c->lchi64, c->lchi32, c->h1tab, c->fix_part, c->fix_done, c->latu, c->chi_z, c->chi_coef};
+                    c->stage32, c->pd, c->pc, c->fix_count, c->fix_list, c->y32, c->F32, c->pr32, c->pd32, c->pc32, c->res32_l0, c->h32tab,
+                    c->work_dev, c->seg, c->lchi64, c->lchi32, c->h1tab, c->fix_part, c->chi_z};
     for (void* b : bufs)
         if (b) cudaFree(b);
     for (RecSet& r : c->rec) {
@@ -551,20 +550,13 @@ extern "C" cfust_status cfust_create(cfust_ctx** out, int p, int q, int g, int64
     ALLOC(chi32, ntab * NM);
     const bool chi_poly = q >= 3 && o.precision != CFUST_PREC_FP64;
     if (chi_poly) {
-        ALLOC(chi_z, NM);
-        ALLOC(chi_coef, (size_t)ntab * 32 * 10);
+        ALLOC(chi_z, NM + (size_t)ntab * 32 * 10);
+        c->chi_coef = c->chi_z + NM;
     }
     if (o.elogw == CFUST_ELOGW_EXACT) {
         ALLOC(lchi64, ntab * NM);
         ALLOC(lchi32, ntab * NM);
     }
-    ALLOC(latu, (size_t)CF_MAXDIM * (33 + o.qmc_shifts));
-    ALLOC(shf64, (size_t)o.qmc_shifts * CF_MAXDIM);
-    ALLOC(shf32, (size_t)o.qmc_shifts * CF_MAXDIM);
-    ALLOC(glx64, c->t2n); ALLOC(glw64, c->t2n); ALLOC(glx32, c->t2n); ALLOC(glw32, c->t2n);
-    ALLOC(glx32h, T2_NH); ALLOC(glw32h, T2_NH);
-    ALLOC(glx32l, T2_LO_TOTAL); ALLOC(glw32l, T2_LO_TOTAL);
-    ALLOC(glx64l, 32); ALLOC(glw64l, 32);
     ALLOC(logf, ng); ALLOC(u, ng); ALLOC(elogu, ng); ALLOC(se, ng); ALLOC(tau, ng);
     ALLOC(eu, ng * q); ALLOC(euu, ng * q * q);
     ALLOC(partial, part);
@@ -589,12 +581,11 @@ extern "C" cfust_status cfust_create(cfust_ctx** out, int p, int q, int g, int64
             per = std::max(per, (size_t)x.ntask * x.nv);
         }
         ALLOC(fix_part, per * c->fix_cap);
-        ALLOC(fix_done, c->fix_cap);
     }
     // T_2 records exist at q = 2 (level 0) and, in the recursion form, at q = 3, 4 (levels 1, 2)
     if (o.precision != CFUST_PREC_FP64 && (q == 2 || (!c->single_pass && (q == 3 || q == 4)))) {
-        ALLOC(h32tab, (size_t)4 * g * H32_CELLS);
-        ALLOC(h32scale, 4 * g);
+        ALLOC(h32tab, (size_t)4 * g * H32_CELLS + g);
+        c->h32scale = reinterpret_cast<float*>(c->h32tab + (size_t)4 * g * H32_CELLS);  // 4 g floats
     }
     if (o.precision == CFUST_PREC_FP64 && o.model == CFUST_MODEL_CFUST &&
         (q == 2 || (!c->single_pass && (q == 3 || q == 4)))) {
@@ -629,13 +620,10 @@ extern "C" cfust_status cfust_create(cfust_ctx** out, int p, int q, int g, int64
     }
     // lattice shifts and Gauss-Legendre nodes
     std::vector<double> s64((size_t)o.qmc_shifts * CF_MAXDIM);
-    std::vector<float> s32(s64.size());
     for (int m = 0; m < o.qmc_shifts; ++m)
         for (int d = 0; d < CF_MAXDIM; ++d) {
             const uint64_t key = o.seed ^ ((uint64_t)(m + 1) << 32) ^ (uint64_t)(d + 1);
             s64[m * CF_MAXDIM + d] = splitmix_u01(key);
-            s32[m * CF_MAXDIM + d] = (float)s64[m * CF_MAXDIM + d];
-            if (s32[m * CF_MAXDIM + d] >= 1.0f) s32[m * CF_MAXDIM + d] = 0.0f;
         }
     std::vector<double> gx, gw;
     gauss_legendre01(c->t2n, gx, gw);
@@ -656,8 +644,8 @@ extern "C" cfust_status cfust_create(cfust_ctx** out, int p, int q, int g, int64
         if (ee != cudaSuccess && s == CFUST_OK)
             s = fail(nullptr, CFUST_ECUDA, std::string("cfust_create: cudaMemcpy: ") + cudaGetErrorString(ee));
     };
-    if (c->fix_done && (e = cudaMemset(c->fix_done, 0, sizeof(int) * c->fix_cap)) != cudaSuccess)
-        s = fail(nullptr, CFUST_ECUDA, std::string("cfust_create: cudaMemset: ") + cudaGetErrorString(e));
+    // the constants: one buffer, one copy (a call of cudaMalloc or cudaMemcpy is about 10 us each,
+    // and there are a dozen of these)
     {
         std::vector<uint32_t> lu((size_t)CF_MAXDIM * (33 + o.qmc_shifts));
         const uint64_t N = (uint64_t)o.qmc_points;
@@ -665,11 +653,39 @@ extern "C" cfust_status cfust_create(cfust_ctx** out, int p, int q, int g, int64
             for (int i = 0; i <= 32; ++i)
                 lu[d * 33 + i] = (uint32_t)((((uint64_t)i * c->lat.z[d] % N << 32) + N / 2) / N);
         for (size_t k = 0; k < s64.size(); ++k) lu[CF_MAXDIM * 33 + k] = (uint32_t)(s64[k] * 4294967296.0);
-        cp(c->latu, lu.data(), sizeof(uint32_t) * lu.size());
+        std::vector<double> gx32n, gw32n;
+        gauss_legendre01(32, gx32n, gw32n);
+        const std::vector<int> zeros(c->fix_cap, 0);
+        std::vector<char> host;
+        std::vector<std::pair<void**, size_t>> at;
+        auto place = [&](auto** ptr, const auto& v) {
+            const size_t bytes = v.size() * sizeof(v[0]);
+            at.emplace_back(reinterpret_cast<void**>(ptr), host.size());
+            host.resize(host.size() + (bytes + 255) / 256 * 256);
+            if (bytes) std::memcpy(host.data() + at.back().second, v.data(), bytes);
+        };
+        place(&c->shf64, s64);
+        place(&c->latu, lu);
+        place(&c->glx64, gx);
+        place(&c->glw64, gw);
+        place(&c->glx64l, gx32n);
+        place(&c->glw64l, gw32n);
+        place(&c->glx32, gx32);
+        place(&c->glw32, gw32);
+        place(&c->glx32h, gxh32);
+        place(&c->glw32h, gwh32);
+        place(&c->glx32l, gxl32);
+        place(&c->glw32l, gwl32);
+        place(&c->fix_done, zeros);
+        if ((e = dalloc(&c->consts, host.size())) != cudaSuccess) {
+            free_all(c);
+            delete c;
+            return fail(nullptr, CFUST_ENOMEM, std::string("cfust_create: cudaMalloc constants: ") + cudaGetErrorString(e));
+        }
+        for (const auto& [ptr, off] : at) *ptr = c->consts + off;
+        cp(c->consts, host.data(), host.size());
     }
-    cp(c->shf64, s64.data(), sizeof(double) * s64.size());
-    cp(c->shf32, s32.data(), sizeof(float) * s32.size());
-    if (chi_poly) {  // before the copies below, which wait for it (legacy stream)
+    if (chi_poly) {
         // the smaller tail of every coordinate 0 is at least pm, so |z| <= sqrt(-2 ln(2 pm))
         double pm = 0.5;
         for (int m = 0; m < o.qmc_shifts; ++m)
@@ -705,20 +721,8 @@ extern "C" cfust_status cfust_create(cfust_ctx** out, int p, int q, int g, int64
         }
         cp(c->wtab, wt.data(), sizeof(float) * wt.size());
     }
-    cp(c->glx64, gx.data(), sizeof(double) * gx.size());
-    {
-        std::vector<double> gx32n, gw32n;
-        gauss_legendre01(32, gx32n, gw32n);
-        cp(c->glx64l, gx32n.data(), sizeof(double) * 32);
-        cp(c->glw64l, gw32n.data(), sizeof(double) * 32);
-    }
-    cp(c->glw64, gw.data(), sizeof(double) * gw.size());
-    cp(c->glx32, gx32.data(), sizeof(float) * gx32.size());
-    cp(c->glw32, gw32.data(), sizeof(float) * gw32.size());
-    cp(c->glx32h, gxh32.data(), sizeof(float) * gxh32.size());
-    cp(c->glw32h, gwh32.data(), sizeof(float) * gwh32.size());
-    cp(c->glx32l, gxl32.data(), sizeof(float) * gxl32.size());
-    cp(c->glw32l, gwl32.data(), sizeof(float) * gwl32.size());
+    if ((e = cudaStreamSynchronize(cudaStreamLegacy)) != cudaSuccess && s == CFUST_OK)  // before any other stream
+        s = fail(nullptr, CFUST_ECUDA, std::string("cfust_create: ") + cudaGetErrorString(e));
     if (s != CFUST_OK) {
         free_all(c);
         delete c;
@@ -906,7 +910,7 @@ static IntegArgs integ_args(const cfust_ctx* c)
     IntegArgs ia;
     ia.cst64 = c->cst64; ia.cst32 = c->cst32;
     ia.F = c->F; ia.lat = c->lat;
-    ia.chi64 = c->chi64; ia.chi32 = c->chi32; ia.shf64 = c->shf64; ia.shf32 = c->shf32;
+    ia.chi64 = c->chi64; ia.chi32 = c->chi32; ia.shf64 = c->shf64;
     ia.glx64 = c->glx64; ia.glw64 = c->glw64; ia.glx32 = c->glx32; ia.glw32 = c->glw32;
     ia.t2n = c->t2n;
     ia.glx32h = c->glx32h; ia.glw32h = c->glw32h;
@@ -1056,7 +1060,7 @@ static cfust_status launch_pairs(cfust_ctx* c, int density_only)
         a.D = c->D; a.Ly = c->Ly; a.lat = c->lat; a.cst64 = c->cst64;
         a.y = c->y; a.F = c->F;
         a.chi64 = c->chi64; a.chi32 = c->chi32;
-        a.shf64 = c->shf64; a.shf32 = c->shf32;
+        a.shf64 = c->shf64;
         a.glx64 = c->glx64; a.glw64 = c->glw64; a.glx32 = c->glx32; a.glw32 = c->glw32;
         a.t2n = c->t2n;
         a.density_only = density_only;
@@ -2028,7 +2032,7 @@ extern "C" cfust_status cfust_tk_eval(cfust_ctx* c, int k, int count, const doub
     auto cleanup = [&]() {
         cudaFree(r.bt); cudaFree(r.fac); cudaFree(r.tab); cudaFree(r.dof); cudaFree(r.res);
         cudaFree(r.se); cudaFree(dF); cudaFree(t64); cudaFree(t32); cudaFree(k64); cudaFree(k32);
-        cudaFree(h32); cudaFree(h32s); cudaFree(r.t2f);
+        cudaFree(h32); cudaFree(r.t2f);
     };
     if ((e = dalloc(&r.bt, bt.size())) != cudaSuccess || (e = dalloc(&r.fac, count)) != cudaSuccess ||
         (e = dalloc(&r.tab, count)) != cudaSuccess || (e = dalloc(&r.dof, count)) != cudaSuccess ||
@@ -2038,12 +2042,12 @@ extern "C" cfust_status cfust_tk_eval(cfust_ctx* c, int k, int count, const doub
         (e = dalloc(&k32, (size_t)count * CST_STRIDE)) != cudaSuccess ||
         (e = dalloc(&t64, lattice ? NM * count : 1)) != cudaSuccess ||
         (e = dalloc(&t32, lattice ? NM * count : 1)) != cudaSuccess ||
-        (e = dalloc(&h32, use_h32 ? (size_t)count * H32_CELLS : 1)) != cudaSuccess ||
-        (e = dalloc(&h32s, use_h32 ? (size_t)count : 1)) != cudaSuccess ||
+        (e = dalloc(&h32, use_h32 ? (size_t)count * H32_CELLS + (count + 3) / 4 : 1)) != cudaSuccess ||
         (k == 2 && c->opts.precision != CFUST_PREC_FP64 && (e = dalloc(&r.t2f, (size_t)2 * count)) != cudaSuccess)) {
         cleanup();
         return fail(c, CFUST_ENOMEM, std::string("cfust_tk_eval: ") + cudaGetErrorString(e));
     }
+    if (use_h32) h32s = reinterpret_cast<float*>(h32 + (size_t)count * H32_CELLS);  // count floats
     do {
         if ((e = cudaMemcpyAsync(r.bt, bt.data(), sizeof(double) * bt.size(), cudaMemcpyHostToDevice, c->st))) break;
         if ((e = cudaMemcpyAsync(r.fac, foff.data(), sizeof(int) * count, cudaMemcpyHostToDevice, c->st))) break;

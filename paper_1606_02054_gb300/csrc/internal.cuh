@@ -170,7 +170,6 @@ struct IntegArgs {
     const double* chi64;   // [(3h + j)][M][N] (or per case for cfust_tk_eval)
     const float* chi32;
     const double* shf64;   // [M][CF_MAXDIM]
-    const float* shf32;
     const double* glx64;   // Gauss-Legendre nodes/weights on [0, 1]
     const double* glw64;
     const float* glx32;
@@ -318,7 +317,6 @@ struct EstepArgs {
     const double* chi64;    // [(3h + k)][M][N]
     const float* chi32;
     const double* shf64;    // [M][CF_MAXDIM]
-    const float* shf32;
     const double* glx64;    // Gauss-Legendre nodes/weights on [0,1]
     const double* glw64;
     const float* glx32;
