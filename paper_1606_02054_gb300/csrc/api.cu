@@ -852,7 +852,7 @@ static cfust_status launch_setup(cfust_ctx* c, int density_only)
     setup_components_kernel<<<c->g, 32, 0, c->st>>>(c->D, c->Ly, c->mu, c->Sigma, c->Delta, c->nu,
                                                  c->F, c->flags);
     LAUNCHED();
-    dof_consts_kernel<<<1, 64, 0, c->st>>>(c->D, c->Ly, c->F, 3 * c->g, c->dofs, c->cst64, c->cst32);
+    dof_consts_kernel<<<1, 256, 0, c->st>>>(c->D, c->Ly, c->F, 3 * c->g, c->dofs, c->cst64, c->cst32);
     LAUNCHED();
     if (c->h32tab || c->h1tab) {
         // tables 4h + e hold H at dof nu_h + p + e: a T_2 record of index 3h + j reads e = j + 1, in FP64
@@ -2061,7 +2061,7 @@ extern "C" cfust_status cfust_tk_eval(cfust_ctx* c, int k, int count, const doub
                 t2_record_f32(bt[2 * i], bt[2 * i + 1], fac[(size_t)i * 4 + 2], dofv[i], &t2f[2 * i]);
             if ((e = cudaMemcpyAsync(r.t2f, t2f.data(), sizeof(float4) * t2f.size(), cudaMemcpyHostToDevice, c->st))) break;
         }
-        dof_consts_kernel<<<(count + 127) / 128, 128, 0, c->st>>>(c->D, c->Ly, nullptr, count, r.dof, k64, k32);
+        dof_consts_kernel<<<(count + 31) / 32, 128, 0, c->st>>>(c->D, c->Ly, nullptr, count, r.dof, k64, k32);
         c->launches++;
         if ((e = cudaGetLastError())) break;
         if (lattice) {

@@ -317,33 +317,48 @@ __global__ void chi_eval_kernel(int ntab, int every, double zr, const double* __
 // E-step tables t = 3h + j have dof nu_h + p + j (j = 0: T_q and T_{q-2},
 // j = 1: T_{q-1}, j = 2: T_q at nu+p+2); with F == nullptr the dofs are
 // already given (cfust_tk_eval, one index per case).
+// Four warps share 32 dofs (a lane each), every warp with some of the constants: a constant is a
+// serial chain of lgamma, exp and sqrt in FP64, and the kernel is as long as its longest warp.
 __global__ void dof_consts_kernel(Dims D, Layout Ly, const double* __restrict__ F, int ndof,
                                   double* dofs, double* c64, float* c32)
 {
-    for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < ndof; t += gridDim.x * blockDim.x) {
+    const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, part = warp & 3;
+    for (int t = (warp >> 2) * 32 + (threadIdx.x & 31); t < ndof; t += gridDim.x * blockDim.x / 4) {
         double v;
         if (F) {
             const int h = t / 3, j = t % 3;
             v = F[(size_t)h * Ly.stride + Ly.scal + SC_NU] + D.p + j;
-            dofs[t] = v;
+            if (part == 0) dofs[t] = v;
         } else {
             v = dofs[t];
         }
-        if (isinf(v)) {  // the normal limit uses none of these constants
-            for (int k = 0; k < CST_STRIDE; ++k) {
-                c64[t * CST_STRIDE + k] = 0.0;
-                c32[t * CST_STRIDE + k] = 0.0f;
-            }
-            continue;
+        const bool fin = !isinf(v);  // the normal limit uses none of these constants: 0
+        auto put = [&](int k, double x) {
+            c64[t * CST_STRIDE + k] = x;
+            c32[t * CST_STRIDE + k] = (float)x;
+        };
+        switch (part) {
+        case 0:
+            put(CST_LGB, fin ? t1_lgb(v) : 0.0);
+            put(CST_LGA, fin ? lgamma(0.5 * v) : 0.0);
+            break;
+        case 1:
+            put(CST_LGB1, fin ? t1_lgb(v + 1.0) : 0.0);
+            put(CST_C2, fin ? cf_t_const(v) : 0.0);
+            break;
+        case 2: {
+            const double lt = fin ? lgamma(0.5 * (v + 1.0)) - lgamma(0.5 * v) - 0.5 * log(v * CF_PI) : 0.0;
+            put(CST_LT1, lt);
+            put(CST_ET1, fin ? exp(lt) * sqrt(v) : 0.0);
+            break;
         }
-        const double lt = lgamma(0.5 * (v + 1.0)) - lgamma(0.5 * v) - 0.5 * log(v * CF_PI);
-        const double ltm = lgamma(0.5 * v) - lgamma(0.5 * (v - 1.0)) - 0.5 * log((v - 1.0) * CF_PI);
-        const double c[CST_STRIDE] = {t1_lgb(v), t1_lgb(v + 1.0),
-                                      cf_t_const(v),
-                                      lt, v > 1.0 ? ltm : 0.0, lgamma(0.5 * v), exp(lt) * sqrt(v), v > 1.0 ? exp(ltm) / sqrt(v - 1.0) : 0.0};
-        for (int k = 0; k < CST_STRIDE; ++k) {
-            c64[t * CST_STRIDE + k] = c[k];
-            c32[t * CST_STRIDE + k] = (float)c[k];
+        default: {
+            const bool ok = fin && v > 1.0;
+            const double ltm = ok ? lgamma(0.5 * v) - lgamma(0.5 * (v - 1.0)) - 0.5 * log((v - 1.0) * CF_PI) : 0.0;
+            put(CST_LT1M, ltm);
+            put(CST_ET1M, ok ? exp(ltm) / sqrt(v - 1.0) : 0.0);
+            break;
+        }
         }
     }
 }
