@@ -23,6 +23,12 @@ This script, in FP64 with numpy/scipy only:
 
 Run:  python fit_t2_classes.py [records]   (prints the bounds and the held-out errors; the
 constants in internal.cuh come from 160,000 training records)
+      python fit_t2_classes.py fp64 [records]
+
+With fp64 it checks the FP64 rule (estep_t2.cu, t2_lo_f64: 32 instead of 64 nodes where
+10 <= nu <= 64, |rho| < 0.9 and L^2 (nu - 1 + 0.5 zs^2) <= 90) in the host's long double (80 bits
+on x86): the error of 32 plain nodes against 220 graded ones, relative to the record's T_2, by
+the rule's score; the worst of the pieces that the rule takes has to stay below 1e-16.
 """
 import sys
 
@@ -142,7 +148,85 @@ def classify(t, bounds):
     return cls
 
 
+LD = np.longdouble
+
+
+def legendre_ld(n):
+    """gauss_legendre01 in long double: Newton steps on P_n from the FP64 nodes."""
+    x = np.polynomial.legendre.leggauss(n)[0].astype(LD)
+    for _ in range(4):
+        p0, p1 = np.ones_like(x), x.copy()
+        for k in range(2, n + 1):
+            p0, p1 = p1, ((2 * k - 1) * x * p1 - (k - 1) * p0) / k
+        dp = n * (x * p1 - p0) / (x * x - 1)
+        x = x - p1 / dp
+    return (x + 1) / 2, 1 / ((1 - x * x) * dp * dp)
+
+
+def log_gamma_ratio(a):
+    """ln Gamma(a + 1/2) - ln Gamma(a): Stirling's series twice from a >= 40 on."""
+    s, a = np.zeros_like(a), a.copy()
+    while (a < 40).any():
+        m = a < 40
+        s, a = np.where(m, s + np.log(a) - np.log(a + LD(0.5)), s), np.where(m, a + 1, a)
+    r = 1 / a
+    c = [-LD(1) / 8, LD(1) / 192, -LD(1) / 640, LD(17) / 14336, -LD(31) / 18432, LD(691) / 180224]
+    return s + LD(0.5) * np.log(a) + r * sum(ck * r ** (2 * k) for k, ck in enumerate(c))
+
+
+def t1_ld(z, v, terms=70):
+    """T_1(z; v) by the continued fraction of I_x(v/2, 1/2), run backwards from a fixed term."""
+    D, a = v + z * z, v / 2
+    y, s2 = v / D, z * z / D
+    low = y < (a + 1) / (a + LD(2.5))
+    A, B, x = np.where(low, a, LD(0.5)), np.where(low, LD(0.5), a), np.where(low, y, s2)
+    p1, p = np.ones_like(x), A + (2 * terms + 1)
+    for m in range(terms, 0, -1):
+        p1 = (A + 2 * m) * p - (A + m) * (A + B + m) * x * p1
+        p = (A + 2 * m - 1) * p1 + m * (B - m) * x * p
+        p1, p = p1 / np.abs(p), np.sign(p)
+    cf = p / (p - (A + B) * x * p1)
+    pre = np.exp(a * np.log(y) + log_gamma_ratio(a)) * np.sqrt(s2) / np.sqrt(LD(np.pi) + LD("1.2246467991473532e-16"))
+    tail = np.where(low, pre * cf / v, LD(0.5) - pre * cf)
+    return np.where(z > 0, 1 - tail, tail)
+
+
+def integrate_ld(piece, zs, nu, x, w):
+    anc, L, d0 = (np.asarray(a, LD) for a in piece)
+    off = L[:, None] * x[None, :]
+    z = zs[:, None] * np.sin(d0[:, None] + off)
+    v = np.broadcast_to((nu + 1)[:, None], z.shape)
+    f = np.exp((nu - 1)[:, None] * np.log(np.abs(np.sin(anc[:, None] + off)))) * t1_ld(z, v.copy())
+    return (f * w[None, :]).sum(1) * np.abs(L)
+
+
+def check_fp64(records):
+    x, w = legendre_ld(220)
+    graded, plain = (x ** 3, w * 3 * x * x), legendre_ld(32)
+    rows = []
+    for s in range(1, 9):
+        nu, rho, h, k = (sample_main if s % 2 else sample_other)(np.random.default_rng(s), records // 8)
+        ok = nu >= 10.0
+        nu, rho, h, k = nu[ok], rho[ok], h[ok], k[ok]
+        p0, p1, split, zs, C = pieces(h, k, rho, nu)
+        n_, z_ = nu.astype(LD), zs.astype(LD)
+        ref = [integrate_ld(p, z_, n_, *graded) for p in (p0, p1)]
+        tot = ref[0] + np.where(split, ref[1], 0)
+        for i, p in enumerate((p0, p1)):
+            keep = np.asarray((tot * C > 1e-60) & (split if i else True))
+            err = np.abs(integrate_ld(p, z_, n_, *plain) - ref[i]) / tot
+            rows.append(np.column_stack([np.abs(p[1]) * np.sqrt(nu - 1.0 + 0.5 * zs * zs), err.astype(float)])[keep])
+    t = np.concatenate(rows)
+    kept = t[:, 0] <= np.sqrt(90.0)
+    print(f"FP64 rule: {len(t)} pieces, {kept.mean():.2f} of them with 32 nodes, worst error {t[kept, 1].max():.1e} of T_2")
+    for lo, hi in ((0.0, 8.0), (8.0, 9.487), (9.487, 10.0), (10.0, 11.0), (11.0, 13.0)):
+        b = (t[:, 0] > lo) & (t[:, 0] <= hi)
+        print(f"  score {lo:g} to {hi:g}: {b.sum()} pieces, worst {t[b, 1].max():.1e}")
+
+
 def main():
+    if len(sys.argv) > 1 and sys.argv[1] == "fp64":
+        return check_fp64(int(sys.argv[2]) if len(sys.argv) > 2 else 8000)
     records = int(sys.argv[1]) if len(sys.argv) > 1 else 40000
     train = np.concatenate([piece_table(*sample_main(np.random.default_rng(s), records // 8)) for s in range(1, 9)])
     bounds = fit(train)
